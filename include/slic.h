@@ -129,8 +129,9 @@ slic_status slic_segment(slic_handle h, const uint8_t *d_image, int32_t *d_label
 slic_status slic_connectivity_components(slic_handle h, const int32_t *d_in, int32_t *d_out, void *stream);
 
 /* Wait for the device, then report whether a bounded device loop of the
-   handle's component connectivity gave up since the last call
-   (SLIC_ERR_TIMEOUT; the labels are then incomplete). Clears the flag. */
+   handle's component connectivity, or a grid barrier of its one-launch
+   segmentation, gave up since the last call (SLIC_ERR_TIMEOUT; the labels
+   are then incomplete). Clears the flag. */
 slic_status slic_status_check(slic_handle h);
 
 /* Wait for the device, then report how many centre updates the last
@@ -174,7 +175,11 @@ slic_status slic_update(slic_handle h, const float *d_features, const int32_t *d
    writes d_out; they must not overlap. */
 slic_status slic_connectivity_pass(slic_handle h, const int32_t *d_in, int32_t *d_out, void *stream);
 
-/* Kernel launches enqueued by this handle since creation (all calls). */
+/* Kernel launches enqueued by this handle since creation (all calls). A
+   launch that runs several stages counts once per stage, as if each had a
+   launch of its own: slic_segment runs a frame whose features fit in the
+   GPU's shared memory (up to about 2.5 Mpx, S >= 7) as one cooperative
+   launch, unless the learned warm start is armed or profiling is enabled. */
 slic_status slic_launch_count(slic_handle h, long long *count);
 
 /* Per-kernel device-time accounting, for measurement. Enabling (from the
@@ -182,6 +187,7 @@ slic_status slic_launch_count(slic_handle h, long long *count);
    records a CUDA event pair around every assignment-kernel launch it
    enqueues, on the launching stream (inside a stream capture these become
    event-record nodes that every replay of the graph re-records).
+   (while enabled, slic_segment launches every stage by itself).
    slic_profile_read waits for those events and returns the summed duration
    (ms) of the recorded pairs and their number; it does not reset them. */
 slic_status slic_profile_enable(slic_handle h, int enable);
@@ -376,8 +382,8 @@ slic_status slic_segment_noalloc(const slic_params *params, const uint8_t *d_ima
                                  float *d_centres, void *stream);
 
 /* Wait for the current device, then report whether a bounded loop of the
-   allocation-free path's component connectivity (enforce_connectivity = 2)
-   gave up since the last check on this device (SLIC_ERR_TIMEOUT: those
+   allocation-free path (component connectivity, enforce_connectivity = 2, or
+   a grid barrier of the one-launch segmentation) gave up since the last check on this device (SLIC_ERR_TIMEOUT: those
    labels are incomplete). Clears the flag. */
 slic_status slic_noalloc_status_check(void);
 

@@ -29,7 +29,8 @@ struct slic_ctx {
     int32_t *lbl_tmp = nullptr;   // [H][W] connectivity ping-pong
     ConvState *cstate = nullptr;  // stopping-test state of the current run
     int *ccl = nullptr;           // component connectivity scratch (mode 2), and its error flag
-    int *ccl_err = nullptr;
+    int *ccl_err = nullptr;       // [0] the flag, [1..2] the barrier counters of the one-launch path
+    ResidentPlan plan{};          // the one-launch path (grid 0: not for this geometry)
     float fix_scale = 0.0f;
     size_t smem_max = 0;
     ConvConsts conv{};
@@ -113,6 +114,7 @@ cudaError_t ensure_lut(int dev) {
     float lut[256];
     make_lut(lut);
     cudaError_t e = upload_lut(lut);
+    if (e == cudaSuccess) e = upload_lut_frame(lut);
     if (e == cudaSuccess) g_lut_devices.push_back(dev);
     return e;
 }
@@ -173,6 +175,46 @@ FrameArgs frame_args(slic_ctx *h, const uint8_t *rgb, float *feat, int P, const 
     a.fix_scale = h->fix_scale;
     a.perturb = h->p.perturb_seeds;
     return a;
+}
+
+// The same frame for the one-launch path.
+ResidentFrame resident_args(const FrameArgs &a, int iterations, bool connect, int32_t *lbl_tmp, long long *acc,
+                            int *ctrl, int *err) {
+    ResidentFrame r{};
+    r.conv = a.conv;
+    r.rgb = a.rgb;
+    r.centres = a.centres_out;
+    r.labels = a.labels;
+    r.lbl_tmp = lbl_tmp;
+    r.acc = acc;
+    r.cstate = a.cstate;
+    r.ctrl = ctrl;
+    r.err = err;
+    r.W = a.W;
+    r.H = a.H;
+    r.C = a.C;
+    r.S = a.S;
+    r.ns_c = a.ns_c;
+    r.ns_r = a.ns_r;
+    r.K = a.ns_c * a.ns_r;
+    r.iterations = iterations;
+    r.perturb = a.perturb;
+    r.connect = connect ? 1 : 0;
+    r.labels_vec = a.labels_vec;
+    r.labels_vec2 = connect || ((uintptr_t)a.labels & 7) == 0 ? 1 : 0;
+    r.w = a.w;
+    r.fix_scale = a.fix_scale;
+    r.eps = a.conv_eps;
+    return r;
+}
+
+// Component connectivity of a handle's labels, in place.
+slic_status components(slic_ctx *h, int32_t *d_labels, cudaStream_t s) {
+    const cudaError_t e = launch_connectivity_components(d_labels, d_labels, h->p.width, h->p.height, h->S * h->S / 4,
+                                                         h->ccl, h->ccl_err, s);
+    if (e != cudaSuccess) return cuda_fail(h, e, "component connectivity launch");
+    h->launches += 9;
+    return SLIC_OK;
 }
 
 }  // namespace
@@ -265,8 +307,8 @@ slic_status slic_create(const slic_params *params, slic_handle *out) {
         dev_alloc(&h->acc, sizeof(long long) * 6 * (size_t)h->K) != cudaSuccess ||
         dev_alloc(&h->lbl_tmp, sizeof(int32_t) * npix) != cudaSuccess ||
         dev_alloc(&h->cstate, sizeof(ConvState)) != cudaSuccess ||
-        cudaMemset(h->cstate, 0, sizeof(ConvState)) != cudaSuccess || dev_alloc(&h->ccl_err, sizeof(int)) != cudaSuccess ||
-        cudaMemset(h->ccl_err, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(h->cstate, 0, sizeof(ConvState)) != cudaSuccess || dev_alloc(&h->ccl_err, 3 * sizeof(int)) != cudaSuccess ||
+        cudaMemset(h->ccl_err, 0, 3 * sizeof(int)) != cudaSuccess ||
         (p.enforce_connectivity == 2 && dev_alloc(&h->ccl, sizeof(int) * ccl_scratch_ints((long long)npix)) != cudaSuccess)) {
         cudaGetLastError();
         cudaFree(h->feat);
@@ -278,6 +320,11 @@ slic_status slic_create(const slic_params *params, slic_handle *out) {
         delete h;
         return fail(nullptr, SLIC_ERR_NOMEM, "device allocation of scratch failed");
     }
+    // One launch per frame where the features fit in shared memory; its three
+    // sets of sums take the place of the features in the scratch.
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess)
+        plan_resident(p.width, p.height, S, h->ns_c, h->ns_r, sms, sizeof(float) * 3 * (size_t)p.height * h->P, &h->plan);
     h->smem_max = assign_smem_bytes(assign_max_window(S, h->ns_c, h->ns_r), true);
     e = ensure_smem(h->device, h->smem_max);
     if (e != cudaSuccess) {
@@ -339,6 +386,22 @@ slic_status slic_segment(slic_handle h, const uint8_t *d_image, int32_t *d_label
     a.conv_eps = h->p.convergence;
     cudaError_t e;
     const bool warm = h->net != nullptr;
+    if (h->plan.grid > 0 && !warm && !h->profiling) {
+        ResidentFrame r = resident_args(a, n, h->p.enforce_connectivity == 1, h->lbl_tmp,
+                                        reinterpret_cast<long long *>(h->feat), h->ccl_err + 1, h->ccl_err);
+        r.init = h->init_centres;
+        e = launch_resident(r, h->plan, s);
+        if (e == cudaSuccess) {
+            h->init_centres = nullptr;
+            h->launches += 2 * n + 2 + (h->p.enforce_connectivity == 1 ? 2 : 0);  // the stages it runs
+            if (h->p.enforce_connectivity == 2) return components(h, d_labels, s);
+            return SLIC_OK;
+        }
+        // (a context limited to part of the GPU cannot hold every CTA at once:
+        // one launch per stage then)
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_fail(h, e, "one-launch segmentation");
+        cudaGetLastError();
+    }
     if (warm) {
         // Learned warm start: features first, the grid (or armed) initial
         // centres, then the member means of the network's labels (written to
@@ -396,10 +459,7 @@ slic_status slic_segment(slic_handle h, const uint8_t *d_image, int32_t *d_label
         if (e != cudaSuccess) return cuda_fail(h, e, "connectivity kernel launch");
         h->launches += 2;
     } else if (h->p.enforce_connectivity == 2) {
-        e = launch_connectivity_components(d_labels, d_labels, h->p.width, h->p.height, h->S * h->S / 4, h->ccl,
-                                           h->ccl_err, s);
-        if (e != cudaSuccess) return cuda_fail(h, e, "component connectivity launch");
-        h->launches += 9;
+        return components(h, d_labels, s);
     }
     return SLIC_OK;
 }
@@ -670,15 +730,30 @@ extern "C" slic_status slic_segment_noalloc(const slic_params *params, const uin
     cudaStream_t s = (cudaStream_t)stream;
     const size_t smem = assign_smem_bytes(win, true);
 
-    // Same stage order as slic_segment; the initialisation kernel zeroes the
-    // sums left in the shared array by the previous call.
-    e = launch_init_from_rgb(a, s);
-    for (int pass = 0; e == cudaSuccess && pass <= p.iterations; ++pass) {
+    // Same stage order as slic_segment, in one launch where the frame fits;
+    // the kernels zero the sums left in the shared array by the previous call.
+    ResidentPlan plan{};
+    int sms = 0;
+    bool done = false;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        plan_resident(p.width, p.height, S, ns_c, ns_r, sms, feat_b, &plan)) {
+        int *const words = reinterpret_cast<int *>(ctrl);
+        e = launch_resident(resident_args(a, p.iterations, p.enforce_connectivity == 1, lbl_tmp,
+                                          reinterpret_cast<long long *>(base), words + 1, words),
+                            plan, s);
+        done = e == cudaSuccess;
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            cudaGetLastError();
+            e = cudaSuccess;
+        }
+    }
+    if (e == cudaSuccess && !done) e = launch_init_from_rgb(a, s);
+    for (int pass = 0; e == cudaSuccess && !done && pass <= p.iterations; ++pass) {
         if (pass > 0)
             e = launch_update(a.acc, d_centres, d_centres, (int)K, 1.0f / a.fix_scale, a.cstate, a.conv_eps, pass, s);
         if (e == cudaSuccess) e = launch_assign(a, pass == 0, pass == p.iterations, false, smem, s);
     }
-    if (e == cudaSuccess && p.enforce_connectivity == 1) {
+    if (e == cudaSuccess && p.enforce_connectivity == 1 && !done) {
         e = launch_connectivity(d_labels, lbl_tmp, p.width, p.height, s);
         if (e == cudaSuccess) e = launch_connectivity(lbl_tmp, d_labels, p.width, p.height, s);
     } else if (e == cudaSuccess && p.enforce_connectivity == 2) {

@@ -254,6 +254,33 @@ cudaError_t launch_connectivity_batch(const FrameArgs *d_frames, int n, int tota
 // (strips x segments) and its strips per row:
 int connectivity2_units(int W, int H, int *strips_x);
 cudaError_t launch_connectivity2_batch(const FrameArgs *d_frames, int n, int total_units, int grid, cudaStream_t s);
+// One frame in one cooperative launch (slic_frame.cu), for frames whose
+// features fit in shared memory. The plan depends on the geometry alone: how
+// a cell splits into units (rectangles of at most cw x uh pixels, ncx x ncy
+// per cell, ppr pixel pairs per row, np pairs per lane), the grid and its
+// shared memory. False: the launch-per-stage path serves the frame.
+struct ResidentPlan {
+    int grid, np, xs, units, max_units, win, cw, uh, ncx, ncy, ppr, conn_rows;
+    size_t smem;
+};
+bool plan_resident(int W, int H, int S, int ns_c, int ns_r, int sms, size_t sums_bytes, ResidentPlan *plan);
+struct ResidentFrame {
+    ConvConsts conv;
+    const uint8_t *rgb;
+    const float *init;      // [K][6] initial centres instead of the grid, or null
+    float *centres;         // [K][6] out
+    int32_t *labels, *lbl_tmp;
+    long long *acc;         // three sets of [K][6] sums
+    ConvState *cstate;
+    int *ctrl;              // two barrier counters, zero before the first launch
+    int *err;               // bit 4: a barrier gave up
+    int W, H, C, S, ns_c, ns_r, K, iterations, perturb, connect, labels_vec, labels_vec2;
+    float w, fix_scale, eps;
+    int units, max_units, win, cw, uh, ncx, ncy, ppr, conn_rows;  // (from the plan)
+};
+cudaError_t launch_resident(ResidentFrame a, const ResidentPlan &p, cudaStream_t s);
+// sRGB table and shared-memory limits of slic_frame.cu (once per device).
+cudaError_t upload_lut_frame(const float *lut256);
 // Component-based connectivity (connectivity mode 2): in -> out over a W x H
 // label map (out may equal in), segments of at most min_size pixels joined
 // to a neighbour. scratch holds ccl_scratch_ints(W*H) ints; a bounded walk
