@@ -329,5 +329,40 @@ __device__ __forceinline__ void conn_strip(const int32_t *in, int32_t *labels, i
     }
 }
 
+// The same for R rows, ry0 .. ry0 + R - 1 (labels of this launch), with every
+// input row loaded before the first is used: conn_strip waits one L2 latency
+// per row.
+template <int R>
+__device__ __forceinline__ void conn_block(const int32_t *in, int32_t *labels, int W, int H, int sx, int ry0,
+                                           bool labels_vec, int lane) {
+    const int x0 = sx - 4 + 4 * lane;
+    const bool vec = (W & 3) == 0, edge_lane = x0 < 0 || x0 + 3 >= W;
+    int4 a[R + 4], l[R + 2];
+#pragma unroll
+    for (int j = 0; j < R + 4; ++j) a[j] = conn_load_row<false>(in, W, H, ry0 - 2 + j, x0, vec);
+    const bool inner = sx >= 4 && sx + 124 <= W && ry0 >= 2 && ry0 + R + 2 <= H;  // no sentinel anywhere
+#pragma unroll
+    for (int j = 0; j < R + 2; ++j)
+        l[j] = inner ? conn_rule4<true>(a[j], a[j + 1], a[j + 2])
+                     : conn_mask_row(conn_rule4<false>(a[j], a[j + 1], a[j + 2]), W, H, ry0 - 1 + j, x0, edge_lane);
+    const bool writer = lane >= 1 && lane <= 30;
+    const bool out_vec = vec && labels_vec && x0 >= 0 && x0 + 3 < W;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int4 o = inner ? conn_rule4<true>(l[j], l[j + 1], l[j + 2]) : conn_rule4<false>(l[j], l[j + 1], l[j + 2]);
+        if (writer && ry0 + j < H) {
+            int32_t *out = labels + (size_t)(ry0 + j) * W;
+            if (out_vec) {
+                *reinterpret_cast<int4 *>(out + x0) = o;
+            } else {
+                const int32_t ov[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (x0 + q >= 0 && x0 + q < W) out[x0 + q] = ov[q];
+            }
+        }
+    }
+}
+
 }  // namespace
 }  // namespace slicgb

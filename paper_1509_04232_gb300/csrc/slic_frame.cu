@@ -18,8 +18,7 @@
 #include "slic_device.cuh"
 
 #include <algorithm>
-#include <mutex>
-#include <vector>
+#include <type_traits>
 
 namespace slicgb {
 
@@ -29,9 +28,22 @@ namespace {
 
 constexpr int kFrThreads = 512;
 constexpr int kFrWarps = kFrThreads / 32;
-constexpr int kFrBinWords = 36;             // 9 candidates x (3 colour words, packed x / y / count)
+// A warp's bins: word q (3 colours, packed x / y / count) of candidate t in
+// copy c at q * 40 + t * 4 + c. Lanes use copy lane % 4: neighbouring lanes
+// mostly pick the same candidate, and with one copy an atomic instruction
+// took 8 passes over shared memory (ncu), a quarter of the launch.
+constexpr int kFrBinWords = 160;
 constexpr unsigned kFrPolls = 1u << 22;     // of the grid barrier: over a second
 constexpr int kFrMaxSmem = 227 * 1024;
+
+// A unit's first pixel and extent (wl x hl pixels, clipped to its cell and the
+// image), its cell k and the window records of its nine candidates (their
+// index times 3, a record being 3 x 16 bytes).
+struct __align__(16) FrUnit {
+    int k, x0, y0;
+    short wl, hl;
+    unsigned short rec[9], pad[7];
+};
 
 __device__ __forceinline__ int ld_acquire(const int *p) {
     int v;
@@ -58,7 +70,8 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
     float4 *const f_la = reinterpret_cast<float4 *>(fr_smem);  // [unit][NP][32] (l0, l1, a0, a1) of a pair
     float2 *const f_b = reinterpret_cast<float2 *>(f_la + (size_t)a.max_units * NP * 32);
     float *const ctab = reinterpret_cast<float *>(f_b + (size_t)a.max_units * NP * 32);
-    unsigned *const bins = reinterpret_cast<unsigned *>(ctab + (size_t)(sent + 1) * kCtabRec) + warp * kFrBinWords;
+    FrUnit *const units = reinterpret_cast<FrUnit *>(ctab + (size_t)(sent + 1) * kCtabRec);
+    unsigned *const bins = reinterpret_cast<unsigned *>(units + a.max_units) + warp * kFrBinWords;
     float *const lut = reinterpret_cast<float *>(bins - warp * kFrBinWords + kFrWarps * kFrBinWords);
 
     // Grid barrier in two halves: every CTA arrives once per barrier; the
@@ -66,7 +79,7 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
     int barriers = 0;
     auto arrive = [&]() {
         __syncthreads();
-        if (tid == 0) {
+        if (tid == kFrThreads - 32) {  // (the other warps go on meanwhile)
             __threadfence();
             atomicAdd(&a.ctrl[0], 1);
         }
@@ -101,6 +114,24 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
 
     for (int i = tid; i < 256; i += kFrThreads) lut[i] = g_lut_frame[i];
     for (int i = lane; i < kFrBinWords; i += 32) bins[i] = 0u;
+    // The units.
+    for (int ul = tid; ul < nu; ul += kFrThreads) {
+        const int u = u0 + ul, k = u / upc, sub = u - k * upc, sy = sub / a.ncx, sx = sub - sy * a.ncx;
+        const int cy = k / ns_c, cx = k - cy * ns_c;
+        FrUnit n;
+        n.k = k;
+        n.x0 = cx * S + sx * a.cw;
+        n.y0 = cy * S + sy * a.uh;
+        n.wl = (short)max(0, min(min(a.cw, (cx + 1) * S - n.x0), W - n.x0));
+        n.hl = (short)max(0, min(min(a.uh, (cy + 1) * S - n.y0), H - n.y0));
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const int dy = t / 3 - 1, dx = t % 3 - 1;
+            const bool in = cy + dy >= 0 && cy + dy < a.ns_r && cx + dx >= 0 && cx + dx < ns_c;
+            n.rec[t] = (unsigned short)(3 * (in ? (dy + 1) * win + k - k0 + 1 + dx : sent));
+        }
+        units[ul] = n;
+    }
     __syncthreads();
     // Initial centres of the window.
     for (int e = tid; e <= sent; e += kFrThreads) {
@@ -150,36 +181,37 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
             pcol[i] = 2 * (p - prow[i] * a.ppr);
         }
     }
-    // Unit u's cell, origin and extent (clipped to the cell and the image).
-    struct Unit {
-        int k, cx, cy, x0, y0, wl, hl;
-    };
-    auto unit_of = [&](int u) {
-        Unit n;
-        n.k = u / upc;
-        const int sub = u - n.k * upc, sy = sub / a.ncx, sx = sub - sy * a.ncx;
-        n.cy = n.k / ns_c;
-        n.cx = n.k - n.cy * ns_c;
-        n.x0 = n.cx * S + sx * a.cw;
-        n.y0 = n.cy * S + sy * a.uh;
-        n.wl = min(min(a.cw, (n.cx + 1) * S - n.x0), W - n.x0);
-        n.hl = min(min(a.uh, (n.cy + 1) * S - n.y0), H - n.y0);
-        return n;
-    };
-
-    // Features of the CTA's units, once (pixels outside a unit are zero).
+    // Features of the CTA's units, once (pixels outside a unit: black).
     for (int ul = warp; ul < nu; ul += kFrWarps) {
-        const Unit n = unit_of(u0 + ul);
+        const FrUnit &n = units[ul];
+        unsigned px[NP][2];  // (r, g, b) bytes of the pairs; all loads first
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-            float f[2][3] = {};
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                if (prow[i] < n.hl && pcol[i] + j < n.wl) {
-                    const uint8_t *q = a.rgb + ((size_t)(n.y0 + prow[i]) * W + n.x0 + pcol[i] + j) * a.C;
-                    convert_pixel(a.conv, __ldg(q), __ldg(q + 1), __ldg(q + 2), lut, f[j][0], f[j][1], f[j][2]);
-                }
+            const bool in0 = prow[i] < n.hl && pcol[i] < n.wl, in1 = in0 && pcol[i] + 1 < n.wl;
+            const uint8_t *q = a.rgb + ((size_t)(n.y0 + prow[i]) * W + n.x0 + pcol[i]) * a.C;
+            px[i][0] = px[i][1] = 0u;
+            if (a.C == 4 && ((uintptr_t)a.rgb & 3) == 0) {
+                if (in0) px[i][0] = __ldg(reinterpret_cast<const unsigned *>(q));
+                if (in1) px[i][1] = __ldg(reinterpret_cast<const unsigned *>(q) + 1);
+            } else if (a.C == 3 && in1 && ((uintptr_t)q & 1) == 0) {
+                const unsigned short *h = reinterpret_cast<const unsigned short *>(q);
+                const unsigned h0 = __ldg(h), h1 = __ldg(h + 1), h2 = __ldg(h + 2);
+                px[i][0] = h0 | (h1 << 16);
+                px[i][1] = (h1 >> 8) | (h2 << 8);
+            } else {
+                if (in0) px[i][0] = __ldg(q) | ((unsigned)__ldg(q + 1) << 8) | ((unsigned)__ldg(q + 2) << 16);
+                if (in1)
+                    px[i][1] = __ldg(q + a.C) | ((unsigned)__ldg(q + a.C + 1) << 8) |
+                               ((unsigned)__ldg(q + a.C + 2) << 16);
             }
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            float f[2][3];
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                convert_pixel(a.conv, px[i][j] & 255u, (px[i][j] >> 8) & 255u, (px[i][j] >> 16) & 255u, lut, f[j][0],
+                              f[j][1], f[j][2]);
             f_la[((size_t)ul * NP + i) * 32 + lane] = make_float4(f[0][0], f[1][0], f[0][1], f[1][1]);
             f_b[((size_t)ul * NP + i) * 32 + lane] = make_float2(f[0][2], f[1][2]);
         }
@@ -255,71 +287,78 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
         const bool last = pass == a.iterations;
         unsigned long long *const acc =
             reinterpret_cast<unsigned long long *>(a.acc) + (size_t)(pass % 3) * set_words;
-        for (int ul = warp; ul < nu; ul += kFrWarps) {
-            const Unit n = unit_of(u0 + ul);
-            if (n.wl <= 0 || n.hl <= 0) continue;  // (the warp's)
-            unsigned long long l[NP], aa[NP], b[NP], x[NP], fy[NP];
+        // M pairs per lane of unit ul, from pair i0 (all NP of them, or one half).
+        auto evaluate_unit = [&](auto pairs, int ul, int i0) {
+            constexpr int M = decltype(pairs)::value;
+            const FrUnit n = units[ul];
+            if (n.wl <= 0 || n.hl <= 0) return;  // (the warp's)
+            int row[M], col[M];
 #pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(f_la + ((size_t)ul * NP + i) * 32 + lane);
+            for (int i = 0; i < M; ++i) {
+                if (M == NP) {
+                    row[i] = prow[i];
+                    col[i] = pcol[i];
+                } else if (XS) {
+                    row[i] = (lane >> 3) + 4 * (i0 + i);
+                    col[i] = 2 * (lane & 7);
+                } else {
+                    const int p = lane + 32 * (i0 + i);
+                    row[i] = p / a.ppr;
+                    col[i] = 2 * (p - row[i] * a.ppr);
+                }
+            }
+            const float4 *const u_la = f_la + ((size_t)ul * NP + i0) * 32 + lane;
+            const float2 *const u_b = f_b + ((size_t)ul * NP + i0) * 32 + lane;
+            unsigned long long l[M], aa[M], b[M], x[M], fy[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(u_la + 32 * i);
                 l[i] = la.x;
                 aa[i] = la.y;
-                b[i] = *reinterpret_cast<const unsigned long long *>(f_b + ((size_t)ul * NP + i) * 32 + lane);
-                const float fx = (float)(n.x0 + pcol[i]), fyi = (float)(n.y0 + prow[i]);
+                b[i] = *reinterpret_cast<const unsigned long long *>(u_b + 32 * i);
+                const float fx = (float)(n.x0 + col[i]), fyi = (float)(n.y0 + row[i]);
                 x[i] = pack2(fx, fx + 1.0f);
                 fy[i] = pack2(fyi, fyi);
             }
-            // Window records of the nine candidates (the sentinel off the grid).
-            const float *rec9[9];
-            {
-                const int base = n.k - k0 + 1;
-#pragma unroll
-                for (int t = 0; t < 9; ++t) {
-                    const int dy = t / 3 - 1, dx = t % 3 - 1;
-                    const bool in = (dy >= 0 || n.cy > 0) && (dy <= 0 || n.cy + 1 < a.ns_r) &&
-                                    (dx >= 0 || n.cx > 0) && (dx <= 0 || n.cx + 1 < ns_c);
-                    rec9[t] = ctab + (size_t)(in ? (dy + 1) * win + base + dx : sent) * kCtabRec;
-                }
-            }
             // Eq. (1), candidates two at a time as in the pipelined kernel
-            float bk[NP][2];
+            float bk[M][2];
 #pragma unroll
-            for (int i = 0; i < NP; ++i) bk[i][0] = bk[i][1] = __int_as_float(0x7F800000);
+            for (int i = 0; i < M; ++i) bk[i][0] = bk[i][1] = __int_as_float(0x7F800000);
 #pragma unroll
             for (int t0 = 0; t0 < 9; t0 += 2) {
                 const int nt = t0 < 8 ? 2 : 1;
-                float kk[2][NP][2];
+                float kk[2][M][2];
 #pragma unroll
                 for (int q = 0; q < nt; ++q) {
-                    const float *rp = rec9[t0 + q];
+                    const float *rp = ctab + 4 * n.rec[t0 + q];
                     const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(rp);
                     const ulonglong2 bx = *reinterpret_cast<const ulonglong2 *>(rp + 4);
                     const unsigned long long yy = *reinterpret_cast<const unsigned long long *>(rp + 8);
 #pragma unroll
-                    for (int i = 0; i < NP; ++i) {
+                    for (int i = 0; i < M; ++i) {
                         const unsigned long long ddy = sub2(yy, fy[i]);
                         eval_keys(la, bx, mul2(ddy, ddy), ww, l[i], aa[i], b[i], XS ? x[0] : x[i], c_tags[t0 + q],
                                   kk[q][i][0], kk[q][i][1]);
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < NP; ++i)
+                for (int i = 0; i < M; ++i)
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
                         bk[i][j] = nt == 2 ? fmin3_nan(bk[i][j], kk[0][i][j], kk[1][i][j])
                                            : fmin_nan(bk[i][j], kk[0][i][j]);
             }
-            int t[NP][2];  // winning candidate, -1 outside the unit
+            int t[M][2];  // winning candidate, -1 outside the unit
 #pragma unroll
-            for (int i = 0; i < NP; ++i)
+            for (int i = 0; i < M; ++i)
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
-                    t[i][j] = prow[i] < n.hl && pcol[i] + j < n.wl ? (int)(__float_as_uint(bk[i][j]) & 15u) : -1;
+                    t[i][j] = row[i] < n.hl && col[i] + j < n.wl ? (int)(__float_as_uint(bk[i][j]) & 15u) : -1;
             if (last) {
                 int32_t *const dst = a.connect ? a.lbl_tmp : a.labels;
 #pragma unroll
-                for (int i = 0; i < NP; ++i) {
-                    const size_t p = (size_t)(n.y0 + prow[i]) * W + n.x0 + pcol[i];
+                for (int i = 0; i < M; ++i) {
+                    const size_t p = (size_t)(n.y0 + row[i]) * W + n.x0 + col[i];
                     int v[2];
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
@@ -343,7 +382,7 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
                 // 16 x 16 unit.
                 unsigned o[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                for (int i = 0; i < NP; ++i) {
+                for (int i = 0; i < M; ++i) {
                     unsigned v[2][4];
                     float f0, f1;
                     unpack2(l[i], f0, f1);
@@ -352,7 +391,7 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
                     fix_round2_biased(f0, f1, fs, v[0][1], v[1][1]);
                     unpack2(b[i], f0, f1);
                     fix_round2_biased(f0, f1, fs, v[0][2], v[1][2]);
-                    v[0][3] = (unsigned)pcol[i] + ((unsigned)prow[i] << 11) + (1u << 22);
+                    v[0][3] = (unsigned)col[i] + ((unsigned)row[i] << 11) + (1u << 22);
                     v[1][3] = v[0][3] + 1u;
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
@@ -361,30 +400,34 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
                             for (int q = 0; q < 4; ++q) o[q] += v[j][q];
                         } else if (t[i][j] >= 0) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) atomicAdd(&bins[t[i][j] * 4 + q], v[j][q]);
+                            for (int q = 0; q < 4; ++q) atomicAdd(&bins[q * 40 + t[i][j] * 4 + (lane & 3)], v[j][q]);
                         }
                     }
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) o[q] = __reduce_add_sync(kFull, o[q]);
                 __syncwarp();
-                // Lane 3 * t + part adds two of candidate t's six sums.
+                // Lane 3 * t + part adds two of candidate t's six sums (one sum
+                // per lane, whole records per instruction, was 8 % slower).
                 if (lane < 27) {
                     const int q = lane / 3, part = lane - 3 * q;
-                    uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
-                    if (q != 4) v = *reinterpret_cast<const uint4 *>(bins + q * 4);
-                    const unsigned cnt = v.w >> 22;
+                    auto word = [&](int w) {  // the four copies' sum (own: the warp's)
+                        if (q == 4) return w == 0 ? o[0] : w == 1 ? o[1] : w == 2 ? o[2] : o[3];
+                        const uint4 p = *reinterpret_cast<const uint4 *>(bins + w * 40 + q * 4);
+                        return p.x + p.y + p.z + p.w;
+                    };
+                    const unsigned xyn = word(3), cnt = xyn >> 22;
                     if (cnt != 0) {
-                        const unsigned bias = cnt * kFixBias, xs = v.w & 0x7FFu, ys = (v.w >> 11) & 0x7FFu;
+                        const unsigned bias = cnt * kFixBias;
                         long long v0, v1;
                         if (part == 0) {
-                            v0 = (int)(v.x - bias);
-                            v1 = (int)(v.y - bias);
+                            v0 = (int)(word(0) - bias);
+                            v1 = (int)(word(1) - bias);
                         } else if (part == 1) {
-                            v0 = (int)(v.z - bias);
-                            v1 = (long long)xs + (long long)cnt * n.x0;
+                            v0 = (int)(word(2) - bias);
+                            v1 = (long long)(xyn & 0x7FFu) + (long long)cnt * n.x0;
                         } else {
-                            v0 = (long long)ys + (long long)cnt * n.y0;
+                            v0 = (long long)((xyn >> 11) & 0x7FFu) + (long long)cnt * n.y0;
                             v1 = (long long)cnt;
                         }
                         unsigned long long *g = acc + (size_t)(n.k + (q / 3 - 1) * ns_c + q % 3 - 1) * 6 + 2 * part;
@@ -393,9 +436,26 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
                     }
                 }
                 __syncwarp();
-                if (lane < 9) *reinterpret_cast<uint4 *>(bins + lane * 4) = make_uint4(0u, 0u, 0u, 0u);
+                reinterpret_cast<uint4 *>(bins)[lane] = make_uint4(0u, 0u, 0u, 0u);
+                if (lane < 8) reinterpret_cast<uint4 *>(bins)[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
                 __syncwarp();
             }
+        };
+        // Each warp takes an equal run of the units; where NP is even, of
+        // half units: with 54 units (1920x1080, S = 16) on 16 warps whole
+        // ones would leave ten warps idle for the fourth round.
+        if (NP % 2 == 0) {
+            constexpr int kHalf = NP % 2 == 0 ? NP / 2 : 1;
+            int h = 2 * nu * warp / kFrWarps;
+            const int h1 = 2 * nu * (warp + 1) / kFrWarps;
+            if ((h & 1) && h < h1) {
+                evaluate_unit(std::integral_constant<int, kHalf>(), h >> 1, kHalf);
+                ++h;
+            }
+            for (; h + 1 < h1; h += 2) evaluate_unit(std::integral_constant<int, NP>(), h >> 1, 0);
+            if (h < h1) evaluate_unit(std::integral_constant<int, kHalf>(), h >> 1, 0);
+        } else {
+            for (int ul = warp; ul < nu; ul += kFrWarps) evaluate_unit(std::integral_constant<int, NP>(), ul, 0);
         }
         if (!last) {
             arrive();
@@ -412,10 +472,15 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
             arrive();
             ok = wait();
             const int strips = (W + kConnOut - 1) / kConnOut, segs = (H + a.conn_rows - 1) / a.conn_rows;
-            for (int u = c * kFrWarps + warp; ok && u < strips * segs; u += G * kFrWarps) {
-                const int seg = u / strips, ry0 = seg * a.conn_rows;
-                conn_strip<false>(a.lbl_tmp, a.labels, W, H, (u - seg * strips) * kConnOut, ry0,
-                                  min(ry0 + a.conn_rows, H), a.labels_vec != 0, lane);
+            for (int u = warp * G + c; ok && u < strips * segs; u += G * kFrWarps) {
+                const int seg = u / strips, sx = (u - seg * strips) * kConnOut, ry0 = seg * a.conn_rows;
+                if (a.conn_rows == 1)
+                    conn_block<1>(a.lbl_tmp, a.labels, W, H, sx, ry0, a.labels_vec != 0, lane);
+                else if (a.conn_rows == 2)
+                    conn_block<2>(a.lbl_tmp, a.labels, W, H, sx, ry0, a.labels_vec != 0, lane);
+                else
+                    conn_strip<false>(a.lbl_tmp, a.labels, W, H, sx, ry0, min(ry0 + a.conn_rows, H), a.labels_vec != 0,
+                                      lane);
             }
         }
     }
@@ -488,20 +553,26 @@ bool plan_resident(int W, int H, int S, int ns_c, int ns_r, int sms, size_t sums
         p.grid = (int)std::min<long long>(sms, units);
         p.max_units = (int)((units + p.grid - 1) / p.grid);
         p.win = (upc == 1 ? p.max_units : (p.max_units - 1) / (int)upc + 2) + 2;
-        p.smem = (size_t)p.max_units * np * 32 * 24 + (size_t)(3 * p.win + 1) * kCtabRec * 4 +
+        p.smem = (size_t)p.max_units * (np * 32 * 24 + sizeof(FrUnit)) + (size_t)(3 * p.win + 1) * kCtabRec * 4 +
                  kFrWarps * kFrBinWords * 4 + 256 * 4;
-        if (p.smem > (size_t)kFrMaxSmem) continue;
+        if (p.smem > (size_t)kFrMaxSmem || 3 * (3 * p.win) > 65535) continue;
         // Rounds of units per warp, each with its own fixed part (window
         // records, warp reductions, flush): about 0.6 of a pair's work.
-        const double cost = ((p.max_units + kFrWarps - 1) / kFrWarps) * (np + 0.6);
+        // Even np: half units (see k_frame), at half a pair's work more.
+        const int halves = (2 * p.max_units + kFrWarps - 1) / kFrWarps, rounds = (p.max_units + kFrWarps - 1) / kFrWarps;
+        const double cost = np % 2 ? rounds * (np + 0.6) : 0.5 * halves * np + 0.6 * (rounds + (halves & 1) * 0.5);
         if (plan->grid == 0 || cost < best) {
             best = cost;
             *plan = p;
         }
     }
     if (plan->grid == 0) return false;
+    // Connectivity: one or two rows per warp while the chip has a warp for
+    // each (a warp's latency is what counts: 320x240 takes 1.5 us this way,
+    // 6.5 us with segments of 4 rows), else segments streamed row by row.
     const long long strips = (W + kConnOut - 1) / kConnOut, warps = (long long)plan->grid * kFrWarps;
-    plan->conn_rows = (int)std::max<long long>(4, std::min<long long>(kConnSeg, (strips * H + warps - 1) / warps));
+    const long long rows = (strips * H + warps - 1) / warps;
+    plan->conn_rows = rows <= 2 ? (int)rows : (int)std::max<long long>(4, std::min<long long>(kConnSeg, rows));
     return true;
 }
 
