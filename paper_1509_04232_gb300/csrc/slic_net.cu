@@ -46,6 +46,11 @@ constexpr int kCinReal[kLayers] = {14, 32, 32, 32};
 constexpr int kCoutReal[kLayers] = {32, 32, 32, 9};
 constexpr int kCinPad[kLayers] = {16, 32, 32, 32};
 constexpr int kCoutPad[kLayers] = {32, 32, 32, 16};
+__host__ __device__ constexpr size_t wcount(int l) {
+    return (size_t)9 * (l == 0 ? 16 : 32) * (l == 3 ? 16 : 32);  // padded weights of layer l
+}
+constexpr size_t kWeights = 9 * (16 * 32 + 2 * 32 * 32 + 32 * 16);  // of all layers
+constexpr size_t kBiases = 32 + 32 + 32 + 16;
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -212,6 +217,50 @@ __device__ __forceinline__ bool tc_wait(unsigned long long *bar, unsigned parity
     return false;
 }
 
+// Walks indices first, first + step, ... as (a, b, c), a fastest, a < na and
+// b < nb, without a division per step (three run-time divisions per tile were
+// a third of the convolution's epilogue instructions).
+struct Stepper {
+    unsigned a, b, c, da, db, dc, na, nb;
+    __device__ __forceinline__ Stepper(unsigned first, unsigned step, unsigned na_, unsigned nb_) : na(na_), nb(nb_) {
+        const unsigned q = first / na, w = step / na;
+        a = first - q * na;
+        b = q % nb;
+        c = q / nb;
+        da = step - w * na;
+        db = w % nb;
+        dc = w / nb;
+    }
+    __device__ __forceinline__ void advance() {
+        a += da;
+        b += db;
+        c += dc;
+        if (a >= na) {
+            a -= na;
+            ++b;
+        }
+        if (b >= nb) {
+            b -= nb;
+            ++c;
+        }
+    }
+};
+
+// Two FP32 sums in one instruction (each rounded as the scalar addition).
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long pack2f(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2f(unsigned long long v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
 // NCOL (16 or 32) consecutive FP32 columns of this warp's 32 TMEM lanes,
 // without the wait (tcgen05.wait::ld follows a batch of these).
 template <int NCOL>
@@ -288,7 +337,7 @@ __device__ __forceinline__ void tc_arrive(unsigned long long *bar) {
 template <int CIN, int COUT, bool RELU, bool OUTF32, bool LABELS, int NS, bool BWD = false>
 __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
     const __grid_constant__ CUtensorMap in_map, const __nv_bfloat16 *wf, const float *bias, void *out, int W, int H,
-    int n_img, int S, int *err, const __nv_bfloat16 *mask) {
+    int n_img, int S, int *err, const __nv_bfloat16 *mask, float *db) {
     constexpr int NP = CIN / 8;                   // 8-channel planes
     constexpr int KC = CIN / 16;                  // K chunks per kernel row
     constexpr int ROWB = CIN * 2;                 // bytes of one staged position
@@ -366,13 +415,14 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
             unsigned u = 0;       // completed rounds of the ring
             unsigned issued = 0;  // bit s: a copy was issued into stage s
             unsigned lastpar = 0; // bit s: parity of that copy's completion
-            for (unsigned t = blockIdx.x; t < total; t += G) {
+            Stepper w(blockIdx.x, G, tiles_x, (unsigned)H);
+            for (unsigned t = blockIdx.x; t < total; t += G, w.advance()) {
                 if (u > 0 && !tc_wait_ab(&empty[s], (u - 1) & 1u, abort)) {
                     fail();
                     break;
                 }
-                const unsigned tx = t % tiles_x, ry = t / tiles_x;
-                const int y = (int)(ry % (unsigned)H), img = (int)(ry / (unsigned)H);
+                const unsigned tx = w.a;
+                const int y = (int)w.b, img = (int)w.c;
                 const unsigned b = tc_smem(&full[s]);
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(BOX) : "memory");
                 const unsigned dst0 = tc_smem(in_s + s * BOX);
@@ -447,11 +497,15 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32*(w%4) .. +31, channels 16*(w/4) .. +15 ----
         const int quarter = warp & 3, c0 = (warp >> 2) * 16;
-        float bv[16];
+        // channel pairs: the layer's biases, or (BWD) this lane's sums of the
+        // results it stores, the bias gradient of the previous layer
+        unsigned long long bv[8];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) bv[c] = !BWD && c0 + c < COUT ? bias[c0 + c] : 0.0f;
+        for (int c = 0; c < 8; ++c)
+            bv[c] = BWD ? 0ull : pack2f(bias[c0 + 2 * c], bias[c0 + 2 * c + 1]);
         unsigned j = 0;
-        for (unsigned t = blockIdx.x; t < total; t += G, ++j) {
+        Stepper w(blockIdx.x, G, tiles_x, (unsigned)H);
+        for (unsigned t = blockIdx.x; t < total; t += G, ++j, w.advance()) {
             const int bf = (int)(j & 1u);
             if (!__all_sync(0xffffffffu, tc_wait_ab(&tfull[bf], (j >> 1) & 1u, abort))) {
                 if (lane == 0) fail();
@@ -470,12 +524,16 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
             // output of lane l (l < 30): positions l, l+1, l+2 of this quarter
             float v[16];
 #pragma unroll
-            for (int c = 0; c < 16; ++c)
-                v[c] = (d0[c] + bv[c]) + __shfl_down_sync(0xffffffffu, d1[c], 1) +
-                       __shfl_down_sync(0xffffffffu, d2[c], 2);
+            for (int c = 0; c < 16; c += 2) {
+                unsigned long long p = pack2f(d0[c], d0[c + 1]);
+                if (!BWD) p = add2(p, bv[c / 2]);
+                p = add2(p, pack2f(__shfl_down_sync(0xffffffffu, d1[c], 1), __shfl_down_sync(0xffffffffu, d1[c + 1], 1)));
+                p = add2(p, pack2f(__shfl_down_sync(0xffffffffu, d2[c], 2), __shfl_down_sync(0xffffffffu, d2[c + 1], 2)));
+                unpack2f(p, v[c], v[c + 1]);
+            }
 
-            const unsigned tx = t % tiles_x, ry = t / tiles_x;
-            const int y = (int)(ry % (unsigned)H), img = (int)(ry / (unsigned)H);
+            const unsigned tx = w.a;
+            const int y = (int)w.b, img = (int)w.c;
             const int xw = (int)tx * kTcOut + kTcSeg * quarter;  // output pixel of lane 0
             const size_t row0 = (size_t)img * H * W + (size_t)y * W;
             if constexpr (BWD) {
@@ -506,6 +564,14 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                                                              : pack_bf16(v[8 * k + 2 * h], v[8 * k + 2 * h + 1]);
                     *reinterpret_cast<uint4 *>(ow + lane * 32 + ((k ^ ((lane >> 2) & 1)) << 4)) =
                         make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                    if constexpr (BWD) {
+                        if (lane < kTcSeg && xw + lane < W) {
+#pragma unroll
+                            for (int h = 0; h < 4; ++h)  // the rounded pair, as stored
+                                bv[4 * k + h] = add2(bv[4 * k + h], pack2f(__uint_as_float(w4[h] << 16),
+                                                                           __uint_as_float(w4[h] & 0xFFFF0000u)));
+                        }
+                    }
                 }
                 __syncwarp();
 #pragma unroll
@@ -550,6 +616,19 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                 }
             }
         }
+        if constexpr (BWD) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) bv[c] = add2(bv[c], __shfl_xor_sync(0xffffffffu, bv[c], o));
+                float lo, hi;
+                unpack2f(bv[c], lo, hi);
+                if (lane == c) {
+                    atomicAdd(&db[c0 + 2 * c], lo);
+                    atomicAdd(&db[c0 + 2 * c + 1], hi);
+                }
+            }
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -563,71 +642,82 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
 // ---------------------------------------------------------------------------
 // Weight gradient on the tensor cores: dW[dy*3+dx][ci][co] = sum over pixels
 // (y, x) of a_in[y+dy-1][x+dx-1][ci] dZ[y][x][co] (zero outside the image).
-// Kernel row dy has its own accumulator in tensor memory, D_dy[m][co] with
-// m = dx*CIN + ci (rows from 3*CIN to 127 stay zero), fed by tcgen05.mma of
-// M128 x N COUT x K16 over pixels: for output row y and the kWgK columns
-// x0 .. of a work strip, A_dy[m][k] = a_in[y+dy-1][x0+k+dx-1][ci] and
-// B[co][k] = dZ[y][x0+k][co], both K-major in the unswizzled canonical
-// layout (planes of 8 pixels, one 16-byte row per m or co: the forward
-// kernel's weight layout).
 //
-// A CTA walks strips of kWgK columns by kWgBand rows. Each input row is
-// staged once (16-byte loads of its NHWC row with a one-pixel halo) and
-// transposed into one of four row slots; output row y then reads the slots
-// of rows y-1, y, y+1 as A_0, A_1, A_2 and its dZ row from one of two B
-// slots, so a row costs one input-row and one dZ-row transposition. One
-// thread issues the 3 x kWgK/16 MMAs of a row; a slot is refilled once the
-// MMAs that read it have completed (tcgen05.commit on an mbarrier). Each CTA
-// writes its partial dW once; k_reduce_partials adds them.
+// The contraction runs over pixels, and both tensors are NHWC, so both
+// operands are MN-major as they lie in memory: no transposition. A stage
+// holds kWgK columns of four input rows (r-1 .. r+2) and two dZ rows (r, r+1)
+// in planes of 8 channels, a pixel's 16 bytes after its neighbour's: core
+// matrices of 8 pixels x 8 channels, 128 bytes apart along K (pixels) and one
+// plane apart along M or N. One tcgen05.mma of M 128 (4 input rows x 32
+// channels) x N 2 * COUT (2 dZ rows) x K 16 forms every pair of an input row i
+// and a dZ row j at one horizontal offset; the pairs with dy = i - j in 0..2
+// (six of eight) are the gradient's. The horizontal tap dx is the start
+// address of A, 16 bytes (one pixel) further per step, with an accumulator
+// per dx in tensor memory.
+//
+// Eight warps copy (cp.async, 16 bytes a lane, zeros outside the image) into
+// a ring of kWgStages stages, one thread issues the MMAs. The plane pitch of
+// kWgK + 2 pixels makes the eight 16-byte pieces of a quarter-warp land in
+// different banks. Per stage (128 pixels) 12 MMAs of about 48 cycles (6 KB of
+// operands each at 128 B/clk) bound the kernel: 32 us for 2.1 Mpx. Staging the
+// operands by transposing rows through shared memory (K-major operands, three
+// CTA barriers per output row) took 310 us per 32 -> 32 layer.
 // ---------------------------------------------------------------------------
-constexpr int kWgK = 64;     // pixels (columns) of a strip
-constexpr int kWgBand = 32;  // rows of a strip
-constexpr int kWgPlanes = kWgK / 8;
-constexpr int kWgThreads = 256;
-__host__ __device__ constexpr int wg_slot_bytes() { return kWgPlanes * 128 * 16; }
-__host__ __device__ constexpr int wg_b_bytes(int cout) { return kWgPlanes * cout * 16; }
-__host__ __device__ constexpr int wg_raw_a(int cin) { return (kWgK + 2) * cin * 2; }
-__host__ __device__ constexpr int wg_raw_z(int cout) { return kWgK * cout * 2; }
-__host__ __device__ constexpr int wg_smem_bytes(int cin, int cout) {
-    return 128 + 4 * wg_slot_bytes() + 2 * wg_b_bytes(cout) + wg_raw_a(cin) + wg_raw_z(cout) + 64;
+constexpr int kWgK = 64;      // pixels (columns) of a stage
+constexpr int kWgStages = 4;
+constexpr int kWgLoaders = 256;
+constexpr int kWgThreads = kWgLoaders + 32;
+constexpr int kWgPlane = (kWgK + 2) * 16;   // bytes of one 8-channel plane of one row
+__host__ __device__ constexpr int wg_a_bytes() { return 16 * kWgPlane; }  // 4 rows x 4 planes (2 of them zero for 16 channels)
+__host__ __device__ constexpr int wg_b_bytes(int cout) { return 2 * (cout / 8) * kWgPlane; }
+__host__ __device__ constexpr int wg_stage_bytes(int cout) { return wg_a_bytes() + wg_b_bytes(cout); }
+__host__ __device__ constexpr int wg_smem_bytes(int cout) {
+    return 128 + kWgStages * wg_stage_bytes(cout) + (2 * kWgStages + 1) * 8 + 16;
 }
 
-// Two bf16 (as raw 16-bit patterns) in one 32-bit word, lo in the low half.
-__device__ __forceinline__ uint32_t bf16_pair(const __nv_bfloat16 &lo, const __nv_bfloat16 &hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+// A 16-byte asynchronous copy, zeros when !ok (nothing is read then).
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16u : 0u) : "memory");
 }
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bfloat16 *a_in,
                                                                    const __nv_bfloat16 *dz, int W, int H, int n_img,
                                                                    float *partial, int *err) {
-    constexpr int M_REAL = 3 * CIN;
-    constexpr int A_PLANE = 128 * 16, B_PLANE = COUT * 16;
-    constexpr int SLOT = wg_slot_bytes(), BSLOT = wg_b_bytes(COUT);
-    constexpr int TCOLS = 128;  // tensor memory: the three accumulators of COUT columns
-    static_assert(M_REAL <= 128 && 3 * COUT <= TCOLS && (COUT == 16 || COUT == 32) && CIN % 8 == 0,
-                  "shapes of the weight-gradient kernel");
+    constexpr int STAGE = wg_stage_bytes(COUT), A_BYTES = wg_a_bytes();
+    constexpr int APL = CIN / 8, BPL = COUT / 8;   // real planes per row
+    constexpr int NN = 2 * COUT;
+    constexpr int TCOLS = 3 * NN <= 128 ? 128 : 256;
+    static_assert((CIN == 16 || CIN == 32) && (COUT == 16 || COUT == 32), "shapes of the weight-gradient kernel");
     extern __shared__ __align__(16) unsigned char wg_dyn[];
-    unsigned char *slots =
+    unsigned char *const ring =
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(wg_dyn) + 127) & ~(uintptr_t)127);
-    unsigned char *bslots = slots + 4 * SLOT;
-    __nv_bfloat16 *ra = reinterpret_cast<__nv_bfloat16 *>(bslots + 2 * BSLOT);  // [kWgK+2][CIN]
-    __nv_bfloat16 *rz = ra + wg_raw_a(CIN) / 2;                                 // [kWgK][COUT]
-    unsigned long long *mma_done = reinterpret_cast<unsigned long long *>(rz + wg_raw_z(COUT) / 2);  // [2]
-    unsigned long long *fin = mma_done + 2;
-    unsigned *tmem_slot = reinterpret_cast<unsigned *>(fin + 1);
+    static_assert(9 * CIN * (COUT + 1) * 4 <= kWgStages * STAGE, "the sums reuse the ring");
+    unsigned long long *const full = reinterpret_cast<unsigned long long *>(ring + kWgStages * STAGE);
+    unsigned long long *const empty = full + kWgStages;
+    unsigned long long *const fin = empty + kWgStages;
+    unsigned *const tmem_slot = reinterpret_cast<unsigned *>(fin + 1);
+    volatile int *const abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // the padding rows of A in every slot stay zero
-    for (int i = tid; i < 4 * kWgPlanes * (128 - M_REAL); i += kWgThreads) {
-        const int r = M_REAL + i % (128 - M_REAL), pl = i / (128 - M_REAL);  // pl = slot * planes + plane
-        *reinterpret_cast<uint4 *>(slots + pl * A_PLANE + r * 16) = make_uint4(0u, 0u, 0u, 0u);
+    if (CIN == 16) {  // planes 2 and 3 of every input row stay zero
+        for (int i = tid; i < kWgStages * 4 * 2 * (kWgPlane / 16); i += kWgThreads) {
+            const int q = i % (kWgPlane / 16), p = i / (kWgPlane / 16);  // p = (stage * 4 + row) * 2 + plane - 2
+            *reinterpret_cast<uint4 *>(ring + (p >> 3) * STAGE + (((p >> 1) & 3) * 4 + 2 + (p & 1)) * kWgPlane + q * 16) =
+                make_uint4(0u, 0u, 0u, 0u);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (tid == 0) {
-        for (int i = 0; i < 3; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(&mma_done[i])));
+        for (int i = 0; i < kWgStages; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc_smem(&full[i])), "n"(kWgLoaders / 32));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(&empty[i])));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(fin)));
+        *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {
+    if (warp == kWgLoaders / 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)),
                      "n"(TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -637,208 +727,230 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bf
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tmem_slot;
 
-    // the input row yy of image img at x0-1 .. x0+kWgK into ra (zeros outside)
-    auto stage_row = [&](size_t base, int yy, int x0) {
-        for (int i = tid; i < (kWgK + 2) * (CIN / 8); i += kWgThreads) {
-            const int v8 = i % (CIN / 8), px = i / (CIN / 8), gx = x0 - 1 + px;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gx >= 0 && gx < W && yy >= 0 && yy < H)
-                v = *reinterpret_cast<const uint4 *>(a_in + (base + (size_t)yy * W + gx) * CIN + v8 * 8);
-            *reinterpret_cast<uint4 *>(ra + (size_t)px * CIN + v8 * 8) = v;
-        }
+    // Stages of this CTA: units blockIdx.x + j * gridDim.x of (image, row
+    // pair, column strip).
+    const unsigned segs = (unsigned)(W + kWgK - 1) / kWgK, pairs = (unsigned)(H + 1) / 2;
+    const unsigned units = (unsigned)n_img * pairs * segs;  // (fewer than the batch's pixels, < 2^31)
+    const int n_stage = blockIdx.x < units ? (int)((units - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+    auto fail = [&]() {
+        *abort = 1;
+        atomicOr(err, 1);
     };
-    // ra transposed into a row slot: rows m = dx*CIN + ci, planes of 8 pixels
-    auto transpose_row = [&](int slot) {
-        unsigned char *A = slots + slot * SLOT;
-        for (int i = tid; i < kWgPlanes * M_REAL; i += kWgThreads) {
-            const int m = i % M_REAL, j = i / M_REAL, dx = m / CIN, ci = m - dx * CIN;
-            const __nv_bfloat16 *src = ra + (size_t)(8 * j + dx) * CIN + ci;
-            *reinterpret_cast<uint4 *>(A + j * A_PLANE + m * 16) =
-                make_uint4(bf16_pair(src[0], src[CIN]), bf16_pair(src[2 * CIN], src[3 * CIN]),
-                           bf16_pair(src[4 * CIN], src[5 * CIN]), bf16_pair(src[6 * CIN], src[7 * CIN]));
-        }
-    };
-    // the MMAs of output row `it` have completed (commits alternate on two barriers)
-    auto row_done = [&](int j) -> bool { return tc_wait(&mma_done[j & 1], (j >> 1) & 1); };
-
-    const int segs = (W + kWgK - 1) / kWgK, bands = (H + kWgBand - 1) / kWgBand;
-    const long long units = (long long)n_img * segs * bands;
-    int it = 0;  // output rows of this CTA so far
-    bool ok = true;
-    for (long long u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int seg = (int)(u % segs);
-        const long long q = u / segs;
-        const int band = (int)(q % bands), img = (int)(q / bands);
-        const int x0 = seg * kWgK, y0 = band * kWgBand, y1 = min(y0 + kWgBand, H);
-        const size_t base = (size_t)img * H * W;
-        // the previous strip's MMAs read every slot: let them complete
-        const bool w = (it < 1 || row_done(it - 1)) && (it < 2 || row_done(it - 2));
-        if (!__syncthreads_and(w ? 1 : 0)) {
-            ok = false;
-            break;
-        }
-        // input rows y0-1 and y0 into slots 0 and 1 (row yy in slot (yy - y0 + 1) % 4)
-        for (int p = 0; p < 2; ++p) {
-            stage_row(base, y0 - 1 + p, x0);
-            __syncthreads();
-            transpose_row(p);
-            __syncthreads();
-        }
-        for (int r = y0; r < y1; ++r, ++it) {
-            // raw rows: input row r+1 (its slot held row r-3, read by row it-2),
-            // dZ row r (B slot it % 2, read by row it-2)
-            stage_row(base, r + 1, x0);
-            for (int i = tid; i < kWgK * (COUT / 8); i += kWgThreads) {
-                const int v8 = i % (COUT / 8), px = i / (COUT / 8), gx = x0 + px;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (gx < W) v = *reinterpret_cast<const uint4 *>(dz + (base + (size_t)r * W + gx) * COUT + v8 * 8);
-                *reinterpret_cast<uint4 *>(rz + px * COUT + v8 * 8) = v;
-            }
-            const bool w2 = r - y0 < 2 || row_done(it - 2);
-            if (!__syncthreads_and(w2 ? 1 : 0)) {  // (also: the raw rows are complete)
-                ok = false;
-                break;
-            }
-            const int sn = (r - y0 + 2) & 3;
-            transpose_row(sn);
-            unsigned char *B = bslots + (it & 1) * BSLOT;
-            for (int i = tid; i < kWgPlanes * COUT; i += kWgThreads) {
-                const int co = i % COUT, j = i / COUT;
-                const __nv_bfloat16 *src = rz + (size_t)(8 * j) * COUT + co;
-                *reinterpret_cast<uint4 *>(B + j * B_PLANE + co * 16) =
-                    make_uint4(bf16_pair(src[0], src[COUT]), bf16_pair(src[2 * COUT], src[3 * COUT]),
-                               bf16_pair(src[4 * COUT], src[5 * COUT]), bf16_pair(src[6 * COUT], src[7 * COUT]));
-            }
-            // generic-proxy writes -> visible to the tensor core
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncthreads();
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const unsigned idesc = tc_idesc(128, COUT);
-                const unsigned b0 = tc_smem(B);
+    if (warp < kWgLoaders / 32) {
+        // ---- loaders ----
+        constexpr int kAhead = kWgStages - 1;
+        bool ok = true;
+        Stepper u(blockIdx.x, gridDim.x, segs, pairs);
+        for (int j = 0; j < n_stage + kAhead; ++j) {
+            if (j < n_stage) {
+                const int s = j % kWgStages;
+                if (j >= kWgStages && !__all_sync(0xffffffffu, tc_wait_ab(&empty[s], (j / kWgStages - 1) & 1, abort))) {
+                    if (lane == 0) fail();
+                    ok = false;
+                    break;
+                }
+                const int r = 2 * (int)u.b, x0 = (int)u.a * kWgK;
+                const size_t base = (size_t)u.c * H * W;
+                u.advance();
+                const unsigned st = tc_smem(ring + s * STAGE);
+                {
+                    // piece: plane fastest, then pixel, then row
+                    constexpr int PER = kWgLoaders / (kWgK * APL);  // rows per sweep
+                    const int pl = tid % APL, px = (tid / APL) % kWgK, row0 = tid / (APL * kWgK);
 #pragma unroll
-                for (int dy = 0; dy < 3; ++dy) {
-                    const unsigned a0 = tc_smem(slots + ((r - y0 + dy) & 3) * SLOT);  // input row r-1+dy
-#pragma unroll
-                    for (int kc = 0; kc < kWgK / 16; ++kc) {
-                        const unsigned long long ad = tc_desc(a0 + 2 * kc * A_PLANE, A_PLANE, 128);
-                        const unsigned long long bd = tc_desc(b0 + 2 * kc * B_PLANE, B_PLANE, 128);
-                        const unsigned acc = (it > 0 || kc > 0) ? 1u : 0u;
-                        asm volatile(
-                            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
-                                tmem + (unsigned)(dy * COUT)),
-                            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+                    for (int i = 0; i < 4 / PER; ++i) {
+                        const int row = row0 + i * PER, yy = r - 1 + row, gx = x0 - 1 + px;
+                        const bool in = gx >= 0 && gx < W && yy >= 0 && yy < H;
+                        cp_async16(st + (row * 4 + pl) * kWgPlane + px * 16,
+                                   a_in + (in ? (base + (size_t)yy * W + gx) * CIN + pl * 8 : 0), in);
+                    }
+                    if (tid < 4 * 2 * APL) {  // the last two columns
+                        const int hp = tid % APL, hx = kWgK + (tid / APL) % 2, row = tid / (2 * APL);
+                        const int yy = r - 1 + row, gx = x0 - 1 + hx;
+                        const bool in = gx < W && yy >= 0 && yy < H;
+                        cp_async16(st + (row * 4 + hp) * kWgPlane + hx * 16,
+                                   a_in + (in ? (base + (size_t)yy * W + gx) * CIN + hp * 8 : 0), in);
                     }
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 tc_smem(&mma_done[it & 1]))
-                             : "memory");
+                {
+                    constexpr int PER = kWgLoaders / (kWgK * BPL);
+                    const int pl = tid % BPL, px = (tid / BPL) % kWgK, row0 = tid / (BPL * kWgK);
+#pragma unroll
+                    for (int i = 0; i < 2 / PER; ++i) {
+                        const int row = row0 + i * PER, yy = r + row, gx = x0 + px;
+                        const bool in = gx < W && yy < H;
+                        cp_async16(st + A_BYTES + (row * BPL + pl) * kWgPlane + px * 16,
+                                   dz + (in ? (base + (size_t)yy * W + gx) * COUT + pl * 8 : 0), in);
+                    }
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            const int d = j - kAhead;  // stage whose copies are complete once kAhead groups are left in flight
+            if (d >= 0) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(kAhead) : "memory");
+                // generic-proxy writes -> visible to the tensor core
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc_arrive(&full[d % kWgStages]);
             }
         }
-    }
-    // every MMA complete, then each accumulator row out: warp w (< 4) reads
-    // lanes 32w .. 32w+31 (rows m), columns dy*COUT .. +COUT-1
-    if (tid == 0)
+        if (!ok) asm volatile("cp.async.wait_all;" ::: "memory");  // no copy may outlive the CTA
+    } else if (lane == 0) {
+        // ---- MMA issuer ----
+        const unsigned idesc = tc_idesc(128, NN) | (1u << 15) | (1u << 16);  // A and B are MN-major
+        for (int j = 0; j < n_stage; ++j) {
+            const int s = j % kWgStages;
+            if (!tc_wait_ab(&full[s], (j / kWgStages) & 1, abort)) {
+                fail();
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const unsigned a0 = tc_smem(ring + s * STAGE), b0 = a0 + A_BYTES;
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                for (int kc = 0; kc < kWgK / 16; ++kc) {
+                    const unsigned long long ad = tc_desc(a0 + (dx + 16 * kc) * 16, 128, kWgPlane);
+                    const unsigned long long bd = tc_desc(b0 + 256 * kc, 128, kWgPlane);
+                    const unsigned acc = (j > 0 || kc > 0) ? 1u : 0u;
+                    asm volatile(
+                        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
+                            tmem + (unsigned)(dx * NN)),
+                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+                }
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             tc_smem(&empty[s]))
+                         : "memory");
+        }
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem(fin))
                      : "memory");
-    const bool f_ok = tc_wait(fin, 0);
-    if (!__syncthreads_and(f_ok ? 1 : 0)) ok = false;
-    if (!ok && tid == 0) atomicOr(err, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp < 4) {
-        const int m = warp * 32 + lane;
-        const int dx = m / CIN, ci = m - dx * CIN;
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-            float v[COUT];
-            tc_ld_cols<COUT>(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(dy * COUT), v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (m < M_REAL) {
-                float4 *dst = reinterpret_cast<float4 *>(partial +
-                                                         (((size_t)blockIdx.x * 9 + dy * 3 + dx) * CIN + ci) * COUT);
-#pragma unroll
-                for (int q = 0; q < COUT / 4; ++q)
-                    dst[q] = it > 0 ? make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3])
-                                    : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-        }
+        if (!tc_wait(fin, 0)) fail();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp == 0) {
+    // Warp i (< 4) holds input row i (lanes = channels): the column block of
+    // dZ row j belongs to dy = i - j. First the blocks of j = 0, then those
+    // of j = 1 added, in shared memory (the ring is free now).
+    float *const sum = reinterpret_cast<float *>(ring);  // [tap][ci][COUT + 1], padded against bank conflicts
+#pragma unroll
+    for (int jrow = 0; jrow < 2; ++jrow) {
+        const int dy = warp - jrow;
+        if (warp < 4) {
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                float v[COUT];
+                tc_ld_cols<COUT>(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(dx * NN + jrow * COUT), v);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (dy >= 0 && dy <= 2 && lane < CIN) {
+                    float *dst = sum + ((dy * 3 + dx) * CIN + lane) * (COUT + 1);
+#pragma unroll
+                    for (int q = 0; q < COUT; ++q) {
+                        const float w = n_stage > 0 ? v[q] : 0.0f;
+                        dst[q] = jrow == 0 ? w : dst[q] + w;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < 9 * CIN * COUT; i += kWgThreads)
+        partial[(size_t)blockIdx.x * 9 * CIN * COUT + i] = sum[i / COUT * (COUT + 1) + i % COUT];
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == kWgLoaders / 32) {
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TCOLS));
     }
 }
 
-__global__ void k_reduce_partials(const float *partial, int n_blocks, int n, float *out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.0f;
-    for (int b = 0; b < n_blocks; ++b) s += partial[(size_t)b * n + i];
-    out[i] = s;
+// The CTAs' partial dW of every layer added up: a block sums 32 elements (of
+// one layer: the layers' sizes are multiples of 32), 8 slices of the CTAs side
+// by side. One launch per layer with one thread per element left the latency
+// of 304 dependent steps: 23 us each.
+__global__ void __launch_bounds__(256) k_reduce_partials(const float *partial, int n_blocks, float *out) {
+    __shared__ float s[8][32];
+    const int e = threadIdx.x & 31, slice = threadIdx.x >> 5, i = blockIdx.x * 32 + e;
+    int l = 0, first = 0;
+    while (l < kLayers - 1 && i >= first + (int)wcount(l)) first += (int)wcount(l++);
+    const size_t n = wcount(l);
+    const float *p = partial + (size_t)first * n_blocks + (i - first);
+    float v = 0.0f;
+    for (int b = slice; b < n_blocks; b += 8) v += p[(size_t)b * n];
+    s[slice][e] = v;
+    __syncthreads();
+    if (slice == 0) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) v += s[q][e];
+        out[i] = v;
+    }
 }
 
-// Bias gradient: db[co] = sum_p dZ[p][co] (per-CTA sums, then atomics).
-template <int COUT>
-__global__ void k_bias_grad(const __nv_bfloat16 *dz, long long n_px, float *db) {
-    __shared__ float s[COUT];
-    if (threadIdx.x < COUT) s[threadIdx.x] = 0.0f;
-    __syncthreads();
-    const int co = threadIdx.x % COUT;
-    float acc = 0.0f;
-    for (long long p = (long long)blockIdx.x * (blockDim.x / COUT) + threadIdx.x / COUT; p < n_px;
-         p += (long long)gridDim.x * (blockDim.x / COUT))
-        acc += __bfloat162float(dz[p * COUT + co]);
-    atomicAdd(&s[co], acc);
-    __syncthreads();
-    if (threadIdx.x < COUT) atomicAdd(&db[threadIdx.x], s[threadIdx.x]);
-}
-
-
-__global__ void k_softmax_ce(const float *logits, const uint8_t *target, int W, int H, int n_img, int S,
-                             float inv_total, __nv_bfloat16 *dz, float *stats) {
-    const long long n_px = (long long)W * H * n_img;
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    float loss = 0.0f, correct = 0.0f;
-    if (p < n_px) {
-        const int x = (int)(p % W), y = (int)((p / W) % H);
-        const int cx = x / S, cy = y / S, ns_c = (W + S - 1) / S, ns_r = (H + S - 1) / S;
-        const float *l = logits + p * 16;
-        float mx = -INFINITY;
+// The last layer's bias gradient (the sums of the stored dL/dlogits) on the
+// way. One pass over 97 B/px by a grid sized for the device, 16-byte loads,
+// and one atomic per sum and block: a thread per pixel with scalar loads and
+// two atomics per warp to the same words took 226 us for 2.1 Mpx.
+__global__ void __launch_bounds__(256) k_softmax_ce(const float *logits, const uint8_t *target, int W, int H, int n_img,
+                                                    int S, float inv_total, __nv_bfloat16 *dz, float *stats,
+                                                    float *db) {
+    const unsigned n_px = (unsigned)n_img * (unsigned)H * (unsigned)W;  // < 2^31
+    const int ns_c = (W + S - 1) / S, ns_r = (H + S - 1) / S;
+    float acc[11] = {};  // loss, correct, the 9 slots' gradients
+    Stepper w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, (unsigned)W, (unsigned)H);
+    for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < n_px; p += gridDim.x * blockDim.x, w.advance()) {
+        const int cx = (int)w.a / S, cy = (int)w.b / S;
+        const float4 *lp = reinterpret_cast<const float4 *>(logits + (size_t)p * 16);
+        const float4 l0 = __ldg(lp), l1 = __ldg(lp + 1);
+        const float l[9] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w, __ldg(logits + (size_t)p * 16 + 8)};
+        const int tg = target[p];
+        float mx = -INFINITY, lt = 0.0f;
         int arg = 0;
-        for (int t = 0; t < 9; ++t)
-            if (slot_valid(t, cx, cy, ns_c, ns_r) && l[t] > mx) {
+        bool ok[9];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            ok[t] = slot_valid(t, cx, cy, ns_c, ns_r);
+            if (ok[t] && l[t] > mx) {
                 mx = l[t];
                 arg = t;
             }
+            if (t == tg) lt = l[t];
+        }
         float e[9], sum = 0.0f;
+#pragma unroll
         for (int t = 0; t < 9; ++t) {
-            e[t] = slot_valid(t, cx, cy, ns_c, ns_r) ? __expf(l[t] - mx) : 0.0f;
+            e[t] = ok[t] ? __expf(l[t] - mx) : 0.0f;
             sum += e[t];
         }
-        const int tg = target[p];
-        loss = -(l[tg] - mx - __logf(sum));
-        correct = (arg == tg) ? 1.0f : 0.0f;
+        acc[0] += -(lt - mx - __logf(sum));
+        acc[1] += (arg == tg) ? 1.0f : 0.0f;
         uint32_t g[8];
+#pragma unroll
         for (int t = 0; t < 16; t += 2) {
-            const float g0 = t < 9 ? (e[t] / sum - (t == tg ? 1.0f : 0.0f)) * inv_total : 0.0f;
-            const float g1 = t + 1 < 9 ? (e[t + 1] / sum - (t + 1 == tg ? 1.0f : 0.0f)) * inv_total : 0.0f;
+            const float g0 = t < 9 ? (e[t < 9 ? t : 0] / sum - (t == tg ? 1.0f : 0.0f)) * inv_total : 0.0f;
+            const float g1 = t + 1 < 9 ? (e[t + 1 < 9 ? t + 1 : 0] / sum - (t + 1 == tg ? 1.0f : 0.0f)) * inv_total : 0.0f;
             g[t / 2] = pack_bf16(g0, g1);
+            if (t < 9) acc[2 + (t < 9 ? t : 0)] += __uint_as_float(g[t / 2] << 16);
+            if (t + 1 < 9) acc[2 + (t + 1 < 9 ? t + 1 : 0)] += __uint_as_float(g[t / 2] & 0xFFFF0000u);
         }
-        uint4 *d = reinterpret_cast<uint4 *>(dz + p * 16);
+        uint4 *d = reinterpret_cast<uint4 *>(dz + (size_t)p * 16);
         d[0] = make_uint4(g[0], g[1], g[2], g[3]);
         d[1] = make_uint4(g[4], g[5], g[6], g[7]);
     }
-    for (int off = 16; off > 0; off >>= 1) {
-        loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
-        correct += __shfl_xor_sync(0xFFFFFFFFu, correct, off);
+    __shared__ float part[8][11];
+#pragma unroll
+    for (int i = 0; i < 11; ++i) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xFFFFFFFFu, acc[i], o);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5][i] = acc[i];
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&stats[0], loss);
-        atomicAdd(&stats[1], correct);
+    __syncthreads();
+    if (threadIdx.x < 11) {
+        float v = 0.0f;
+        for (int q = 0; q < 8; ++q) v += part[q][threadIdx.x];
+        atomicAdd(threadIdx.x < 2 ? &stats[threadIdx.x] : &db[threadIdx.x - 2], v);
     }
 }
 
@@ -938,7 +1050,10 @@ struct slic_net_ctx {
     __nv_bfloat16 *act[kLayers] = {};
     float *logits = nullptr;
     __nv_bfloat16 *dzA = nullptr, *dzB = nullptr;
-    float *partial = nullptr;
+    // every gradient in one buffer (the layers' wg in order, then their bg),
+    // and after it the loss statistics, so that one clear serves them
+    float *grads = nullptr;
+    float *partial = nullptr;   // per layer [partial_blocks][9][Cin_p][Cout_p]
     int partial_blocks = 0;
     float *stats = nullptr;
     int *tc_err = nullptr;   // set by a timed-out wait of the tensor-core convolution
@@ -978,11 +1093,11 @@ bool nalloc(slic_net_ctx *n, T **p, size_t count) {
     return true;
 }
 
-size_t wcount(int l) { return (size_t)9 * kCinPad[l] * kCoutPad[l]; }
 
 template <int CIN, int COUT, bool RELU, bool OUTF32, bool LABELS, int NS, bool BWD = false>
 cudaError_t conv_fwd_tc(const CUtensorMap &in_map, const __nv_bfloat16 *wf, const float *b, void *out, int W, int H,
-                        int n, int S, int *err, int sms, cudaStream_t s, const __nv_bfloat16 *mask = nullptr) {
+                        int n, int S, int *err, int sms, cudaStream_t s, const __nv_bfloat16 *mask = nullptr,
+                        float *db = nullptr) {
     auto kern = k_conv_fwd_tc<CIN, COUT, RELU, OUTF32, LABELS, NS, BWD>;
     const int smem = tc_smem_bytes(CIN, COUT, !OUTF32 && !LABELS, NS);
     const int threads = (tc_epi_warps(COUT) + 2) * 32;
@@ -1008,7 +1123,7 @@ cudaError_t conv_fwd_tc(const CUtensorMap &in_map, const __nv_bfloat16 *wf, cons
     per_sm = std::max(per_sm, 1);
     const long long tiles = (long long)n * H * ((W + kTcOut - 1) / kTcOut);
     const int grid = (int)(tiles < (long long)per_sm * sms ? tiles : (long long)per_sm * sms);
-    kern<<<grid, threads, smem, s>>>(in_map, wf, b, out, W, H, n, S, err, mask);
+    kern<<<grid, threads, smem, s>>>(in_map, wf, b, out, W, H, n, S, err, mask, db);
     return cudaGetLastError();
 }
 
@@ -1016,7 +1131,7 @@ template <int CIN, int COUT>
 cudaError_t conv_bwd_weight_tc(const __nv_bfloat16 *a_in, const __nv_bfloat16 *dz, int W, int H, int n,
                                float *partial, int blocks, int *err, cudaStream_t s) {
     auto kern = k_conv_bwd_weight_tc<CIN, COUT>;
-    const int smem = wg_smem_bytes(CIN, COUT);
+    const int smem = wg_smem_bytes(COUT);
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     kern<<<blocks, kWgThreads, smem, s>>>(a_in, dz, W, H, n, partial, err);
@@ -1037,14 +1152,17 @@ cudaError_t conv_fwd(const slic_net_ctx *nc, int l, const __nv_bfloat16 *wf, con
 }
 
 // Forward pass into n->logits, or, with labels_out, straight to labels.
+// (the logits into `logits` instead of n->logits when given, 16-byte aligned)
 slic_status forward_all(slic_net_ctx *n, int batch, const uint8_t *d_images, cudaStream_t s,
-                        int32_t *labels_out = nullptr, const uint8_t *const *d_table = nullptr, int C = 3) {
+                        int32_t *labels_out = nullptr, const uint8_t *const *d_table = nullptr, int C = 3,
+                        float *logits = nullptr) {
     const dim3 pg((n->W + 127) / 128, n->H, batch);
     k_net_prep<<<pg, 128, 0, s>>>(n->conv, d_images, d_table, n->W, n->H, C, n->S, n->m / (float)n->S, n->act[0]);
     cudaError_t e = cudaGetLastError();
     for (int l = 0; l < kLayers && e == cudaSuccess; ++l) {
         void *out = l < 3 ? static_cast<void *>(n->act[l + 1])
-                          : (labels_out ? static_cast<void *>(labels_out) : static_cast<void *>(n->logits));
+                          : (labels_out ? static_cast<void *>(labels_out)
+                                      : static_cast<void *>(logits ? logits : n->logits));
         e = conv_fwd(n, l, n->wf[l], n->b[l], out, n->W, n->H, batch, labels_out != nullptr, s);
     }
     if (e != cudaSuccess) return nfail(n, SLIC_ERR_CUDA, std::string("network forward launch: ") + cudaGetErrorString(e));
@@ -1055,46 +1173,45 @@ slic_status forward_all(slic_net_ctx *n, int batch, const uint8_t *d_images, cud
 slic_status backward_all(slic_net_ctx *n, int batch, const uint8_t *d_targets, cudaStream_t s) {
     const int W = n->W, H = n->H;
     const long long n_px = (long long)W * H * batch;
-    cudaError_t e = cudaMemsetAsync(n->stats, 0, 2 * sizeof(float), s);
+    cudaError_t e = cudaMemsetAsync(n->bg[0], 0, (kBiases + 2) * sizeof(float), s);  // (and the statistics)
     if (e == cudaSuccess) {
-        k_softmax_ce<<<(unsigned)((n_px + 255) / 256), 256, 0, s>>>(n->logits, d_targets, W, H, batch, n->S,
-                                                                   1.0f / (float)n_px, n->dzA, n->stats);
+        const long long blocks = std::min<long long>((n_px + 255) / 256, 8LL * n->sms);
+        k_softmax_ce<<<(unsigned)blocks, 256, 0, s>>>(n->logits, d_targets, W, H, batch, n->S, 1.0f / (float)n_px,
+                                                     n->dzA, n->stats, n->bg[kLayers - 1]);
         e = cudaGetLastError();
     }
     __nv_bfloat16 *dz = n->dzA, *dz_prev = n->dzB;
+    float *partial = n->partial + kWeights * n->partial_blocks;
     for (int l = kLayers - 1; l >= 0 && e == cudaSuccess; --l) {
-        const int cin = kCinPad[l], cout = kCoutPad[l];
-        // weight gradient of layer l from its input act[l] and dz (per-CTA
-        // partials on the tensor cores, then their sum)
+        // weight gradient of layer l from its input act[l] and dz: per-CTA
+        // partials on the tensor cores, added up after the last layer
+        partial -= wcount(l) * n->partial_blocks;
         if (l == 0)
-            e = conv_bwd_weight_tc<16, 32>(n->act[0], dz, W, H, batch, n->partial, n->partial_blocks, n->tc_err, s);
+            e = conv_bwd_weight_tc<16, 32>(n->act[0], dz, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
         else if (l < 3)
-            e = conv_bwd_weight_tc<32, 32>(n->act[l], dz, W, H, batch, n->partial, n->partial_blocks, n->tc_err, s);
+            e = conv_bwd_weight_tc<32, 32>(n->act[l], dz, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
         else
-            e = conv_bwd_weight_tc<32, 16>(n->act[l], dz, W, H, batch, n->partial, n->partial_blocks, n->tc_err, s);
-        if (e != cudaSuccess) break;
-        const int cnt = 9 * cin * cout;
-        k_reduce_partials<<<(cnt + 255) / 256, 256, 0, s>>>(n->partial, n->partial_blocks, cnt, n->wg[l]);
-        e = cudaMemsetAsync(n->bg[l], 0, sizeof(float) * cout, s);
-        if (e != cudaSuccess) break;
-        if (cout == 32)
-            k_bias_grad<32><<<n->partial_blocks, 256, 0, s>>>(dz, n_px, n->bg[l]);
-        else
-            k_bias_grad<16><<<n->partial_blocks, 256, 0, s>>>(dz, n_px, n->bg[l]);
-        e = cudaGetLastError();
+            e = conv_bwd_weight_tc<32, 16>(n->act[l], dz, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
         if (l > 0 && e == cudaSuccess) {
-            // dz of layer l-1 (its output act[l] is layer l's input), on the
-            // tensor cores: the forward convolution in its BWD form, reading
-            // dz through its tensor map (dzA: 16 channels for l = 3, else 32)
+            // dz of layer l-1 (its output act[l] is layer l's input) and that
+            // layer's bias gradient, on the tensor cores: the forward
+            // convolution in its BWD form, reading dz through its tensor map
+            // (dzA: 16 channels for l = 3, else 32)
             const CUtensorMap &m = n->dz_map[l == 3 ? 0 : (dz == n->dzB ? 1 : 2)];
             if (l < 3)
                 e = conv_fwd_tc<32, 32, false, false, false, 3, true>(m, n->wb[l], nullptr, dz_prev, W, H, batch,
-                                                                      n->S, n->tc_err, n->sms, s, n->act[l]);
+                                                                      n->S, n->tc_err, n->sms, s, n->act[l],
+                                                                      n->bg[l - 1]);
             else
                 e = conv_fwd_tc<16, 32, false, false, false, 4, true>(m, n->wb[l], nullptr, dz_prev, W, H, batch,
-                                                                      n->S, n->tc_err, n->sms, s, n->act[l]);
+                                                                      n->S, n->tc_err, n->sms, s, n->act[l],
+                                                                      n->bg[l - 1]);
             std::swap(dz, dz_prev);
         }
+    }
+    if (e == cudaSuccess) {
+        k_reduce_partials<<<(unsigned)(kWeights / 32), 256, 0, s>>>(n->partial, n->partial_blocks, n->grads);
+        e = cudaGetLastError();
     }
     if (e != cudaSuccess) return nfail(n, SLIC_ERR_CUDA, std::string("network backward launch: ") + cudaGetErrorString(e));
     return SLIC_OK;
@@ -1160,17 +1277,28 @@ slic_status slic_net_create(int max_batch, int width, int height, int S, float m
     bool ok = true;
     for (int l = 0; l < kLayers && ok; ++l) {
         ok = nalloc(n, &n->w[l], wcount(l)) && nalloc(n, &n->wm[l], wcount(l)) && nalloc(n, &n->wv[l], wcount(l)) &&
-             nalloc(n, &n->wg[l], wcount(l)) && nalloc(n, &n->b[l], kCoutPad[l]) && nalloc(n, &n->bm[l], kCoutPad[l]) &&
-             nalloc(n, &n->bv[l], kCoutPad[l]) && nalloc(n, &n->bg[l], kCoutPad[l]) &&
+             nalloc(n, &n->b[l], kCoutPad[l]) && nalloc(n, &n->bm[l], kCoutPad[l]) &&
+             nalloc(n, &n->bv[l], kCoutPad[l]) &&
              nalloc(n, &n->wf[l], wcount(l)) && nalloc(n, &n->wb[l], wcount(l)) &&
              nalloc(n, &n->act[l], px * kCinPad[l]);
     }
     ok = ok && nalloc(n, &n->logits, px * 16) && nalloc(n, &n->dzA, px * 32) && nalloc(n, &n->dzB, px * 32) &&
-         nalloc(n, &n->partial, (size_t)n->partial_blocks * 9 * 32 * 32) && nalloc(n, &n->stats, 2) &&
+         nalloc(n, &n->partial, kWeights * n->partial_blocks) && nalloc(n, &n->grads, kWeights + kBiases + 2) &&
+         cudaMemset(n->grads, 0, sizeof(float) * (kWeights + kBiases + 2)) == cudaSuccess &&
          nalloc(n, &n->tc_err, 1) && cudaMemset(n->tc_err, 0, sizeof(int)) == cudaSuccess;
     if (!ok) {
         slic_net_destroy(n);
         return nfail(nullptr, SLIC_ERR_NOMEM, "device allocation for the network failed");
+    }
+    {
+        float *wg = n->grads, *bg = n->grads + kWeights;
+        for (int l = 0; l < kLayers; ++l) {
+            n->wg[l] = wg;
+            n->bg[l] = bg;
+            wg += wcount(l);
+            bg += kCoutPad[l];
+        }
+        n->stats = bg;
     }
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     for (int l = 0; l < kLayers && ok; ++l) {
@@ -1312,13 +1440,17 @@ slic_status slic_net_forward(slic_net n, int batch, const uint8_t *d_images, flo
     if (batch <= 0 || batch > n->max_batch || !d_images) return nfail(n, SLIC_ERR_INVALID, "bad batch or images");
     cudaStream_t s = (cudaStream_t)stream;
     if (d_labels && !d_logits) return forward_all(n, batch, d_images, s, d_labels);  // labels fused into the last layer
-    slic_status st = forward_all(n, batch, d_images, s);
+    // the last layer stores the logits where the caller wants them (a copy
+    // of 64 B/px took 0.16 ms of 1.18 for four 1080p images)
+    const bool direct = d_logits && ((uintptr_t)d_logits & 15) == 0;
+    float *const logits = direct ? d_logits : n->logits;
+    slic_status st = forward_all(n, batch, d_images, s, nullptr, nullptr, 3, logits);
     if (st != SLIC_OK) return st;
     const long long n_px = (long long)n->W * n->H * batch;
     cudaError_t e = cudaSuccess;
-    if (d_logits) e = cudaMemcpyAsync(d_logits, n->logits, sizeof(float) * 16 * n_px, cudaMemcpyDeviceToDevice, s);
+    if (d_logits && !direct) e = cudaMemcpyAsync(d_logits, n->logits, sizeof(float) * 16 * n_px, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess && d_labels) {
-        k_net_labels<<<(unsigned)((n_px + 255) / 256), 256, 0, s>>>(n->logits, n->W, n->H, batch, n->S, d_labels);
+        k_net_labels<<<(unsigned)((n_px + 255) / 256), 256, 0, s>>>(logits, n->W, n->H, batch, n->S, d_labels);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return nfail(n, SLIC_ERR_CUDA, std::string("network output: ") + cudaGetErrorString(e));
