@@ -507,6 +507,20 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
         Stepper w(blockIdx.x, G, tiles_x, (unsigned)H);
         for (unsigned t = blockIdx.x; t < total; t += G, ++j, w.advance()) {
             const int bf = (int)(j & 1u);
+            const unsigned tx = w.a;
+            const int y = (int)w.b, img = (int)w.c;
+            const int xw = (int)tx * kTcOut + kTcSeg * quarter;  // output pixel of lane 0
+            const size_t row0 = (size_t)img * H * W + (size_t)y * W;
+            const bool in_image = lane < kTcSeg && xw + lane < W;
+            uint4 m0 = make_uint4(0u, 0u, 0u, 0u), m1 = m0;
+            if (BWD && in_image) {
+                // the previous layer's stored output, in flight while the
+                // accumulator is awaited (loaded after it, a third of the
+                // kernel's time was this load's latency)
+                const uint4 *mp = reinterpret_cast<const uint4 *>(mask + (row0 + xw + lane) * COUT + c0);
+                m0 = __ldg(mp);
+                m1 = __ldg(mp + 1);
+            }
             if (!__all_sync(0xffffffffu, tc_wait_ab(&tfull[bf], (j >> 1) & 1u, abort))) {
                 if (lane == 0) fail();
                 break;
@@ -532,22 +546,13 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                 unpack2f(p, v[c], v[c + 1]);
             }
 
-            const unsigned tx = w.a;
-            const int y = (int)w.b, img = (int)w.c;
-            const int xw = (int)tx * kTcOut + kTcSeg * quarter;  // output pixel of lane 0
-            const size_t row0 = (size_t)img * H * W + (size_t)y * W;
             if constexpr (BWD) {
                 // ReLU derivative of the previous layer: its stored output > 0
-                const int x = xw + lane;
-                if (lane < kTcSeg && x < W) {
-                    const uint4 *mp = reinterpret_cast<const uint4 *>(mask + (row0 + x) * COUT + c0);
-                    const uint4 m0 = mp[0], m1 = mp[1];
-                    const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        const uint32_t h = (mw[c >> 1] >> (16 * (c & 1))) & 0xFFFFu;  // bf16 bits
-                        if (!(__uint_as_float(h << 16) > 0.0f)) v[c] = 0.0f;
-                    }
+                for (int c = 0; c < 16; ++c) {
+                    const uint32_t h = (mw[c >> 1] >> (16 * (c & 1))) & 0xFFFFu;  // bf16 bits
+                    if (!(__uint_as_float(h << 16) > 0.0f)) v[c] = 0.0f;
                 }
             }
             if constexpr (STAGED) {
@@ -565,7 +570,7 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                     *reinterpret_cast<uint4 *>(ow + lane * 32 + ((k ^ ((lane >> 2) & 1)) << 4)) =
                         make_uint4(w4[0], w4[1], w4[2], w4[3]);
                     if constexpr (BWD) {
-                        if (lane < kTcSeg && xw + lane < W) {
+                        if (in_image) {
 #pragma unroll
                             for (int h = 0; h < 4; ++h)  // the rounded pair, as stored
                                 bv[4 * k + h] = add2(bv[4 * k + h], pack2f(__uint_as_float(w4[h] << 16),
@@ -645,79 +650,75 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
 //
 // The contraction runs over pixels, and both tensors are NHWC, so both
 // operands are MN-major as they lie in memory: no transposition. A stage
-// holds kWgK columns of four input rows (r-1 .. r+2) and two dZ rows (r, r+1)
-// in planes of 8 channels, a pixel's 16 bytes after its neighbour's: core
-// matrices of 8 pixels x 8 channels, 128 bytes apart along K (pixels) and one
-// plane apart along M or N. One tcgen05.mma of M 128 (4 input rows x 32
-// channels) x N 2 * COUT (2 dZ rows) x K 16 forms every pair of an input row i
-// and a dZ row j at one horizontal offset; the pairs with dy = i - j in 0..2
-// (six of eight) are the gradient's. The horizontal tap dx is the start
-// address of A, 16 bytes (one pixel) further per step, with an accumulator
-// per dx in tensor memory.
+// holds, each copied by one tensor-map box with a swizzle as wide as a pixel,
+// kWgCols columns of four input rows (r-1 .. r+2) and kWgK columns of two dZ
+// rows (r, r+1). One tcgen05.mma of M 128 (4 input rows x 32 channels) x N
+// 2 * COUT (2 dZ rows) x K 16 forms every pair of an input row i and a dZ row
+// j at one horizontal offset; the pairs with dy = i - j in 0..2 (six of eight)
+// are the gradient's. The horizontal tap dx moves the start of A by one pixel
+// per step, with an accumulator per dx in tensor memory. (With 16 channels
+// four rows fill half of M; the other half reads whatever follows, and its
+// accumulator rows are not used.)
 //
-// Eight warps copy (cp.async, 16 bytes a lane, zeros outside the image) into
-// a ring of kWgStages stages, one thread issues the MMAs. The plane pitch of
-// kWgK + 2 pixels makes the eight 16-byte pieces of a quarter-warp land in
-// different banks. Per stage (128 pixels) 12 MMAs of about 48 cycles (6 KB of
-// operands each at 128 B/clk) bound the kernel: 32 us for 2.1 Mpx. Staging the
-// operands by transposing rows through shared memory (K-major operands, three
-// CTA barriers per output row) took 310 us per 32 -> 32 layer.
+// One thread copies into a ring of kWgStages stages, one issues the MMAs, four
+// warps store the sums. Per stage (128 pixels) 12 MMAs of about 48 cycles (6 KB
+// of operands each at 128 B/clk) would take 32 us for 2.1 Mpx, the copies'
+// 208 B/px from L2 about 45 us. Staging K-major operands by transposing rows
+// through shared memory took 310 us per 32 -> 32 layer; MN-major planes of 8
+// channels filled by 16-byte cp.async 133 us (bound by the loads in flight).
 // ---------------------------------------------------------------------------
 constexpr int kWgK = 64;      // pixels (columns) of a stage
+constexpr int kWgCols = 72;   // input columns copied: kWgK + 2, rounded up to whole swizzle patterns (8 pixels)
 constexpr int kWgStages = 4;
-constexpr int kWgLoaders = 256;
-constexpr int kWgThreads = kWgLoaders + 32;
-constexpr int kWgPlane = (kWgK + 2) * 16;   // bytes of one 8-channel plane of one row
-__host__ __device__ constexpr int wg_a_bytes() { return 16 * kWgPlane; }  // 4 rows x 4 planes (2 of them zero for 16 channels)
-__host__ __device__ constexpr int wg_b_bytes(int cout) { return 2 * (cout / 8) * kWgPlane; }
-__host__ __device__ constexpr int wg_stage_bytes(int cout) { return wg_a_bytes() + wg_b_bytes(cout); }
-__host__ __device__ constexpr int wg_smem_bytes(int cout) {
-    return 128 + kWgStages * wg_stage_bytes(cout) + (2 * kWgStages + 1) * 8 + 16;
+constexpr int kWgThreads = 192;  // four epilogue warps, producer, issuer
+__host__ __device__ constexpr int wg_a_bytes(int cin) { return 4 * kWgCols * cin * 2; }
+__host__ __device__ constexpr int wg_b_bytes(int cout) { return 2 * kWgK * cout * 2; }
+__host__ __device__ constexpr int wg_stage_bytes(int cin, int cout) { return wg_a_bytes(cin) + wg_b_bytes(cout); }
+// (1 KB for aligning the ring, 1 KB past it for the rows beyond A of the last stage)
+__host__ __device__ constexpr int wg_ring_bytes(int cin, int cout) { return kWgStages * wg_stage_bytes(cin, cout) + 1024; }
+__host__ __device__ constexpr int wg_smem_bytes(int cin, int cout) {
+    return 1024 + wg_ring_bytes(cin, cout) + (2 * kWgStages + 1) * 8 + 16;
 }
 
-// A 16-byte asynchronous copy, zeros when !ok (nothing is read then).
-__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool ok) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16u : 0u) : "memory");
+// Descriptor of an MN-major operand with a 32- or 64-byte swizzle (a K row,
+// here a pixel, is one swizzle span of 16 or 32 elements): lbo, bytes from one
+// group of 16 or 32 rows of M (or N) to the next; sbo, from 8 pixels to the
+// next 8.
+template <int C>
+__device__ __forceinline__ unsigned long long tc_desc_mn(unsigned addr, unsigned lbo) {
+    return (unsigned long long)((addr & 0x3FFFFu) >> 4) | ((unsigned long long)((lbo & 0x3FFFFu) >> 4) << 16) |
+           ((unsigned long long)((8u * C * 2u) >> 4) << 32) | (1ull << 46) | ((C == 32 ? 4ull : 6ull) << 61);
 }
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bfloat16 *a_in,
-                                                                   const __nv_bfloat16 *dz, int W, int H, int n_img,
-                                                                   float *partial, int *err) {
-    constexpr int STAGE = wg_stage_bytes(COUT), A_BYTES = wg_a_bytes();
-    constexpr int APL = CIN / 8, BPL = COUT / 8;   // real planes per row
+__global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __grid_constant__ CUtensorMap a_map,
+                                                                   const __grid_constant__ CUtensorMap z_map, int W,
+                                                                   int H, int n_img, float *partial, int *err) {
+    constexpr int STAGE = wg_stage_bytes(CIN, COUT), A_BYTES = wg_a_bytes(CIN);
     constexpr int NN = 2 * COUT;
     constexpr int TCOLS = 3 * NN <= 128 ? 128 : 256;
     static_assert((CIN == 16 || CIN == 32) && (COUT == 16 || COUT == 32), "shapes of the weight-gradient kernel");
+    static_assert(STAGE % 1024 == 0 && A_BYTES % 512 == 0, "stages and rows must keep the swizzle pattern aligned");
+    static_assert(((128 / CIN - 1) * kWgCols + kWgK + 2) * CIN * 2 <= STAGE + 1024, "rows beyond A stay in the ring");
+    static_assert(9 * CIN * (COUT + 1) * 4 <= kWgStages * STAGE, "the sums reuse the ring");
     extern __shared__ __align__(16) unsigned char wg_dyn[];
     unsigned char *const ring =
-        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(wg_dyn) + 127) & ~(uintptr_t)127);
-    static_assert(9 * CIN * (COUT + 1) * 4 <= kWgStages * STAGE, "the sums reuse the ring");
-    unsigned long long *const full = reinterpret_cast<unsigned long long *>(ring + kWgStages * STAGE);
+        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(wg_dyn) + 1023) & ~(uintptr_t)1023);
+    unsigned long long *const full = reinterpret_cast<unsigned long long *>(ring + wg_ring_bytes(CIN, COUT));
     unsigned long long *const empty = full + kWgStages;
     unsigned long long *const fin = empty + kWgStages;
     unsigned *const tmem_slot = reinterpret_cast<unsigned *>(fin + 1);
     volatile int *const abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int PRODUCER = 4, ISSUER = 5;
 
-    if (CIN == 16) {  // planes 2 and 3 of every input row stay zero
-        for (int i = tid; i < kWgStages * 4 * 2 * (kWgPlane / 16); i += kWgThreads) {
-            const int q = i % (kWgPlane / 16), p = i / (kWgPlane / 16);  // p = (stage * 4 + row) * 2 + plane - 2
-            *reinterpret_cast<uint4 *>(ring + (p >> 3) * STAGE + (((p >> 1) & 3) * 4 + 2 + (p & 1)) * kWgPlane + q * 16) =
-                make_uint4(0u, 0u, 0u, 0u);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
     if (tid == 0) {
-        for (int i = 0; i < kWgStages; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc_smem(&full[i])), "n"(kWgLoaders / 32));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(&empty[i])));
-        }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(fin)));
+        for (int i = 0; i < 2 * kWgStages + 1; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(&full[i])));
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == kWgLoaders / 32) {
+    if (warp == ISSUER) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)),
                      "n"(TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -736,67 +737,33 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bf
         *abort = 1;
         atomicOr(err, 1);
     };
-    if (warp < kWgLoaders / 32) {
-        // ---- loaders ----
-        constexpr int kAhead = kWgStages - 1;
-        bool ok = true;
+    if (warp == PRODUCER && lane == 0) {
         Stepper u(blockIdx.x, gridDim.x, segs, pairs);
-        for (int j = 0; j < n_stage + kAhead; ++j) {
-            if (j < n_stage) {
-                const int s = j % kWgStages;
-                if (j >= kWgStages && !__all_sync(0xffffffffu, tc_wait_ab(&empty[s], (j / kWgStages - 1) & 1, abort))) {
-                    if (lane == 0) fail();
-                    ok = false;
-                    break;
-                }
-                const int r = 2 * (int)u.b, x0 = (int)u.a * kWgK;
-                const size_t base = (size_t)u.c * H * W;
-                u.advance();
-                const unsigned st = tc_smem(ring + s * STAGE);
-                {
-                    // piece: plane fastest, then pixel, then row
-                    constexpr int PER = kWgLoaders / (kWgK * APL);  // rows per sweep
-                    const int pl = tid % APL, px = (tid / APL) % kWgK, row0 = tid / (APL * kWgK);
-#pragma unroll
-                    for (int i = 0; i < 4 / PER; ++i) {
-                        const int row = row0 + i * PER, yy = r - 1 + row, gx = x0 - 1 + px;
-                        const bool in = gx >= 0 && gx < W && yy >= 0 && yy < H;
-                        cp_async16(st + (row * 4 + pl) * kWgPlane + px * 16,
-                                   a_in + (in ? (base + (size_t)yy * W + gx) * CIN + pl * 8 : 0), in);
-                    }
-                    if (tid < 4 * 2 * APL) {  // the last two columns
-                        const int hp = tid % APL, hx = kWgK + (tid / APL) % 2, row = tid / (2 * APL);
-                        const int yy = r - 1 + row, gx = x0 - 1 + hx;
-                        const bool in = gx < W && yy >= 0 && yy < H;
-                        cp_async16(st + (row * 4 + hp) * kWgPlane + hx * 16,
-                                   a_in + (in ? (base + (size_t)yy * W + gx) * CIN + hp * 8 : 0), in);
-                    }
-                }
-                {
-                    constexpr int PER = kWgLoaders / (kWgK * BPL);
-                    const int pl = tid % BPL, px = (tid / BPL) % kWgK, row0 = tid / (BPL * kWgK);
-#pragma unroll
-                    for (int i = 0; i < 2 / PER; ++i) {
-                        const int row = row0 + i * PER, yy = r + row, gx = x0 + px;
-                        const bool in = gx < W && yy < H;
-                        cp_async16(st + A_BYTES + (row * BPL + pl) * kWgPlane + px * 16,
-                                   dz + (in ? (base + (size_t)yy * W + gx) * COUT + pl * 8 : 0), in);
-                    }
-                }
+        int issued = 0;
+        for (int j = 0; j < n_stage; ++j, ++issued, u.advance()) {
+            const int s = j % kWgStages;
+            if (j >= kWgStages && !tc_wait_ab(&empty[s], (j / kWgStages - 1) & 1, abort)) {
+                fail();
+                break;
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            const int d = j - kAhead;  // stage whose copies are complete once kAhead groups are left in flight
-            if (d >= 0) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(kAhead) : "memory");
-                // generic-proxy writes -> visible to the tensor core
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) tc_arrive(&full[d % kWgStages]);
-            }
+            const unsigned b = tc_smem(&full[s]), dst = tc_smem(ring + s * STAGE);
+            const int x0 = (int)u.a * kWgK, r = 2 * (int)u.b, img = (int)u.c;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"((unsigned)STAGE)
+                         : "memory");
+            asm volatile(
+                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
+                "{%2, %3, %4, %5}], [%6];" ::"r"(dst),
+                "l"(reinterpret_cast<uint64_t>(&a_map)), "r"(0), "r"(x0 - 1), "r"(r - 1), "r"(img), "r"(b)
+                : "memory");
+            asm volatile(
+                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
+                "{%2, %3, %4, %5}], [%6];" ::"r"(dst + A_BYTES),
+                "l"(reinterpret_cast<uint64_t>(&z_map)), "r"(0), "r"(x0), "r"(r), "r"(img), "r"(b)
+                : "memory");
         }
-        if (!ok) asm volatile("cp.async.wait_all;" ::: "memory");  // no copy may outlive the CTA
-    } else if (lane == 0) {
-        // ---- MMA issuer ----
+        // every copy lands before the shared memory is released
+        for (int j = max(0, issued - kWgStages); j < issued; ++j) tc_wait(&full[j % kWgStages], (j / kWgStages) & 1);
+    } else if (warp == ISSUER && lane == 0) {
         const unsigned idesc = tc_idesc(128, NN) | (1u << 15) | (1u << 16);  // A and B are MN-major
         for (int j = 0; j < n_stage; ++j) {
             const int s = j % kWgStages;
@@ -810,8 +777,8 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bf
             for (int dx = 0; dx < 3; ++dx) {
 #pragma unroll
                 for (int kc = 0; kc < kWgK / 16; ++kc) {
-                    const unsigned long long ad = tc_desc(a0 + (dx + 16 * kc) * 16, 128, kWgPlane);
-                    const unsigned long long bd = tc_desc(b0 + 256 * kc, 128, kWgPlane);
+                    const unsigned long long ad = tc_desc_mn<CIN>(a0 + (16 * kc + dx) * CIN * 2, kWgCols * CIN * 2);
+                    const unsigned long long bd = tc_desc_mn<COUT>(b0 + 16 * kc * COUT * 2, kWgK * COUT * 2);
                     const unsigned acc = (j > 0 || kc > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -831,21 +798,22 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bf
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // Warp i (< 4) holds input row i (lanes = channels): the column block of
-    // dZ row j belongs to dy = i - j. First the blocks of j = 0, then those
-    // of j = 1 added, in shared memory (the ring is free now).
+    // Accumulator lane m is channel m % CIN of input row i = m / CIN; the
+    // column block of dZ row j belongs to dy = i - j. First the blocks of
+    // j = 0, then those of j = 1 added, in shared memory (the ring is free).
     float *const sum = reinterpret_cast<float *>(ring);  // [tap][ci][COUT + 1], padded against bank conflicts
+    const int row = tid / CIN, ci = tid % CIN;
 #pragma unroll
     for (int jrow = 0; jrow < 2; ++jrow) {
-        const int dy = warp - jrow;
+        const int dy = row - jrow;
         if (warp < 4) {
 #pragma unroll
             for (int dx = 0; dx < 3; ++dx) {
                 float v[COUT];
                 tc_ld_cols<COUT>(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(dx * NN + jrow * COUT), v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (dy >= 0 && dy <= 2 && lane < CIN) {
-                    float *dst = sum + ((dy * 3 + dx) * CIN + lane) * (COUT + 1);
+                if (row < 4 && dy >= 0 && dy <= 2) {
+                    float *dst = sum + ((dy * 3 + dx) * CIN + ci) * (COUT + 1);
 #pragma unroll
                     for (int q = 0; q < COUT; ++q) {
                         const float w = n_stage > 0 ? v[q] : 0.0f;
@@ -861,7 +829,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_bwd_weight_tc(const __nv_bf
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp == kWgLoaders / 32) {
+    if (warp == ISSUER) {
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TCOLS));
     }
@@ -1063,6 +1031,9 @@ struct slic_net_ctx {
     // the gradient buffers as inputs of the input-gradient convolutions:
     // dzA with 16 channels (dL/dlogits), dzB and dzA with 32
     CUtensorMap dz_map[3] = {};
+    // the same tensors in the weight gradient's boxes: kWgCols columns of four
+    // input rows, kWgK columns of two gradient rows
+    CUtensorMap wg_in_map[kLayers] = {}, wg_dz_map[3] = {};
     int sms = 0;
     ConvConsts conv{};
     std::string err;
@@ -1128,13 +1099,13 @@ cudaError_t conv_fwd_tc(const CUtensorMap &in_map, const __nv_bfloat16 *wf, cons
 }
 
 template <int CIN, int COUT>
-cudaError_t conv_bwd_weight_tc(const __nv_bfloat16 *a_in, const __nv_bfloat16 *dz, int W, int H, int n,
+cudaError_t conv_bwd_weight_tc(const CUtensorMap &a_map, const CUtensorMap &z_map, int W, int H, int n,
                                float *partial, int blocks, int *err, cudaStream_t s) {
     auto kern = k_conv_bwd_weight_tc<CIN, COUT>;
-    const int smem = wg_smem_bytes(COUT);
+    const int smem = wg_smem_bytes(CIN, COUT);
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, kWgThreads, smem, s>>>(a_in, dz, W, H, n, partial, err);
+    kern<<<blocks, kWgThreads, smem, s>>>(a_map, z_map, W, H, n, partial, err);
     return cudaGetLastError();
 }
 
@@ -1186,18 +1157,19 @@ slic_status backward_all(slic_net_ctx *n, int batch, const uint8_t *d_targets, c
         // weight gradient of layer l from its input act[l] and dz: per-CTA
         // partials on the tensor cores, added up after the last layer
         partial -= wcount(l) * n->partial_blocks;
+        const int zi = l == 3 ? 0 : (dz == n->dzB ? 1 : 2);  // dzA: 16 channels for l = 3, else 32
+        const CUtensorMap &z = n->wg_dz_map[zi];
         if (l == 0)
-            e = conv_bwd_weight_tc<16, 32>(n->act[0], dz, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
+            e = conv_bwd_weight_tc<16, 32>(n->wg_in_map[0], z, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
         else if (l < 3)
-            e = conv_bwd_weight_tc<32, 32>(n->act[l], dz, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
+            e = conv_bwd_weight_tc<32, 32>(n->wg_in_map[l], z, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
         else
-            e = conv_bwd_weight_tc<32, 16>(n->act[l], dz, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
+            e = conv_bwd_weight_tc<32, 16>(n->wg_in_map[l], z, W, H, batch, partial, n->partial_blocks, n->tc_err, s);
         if (l > 0 && e == cudaSuccess) {
             // dz of layer l-1 (its output act[l] is layer l's input) and that
             // layer's bias gradient, on the tensor cores: the forward
             // convolution in its BWD form, reading dz through its tensor map
-            // (dzA: 16 channels for l = 3, else 32)
-            const CUtensorMap &m = n->dz_map[l == 3 ? 0 : (dz == n->dzB ? 1 : 2)];
+            const CUtensorMap &m = n->dz_map[zi];
             if (l < 3)
                 e = conv_fwd_tc<32, 32, false, false, false, 3, true>(m, n->wb[l], nullptr, dz_prev, W, H, batch,
                                                                       n->S, n->tc_err, n->sms, s, n->act[l],
@@ -1301,25 +1273,24 @@ slic_status slic_net_create(int max_batch, int width, int height, int S, float m
         n->stats = bg;
     }
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    for (int l = 0; l < kLayers && ok; ++l) {
-        const cuuint64_t c = (cuuint64_t)kCinPad[l];
+    // [max_batch][H][W][c] bf16 in boxes of cols x rows pixels, a pixel's
+    // channels (32 or 64 bytes) as wide as the swizzle
+    auto encode = [&](CUtensorMap *map, void *base, cuuint64_t c, int cols, int rows) {
         const cuuint64_t dims[4] = {c, (cuuint64_t)width, (cuuint64_t)height, (cuuint64_t)max_batch};
         const cuuint64_t strides[3] = {c * 2, c * 2 * width, c * 2 * width * height};
-        const cuuint32_t box[4] = {(cuuint32_t)c, 32, 1, 1};
+        const cuuint32_t box[4] = {(cuuint32_t)c, (cuuint32_t)cols, (cuuint32_t)rows, 1};
         const cuuint32_t ones[4] = {1, 1, 1, 1};
-        ok = enc && enc(&n->in_map[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, n->act[l], dims, strides, box, ones,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    }
+        return enc && enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, ones,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    for (int l = 0; l < kLayers && ok; ++l)
+        ok = encode(&n->in_map[l], n->act[l], kCinPad[l], 32, 1) &&
+             encode(&n->wg_in_map[l], n->act[l], kCinPad[l], kWgCols, 4);
     for (int k = 0; k < 3 && ok; ++k) {
-        const cuuint64_t c = k == 0 ? 16 : 32;
-        const cuuint64_t dims[4] = {c, (cuuint64_t)width, (cuuint64_t)height, (cuuint64_t)max_batch};
-        const cuuint64_t strides[3] = {c * 2, c * 2 * width, c * 2 * width * height};
-        const cuuint32_t box[4] = {(cuuint32_t)c, 32, 1, 1};
-        const cuuint32_t ones[4] = {1, 1, 1, 1};
-        ok = enc(&n->dz_map[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, k == 1 ? n->dzB : n->dzA, dims, strides, box,
-                 ones, CU_TENSOR_MAP_INTERLEAVE_NONE, c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
-                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+        void *const dz = k == 1 ? n->dzB : n->dzA;
+        ok = encode(&n->dz_map[k], dz, k == 0 ? 16 : 32, 32, 1) && encode(&n->wg_dz_map[k], dz, k == 0 ? 16 : 32, kWgK, 2);
     }
     if (!ok) {
         slic_net_destroy(n);
