@@ -157,10 +157,12 @@ __global__ void __launch_bounds__(128) k_net_prep(ConvConsts cc, const uint8_t *
 // The roles meet on mbarrier rings: NS input stages (full / empty) and two
 // accumulator buffers (full / empty).
 //
-// A work tile is 120 output pixels of one image row, 30 per TMEM lane
-// quarter (epilogue warp q % 4). Quarter q's 32 MMA rows (positions) are
-// x0-1+30q .. x0+30+30q, so the 30 outputs of a quarter need only its own
-// rows; all CIN channels of a position form one row of CIN*2 bytes, copied
+// A work tile is four segments of 30 output pixels of an image row, one per
+// TMEM lane quarter (epilogue warp q % 4), consecutive in the list of all
+// rows' segments: a tile may span rows, so a row of 256 pixels takes 9
+// segments and not 3 whole tiles of 120. A quarter's 32 MMA rows (positions)
+// are x0-1 .. x0+30 for the segment from x0, so its 30 outputs need only its
+// own rows; all CIN channels of a position form one row of CIN*2 bytes, copied
 // with the 32-byte (CIN 16) or 64-byte (CIN 32) swizzle, zeros outside the
 // image (the zero padding). For each kernel row dy one MMA chunk (M 128
 // positions x N 3*COUT x K16) takes all three horizontal taps at once:
@@ -173,9 +175,8 @@ __global__ void __launch_bounds__(128) k_net_prep(ConvConsts cc, const uint8_t *
 // 16-byte core matrices, leading offset = one 8-channel plane), staged once
 // per CTA.
 // ---------------------------------------------------------------------------
-constexpr int kTcOut = 120;               // output pixels per tile
 constexpr int kTcIn = 128;                // MMA rows (positions) per tile
-constexpr int kTcSeg = 30;                // outputs per lane quarter
+constexpr int kTcSeg = 30;                // outputs per lane quarter (segment)
 constexpr unsigned kTcWaitPolls = 1u << 20;
 
 __device__ __forceinline__ unsigned tc_smem(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -245,6 +246,11 @@ struct Stepper {
         }
     }
 };
+
+// All ones in each half of the word whose bf16 is above zero.
+__device__ __forceinline__ uint32_t positive2(uint32_t v) {
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&v), __floats2bfloat162_rn(0.0f, 0.0f));
+}
 
 // Two FP32 sums in one instruction (each rounded as the scalar addition).
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
@@ -400,8 +406,9 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tmem_slot;
-    const unsigned tiles_x = (unsigned)((W + kTcOut - 1) / kTcOut);
-    const unsigned total = (unsigned)n_img * (unsigned)H * tiles_x;  // < 2^31 (pixels < 2^31)
+    const unsigned segs_x = (unsigned)((W + kTcSeg - 1) / kTcSeg);
+    const unsigned segs = (unsigned)n_img * (unsigned)H * segs_x;  // < 2^31 (pixels < 2^31)
+    const unsigned total = (segs + 3) / 4;
     const unsigned G = gridDim.x;
     auto fail = [&]() {
         *abort = 1;
@@ -415,27 +422,35 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
             unsigned u = 0;       // completed rounds of the ring
             unsigned issued = 0;  // bit s: a copy was issued into stage s
             unsigned lastpar = 0; // bit s: parity of that copy's completion
-            Stepper w(blockIdx.x, G, tiles_x, (unsigned)H);
+            Stepper w(4 * blockIdx.x, 4 * G, segs_x, (unsigned)H);
             for (unsigned t = blockIdx.x; t < total; t += G, w.advance()) {
                 if (u > 0 && !tc_wait_ab(&empty[s], (u - 1) & 1u, abort)) {
                     fail();
                     break;
                 }
-                const unsigned tx = w.a;
-                const int y = (int)w.b, img = (int)w.c;
                 const unsigned b = tc_smem(&full[s]);
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(BOX) : "memory");
                 const unsigned dst0 = tc_smem(in_s + s * BOX);
+                int sx = (int)w.a, y = (int)w.b, img = (int)w.c;
 #pragma unroll
-                for (int dy = 0; dy < 3; ++dy) {
+                for (int q = 0; q < 4; ++q) {
+                    // (past the last segment: the rows of an image outside the
+                    // batch, or zeros; their results are not stored)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
+                    for (int dy = 0; dy < 3; ++dy) {
                         asm volatile(
                             "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
                             "{%2, %3, %4, %5}], [%6];" ::"r"(dst0 + (unsigned)((dy * kTcIn + 32 * q) * ROWB)),
-                            "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(0),
-                            "r"((int)tx * kTcOut - 1 + kTcSeg * q), "r"(y + dy - 1), "r"(img), "r"(b)
+                            "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(0), "r"(sx * kTcSeg - 1), "r"(y + dy - 1),
+                            "r"(img), "r"(b)
                             : "memory");
+                    }
+                    if (++sx == (int)segs_x) {
+                        sx = 0;
+                        if (++y == H) {
+                            y = 0;
+                            ++img;
+                        }
                     }
                 }
                 issued |= 1u << s;
@@ -497,29 +512,34 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32*(w%4) .. +31, channels 16*(w/4) .. +15 ----
         const int quarter = warp & 3, c0 = (warp >> 2) * 16;
-        // channel pairs: the layer's biases, or (BWD) this lane's sums of the
-        // results it stores, the bias gradient of the previous layer
+        // channel pairs: the layer's biases, or (BWD, four of them) this lane's
+        // sums of the results it stores, the bias gradient of the previous layer
         unsigned long long bv[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c)
             bv[c] = BWD ? 0ull : pack2f(bias[c0 + 2 * c], bias[c0 + 2 * c + 1]);
         unsigned j = 0;
-        Stepper w(blockIdx.x, G, tiles_x, (unsigned)H);
+        Stepper w(4 * blockIdx.x + quarter, 4 * G, segs_x, (unsigned)H);
         for (unsigned t = blockIdx.x; t < total; t += G, ++j, w.advance()) {
             const int bf = (int)(j & 1u);
-            const unsigned tx = w.a;
-            const int y = (int)w.b, img = (int)w.c;
-            const int xw = (int)tx * kTcOut + kTcSeg * quarter;  // output pixel of lane 0
-            const size_t row0 = (size_t)img * H * W + (size_t)y * W;
-            const bool in_image = lane < kTcSeg && xw + lane < W;
-            uint4 m0 = make_uint4(0u, 0u, 0u, 0u), m1 = m0;
-            if (BWD && in_image) {
-                // the previous layer's stored output, in flight while the
-                // accumulator is awaited (loaded after it, a third of the
-                // kernel's time was this load's latency)
-                const uint4 *mp = reinterpret_cast<const uint4 *>(mask + (row0 + xw + lane) * COUT + c0);
-                m0 = __ldg(mp);
-                m1 = __ldg(mp + 1);
+            const int y = (int)w.b, xw = (int)w.a * kTcSeg;  // xw: output pixel of lane 0
+            const size_t row0 = ((size_t)w.c * H + y) * W;
+            const int n_out = 4 * t + quarter < segs ? min(kTcSeg, W - xw) : 0;  // pixels of this segment
+            uint4 m[2] = {};
+            if constexpr (BWD) {
+                // The previous layer's stored outputs, in the store's chunks (8
+                // channels of pixel 16 i + lane / 2), in flight while the
+                // accumulator is awaited
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int pp = i * 16 + (lane >> 1);
+                    if (pp < n_out) {
+                        const __nv_bfloat16 *mp = mask + (row0 + xw + pp) * COUT + c0 + 8 * (lane & 1);
+                        asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                     : "=r"(m[i].x), "=r"(m[i].y), "=r"(m[i].z), "=r"(m[i].w)
+                                     : "l"(mp));
+                    }
+                }
             }
             if (!__all_sync(0xffffffffu, tc_wait_ab(&tfull[bf], (j >> 1) & 1u, abort))) {
                 if (lane == 0) fail();
@@ -546,15 +566,6 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                 unpack2f(p, v[c], v[c + 1]);
             }
 
-            if constexpr (BWD) {
-                // ReLU derivative of the previous layer: its stored output > 0
-                const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const uint32_t h = (mw[c >> 1] >> (16 * (c & 1))) & 0xFFFFu;  // bf16 bits
-                    if (!(__uint_as_float(h << 16) > 0.0f)) v[c] = 0.0f;
-                }
-            }
             if constexpr (STAGED) {
                 // Each lane packs its pixel's 32 bytes (16 channels) into the
                 // warp's staging rows (16-byte chunks swizzled by pixel
@@ -569,28 +580,33 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                                                              : pack_bf16(v[8 * k + 2 * h], v[8 * k + 2 * h + 1]);
                     *reinterpret_cast<uint4 *>(ow + lane * 32 + ((k ^ ((lane >> 2) & 1)) << 4)) =
                         make_uint4(w4[0], w4[1], w4[2], w4[3]);
-                    if constexpr (BWD) {
-                        if (in_image) {
-#pragma unroll
-                            for (int h = 0; h < 4; ++h)  // the rounded pair, as stored
-                                bv[4 * k + h] = add2(bv[4 * k + h], pack2f(__uint_as_float(w4[h] << 16),
-                                                                           __uint_as_float(w4[h] & 0xFFFF0000u)));
-                        }
-                    }
                 }
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     const int pp = i * 16 + (lane >> 1), k = lane & 1;
-                    const uint4 c = *reinterpret_cast<const uint4 *>(ow + pp * 32 + ((k ^ ((pp >> 2) & 1)) << 4));
-                    if (pp < kTcSeg && xw + pp < W)
+                    uint4 c = *reinterpret_cast<const uint4 *>(ow + pp * 32 + ((k ^ ((pp >> 2) & 1)) << 4));
+                    if constexpr (BWD) {
+                        // ReLU derivative of the previous layer (its stored
+                        // output > 0; zeros outside the segment)
+                        c.x &= positive2(m[i].x);
+                        c.y &= positive2(m[i].y);
+                        c.z &= positive2(m[i].z);
+                        c.w &= positive2(m[i].w);
+                        const uint32_t cw[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)  // the pair's sums, as stored
+                            bv[h] = add2(bv[h], pack2f(__uint_as_float(cw[h] << 16),
+                                                       __uint_as_float(cw[h] & 0xFFFF0000u)));
+                    }
+                    if (pp < n_out)
                         *reinterpret_cast<uint4 *>(static_cast<unsigned char *>(out) + (row0 + xw + pp) * 64 + c0 * 2 +
                                                    k * 16) = c;
                 }
                 __syncwarp();
             } else {
                 const int x = xw + lane;
-                if (lane < kTcSeg && x < W) {
+                if (lane < n_out) {
                     const size_t px = row0 + x;
                     if constexpr (LABELS) {
                         // argmax of the valid slots' logits (first maximum in
@@ -623,14 +639,14 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
         }
         if constexpr (BWD) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
+            for (int h = 0; h < 4; ++h) {
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) bv[c] = add2(bv[c], __shfl_xor_sync(0xffffffffu, bv[c], o));
+                for (int o = 16; o > 1; o >>= 1) bv[h] = add2(bv[h], __shfl_xor_sync(0xffffffffu, bv[h], o));
                 float lo, hi;
-                unpack2f(bv[c], lo, hi);
-                if (lane == c) {
-                    atomicAdd(&db[c0 + 2 * c], lo);
-                    atomicAdd(&db[c0 + 2 * c + 1], hi);
+                unpack2f(bv[h], lo, hi);
+                if (lane < 2) {  // lane k: channels c0 + 8 k ..
+                    atomicAdd(&db[c0 + 8 * lane + 2 * h], lo);
+                    atomicAdd(&db[c0 + 8 * lane + 2 * h + 1], hi);
                 }
             }
         }
@@ -1092,7 +1108,7 @@ cudaError_t conv_fwd_tc(const CUtensorMap &in_map, const __nv_bfloat16 *wf, cons
     per_sm = std::min(per_sm, regs_sm / (warp_regs * warps));
     per_sm = std::min(per_sm, warps_sm / 32 / warps);
     per_sm = std::max(per_sm, 1);
-    const long long tiles = (long long)n * H * ((W + kTcOut - 1) / kTcOut);
+    const long long tiles = ((long long)n * H * ((W + kTcSeg - 1) / kTcSeg) + 3) / 4;
     const int grid = (int)(tiles < (long long)per_sm * sms ? tiles : (long long)per_sm * sms);
     kern<<<grid, threads, smem, s>>>(in_map, wf, b, out, W, H, n, S, err, mask, db);
     return cudaGetLastError();
