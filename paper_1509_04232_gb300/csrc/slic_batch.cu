@@ -46,6 +46,9 @@ struct slic_batch_ctx {
     bool any_conv = false;            // some frame has a stopping threshold
     int total_tiles = 0, total_centres = 0, total_rows = 0, max_w = 0, win_max = 0;
     int total_tiles64 = 0, win_max64 = 0;  // the same for 32x64 tiles
+    // Passes with one row group per warp: frames whose S is a multiple of 16
+    // run over 16x16 blocks (k_assign_blocks), the others over tiles
+    int total_blocks = 0, total_rest = 0, block_occ = 0;
     int total_chunks = 0;    // update chunks of all frames (fused passes)
     bool fused = false;      // the passes before the last in one cooperative launch
     // Groups: the frames run as `groups` runs of consecutive frames (split
@@ -149,6 +152,16 @@ bool encode_maps(FrameArgs &a) {
     // 32x64 tiles: a box twice as high, and the taller window of centres
     const cuuint32_t fbox64[3] = {(cuuint32_t)kTileW, (cuuint32_t)(2 * kTileH), 3};
     const cuuint32_t cbox64[2] = {(cuuint32_t)a.box_w * kCtabRec, (cuuint32_t)a.box_h64};
+    // 16x16 blocks and the 3x3 records around a cell
+    const cuuint32_t fbox16[3] = {16, 16, 3};
+    const cuuint32_t cbox9[2] = {3 * kCtabRec, 3};
+    if (enc(&a.feat_map16, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.feat, fdim, fstride, fbox16, ones,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+        enc(&a.ctab_map9, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.ctab, cdim, cstride, cbox9, ones,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
     return enc(&a.feat_map64, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.feat, fdim, fstride, fbox64, ones,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
@@ -319,6 +332,8 @@ cudaError_t upload_tables(slic_batch_ctx *b, int k, cudaStream_t s) {
             a.row_base -= a0.row_base;
             a.strip_base -= a0.strip_base;
             a.chunk_base -= a0.chunk_base;
+            a.block_base -= a0.block_base;
+            a.rest_base -= a0.rest_base;
             gt[f] = a;
         }
     }
@@ -498,6 +513,21 @@ slic_status slic_batch_create(const slic_params *params, int n_frames, slic_batc
         a.cstate = reinterpret_cast<ConvState *>(b->scratch + off_cs[f]);
         if (b->pipe && !encode_maps(a)) b->pipe = false;  // then every pass uses k_assign_batch
     }
+    {
+        // Blocks or 32x32 tiles, per frame, with one row group: at other S a
+        // 16x16 block does not lie in one cell.
+        b->block_occ = b->pipe ? assign_blocks_occupancy() : 0;
+        for (FrameArgs &a : b->frames) {
+            a.block_base = b->total_blocks;
+            a.rest_base = b->total_rest;
+            if (b->block_occ > 0 && a.S % 16 == 0) {
+                a.blocks_x = (a.W + 15) / 16;
+                b->total_blocks += a.blocks_x * ((a.H + 15) / 16);
+            } else {
+                b->total_rest += a.n_tiles;
+            }
+        }
+    }
     b->d_err = reinterpret_cast<int *>(b->scratch + off_err);
     if (b->connectivity == 2) b->ccl = reinterpret_cast<int *>(b->scratch + off_ccl);
     if (cudaMemset(b->d_err, 0, sizeof(int)) != cudaSuccess) {
@@ -571,14 +601,14 @@ namespace {
 // (bases counted from its first frame) and its totals.
 struct Span {
     const FrameArgs *frames;
-    int n, tiles, tiles64, centres, rows, units, chunks;
+    int n, tiles, tiles64, centres, rows, units, chunks, blocks, rest;
 };
 
 // Group g of the batch (g < 0: the whole batch, with its own table).
 Span span_of(const slic_batch_ctx *b, int g) {
     if (g < 0)
         return Span{b->d_frames, b->n, b->total_tiles, b->total_tiles64, b->total_centres, b->total_rows,
-                    b->total_units, b->total_chunks};
+                    b->total_units, b->total_chunks, b->total_blocks, b->total_rest};
     const int f0 = b->group_first[g], f1 = b->group_first[g + 1];
     const FrameArgs &a = b->frames[f0];
     const bool end = f1 == b->n;
@@ -589,7 +619,9 @@ Span span_of(const slic_batch_ctx *b, int g) {
                 (end ? b->total_centres : z->centre_base) - a.centre_base,
                 (end ? b->total_rows : z->row_base) - a.row_base,
                 (end ? b->total_units : z->strip_base) - a.strip_base,
-                (end ? b->total_chunks : z->chunk_base) - a.chunk_base};
+                (end ? b->total_chunks : z->chunk_base) - a.chunk_base,
+                (end ? b->total_blocks : z->block_base) - a.block_base,
+                (end ? b->total_rest : z->rest_base) - a.rest_base};
 }
 
 // Every stage of a segmentation of the span's frames, enqueued on s: the
@@ -652,12 +684,21 @@ cudaError_t enqueue_span(slic_batch_ctx *b, const Span &sp, cudaStream_t s, bool
     const int tiles_th = b->tile_h == 64 ? sp.tiles64 : sp.tiles;
     const int win_th = b->tile_h == 64 ? b->win_max64 : b->win_max;
     auto last_or_pass = [&](int pass) {
-        return [&, pass]() {
-            return b->pipe ? launch_assign_pipe(sp.frames, sp.n, tiles_th, win_th, b->same, pass == b->iterations,
-                                                b->stages, b->rows, b->tile_h, pipe_per_sm, grid_pipe, b->d_err,
-                                                b->any_conv ? 1 : 0, s)
-                           : launch_assign_batch(sp.frames, sp.n, sp.tiles, b->win_max, b->same, pass == 0 && !warm,
-                                                 pass == b->iterations, b->smem, grid, s);
+        return [&, pass]() -> cudaError_t {
+            const bool last = pass == b->iterations;
+            if (!b->pipe)
+                return launch_assign_batch(sp.frames, sp.n, sp.tiles, b->win_max, b->same, pass == 0 && !warm, last,
+                                           b->smem, grid, s);
+            if (b->rows == 2)
+                return launch_assign_pipe(sp.frames, sp.n, tiles_th, win_th, b->same, last, b->stages, b->rows,
+                                          b->tile_h, pipe_per_sm, grid_pipe, b->d_err, b->any_conv ? 1 : 0, s);
+            if (sp.blocks > 0 && sp.rest > 0) ++n_launch;  // (two launches)
+            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, last, grid_for(b, b->block_occ), b->d_err,
+                                                 b->any_conv ? 1 : 0, s);
+            if (r == cudaSuccess)
+                r = launch_assign_pipe(sp.frames, sp.n, sp.rest, win_th, b->same, last, b->stages, b->rows, b->tile_h,
+                                       pipe_per_sm, grid_pipe, b->d_err, b->any_conv ? 1 : 0, s);
+            return r;
         };
     };
     if (e == cudaSuccess && b->pipe && b->fused && whole && b->iterations > 0) {

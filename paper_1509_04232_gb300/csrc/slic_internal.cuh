@@ -116,6 +116,8 @@ struct FrameArgs {
     CUtensorMap ctab_map;   // padded centre table as [(ns_r+2)][(ns_c+2)*kCtabRec] f32, box box_w*kCtabRec x box_h
     CUtensorMap feat_map64; // the same for 32x64 tiles: box 32x64x3, and
     CUtensorMap ctab_map64; // box box_w*kCtabRec x box_h64
+    CUtensorMap feat_map16; // for 16x16 blocks: box 16x16x3, and the
+    CUtensorMap ctab_map9;  // 3x3 records around a cell
     ConvConsts conv;
     const uint8_t *rgb;     // [H][W][C]
     float *feat;            // 3 planes [H][P]; plane stride H*P
@@ -154,6 +156,11 @@ struct FrameArgs {
     // batch's list of chunks
     int n_tiles, n_tiles64, n_chunks;
     int chunk_base;
+    // Split of a pass with one row group per warp (see k_assign_blocks): 16x16
+    // blocks of the frame per row and its first one in the batch's list (frames
+    // whose S is a multiple of 16), and its first 32x32 tile in the list of the
+    // other frames' tiles. A frame has no entry in the list it is not in.
+    int blocks_x, block_base, rest_base;
 };
 constexpr int kUpdateChunk = 256;  // centres per update work item of the fused assignment
 
@@ -219,7 +226,13 @@ cudaError_t launch_update_batch(const FrameArgs *d_frames, int n, int total_cent
 cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles, int win_max, bool same, bool last,
                                int nst, int rows, int tile_h, int ctas_per_sm, int grid, int *err, int check_stop,
                                cudaStream_t s);
-// Fused multi-pass form of the same kernel, one cooperative launch: passes
+// The same pass over 16x16 blocks, a warp per block, for the frames whose S is
+// a multiple of 16 (total_blocks of them in all); launch_assign_pipe then
+// takes the tiles of the rest. Resident CTAs per SM of its kernels.
+cudaError_t launch_assign_blocks(const FrameArgs *d_frames, int n, int total_blocks, bool last, int grid, int *err,
+                                 int check_stop, cudaStream_t s);
+int assign_blocks_occupancy();
+// Fused multi-pass form of the tile kernel, one cooperative launch: passes
 // 0 .. passes-1 with the update after each (updates 1 .. passes), ordered
 // per frame by the phase counters in its ConvState (reset by the
 // initialisation); the last pass is a separate launch_assign_pipe. Each CTA

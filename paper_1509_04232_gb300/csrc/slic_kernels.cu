@@ -43,7 +43,9 @@ __device__ __forceinline__ int div_s(int x, unsigned s_mul, int S) {
 
 // Index of the frame whose [base, next base) range holds `idx` (frames are
 // sorted by base; base of frame 0 is 0).
-enum BaseField { kTileBase, kCentreBase, kRowBase, kStripBase, kTileBase64, kChunkBase };
+enum BaseField {
+    kTileBase, kCentreBase, kRowBase, kStripBase, kTileBase64, kChunkBase, kBlockBase, kRestBase
+};
 template <BaseField F>
 __device__ __forceinline__ int base_of(const FrameArgs &a) {
     return F == kTileBase ? a.tile_base
@@ -51,6 +53,8 @@ __device__ __forceinline__ int base_of(const FrameArgs &a) {
            : F == kRowBase ? a.row_base
            : F == kStripBase ? a.strip_base
            : F == kTileBase64 ? a.tile_base64
+           : F == kBlockBase ? a.block_base
+           : F == kRestBase ? a.rest_base
                               : a.chunk_base;
 }
 template <BaseField F>
@@ -1143,9 +1147,11 @@ __device__ __forceinline__ void assign_pipe_body(const FrameArgs *frames, int n_
             if (use > 0 && !mbar_wait(&empty[q], (use - 1) & 1)) return false;
             // A producer thread's tiles come in increasing order: its frame
             // index only moves forward.
-            while (pf + 1 < n_frames && base_of<TH == 64 ? kTileBase64 : kTileBase>(frames[pf + 1]) <= t) ++pf;
+            // (one row group: only the frames that k_assign_blocks leaves)
+            constexpr BaseField kBase = TH == 64 ? kTileBase64 : ROWS == 2 ? kTileBase : kRestBase;
+            while (pf + 1 < n_frames && base_of<kBase>(frames[pf + 1]) <= t) ++pf;
             const int f = pf;
-            TileGeom g = tile_geom<TH>(frames[f], t - base_of<TH == 64 ? kTileBase64 : kTileBase>(frames[f]));
+            TileGeom g = tile_geom<TH>(frames[f], t - base_of<kBase>(frames[f]));
             g.f = f;
             g.skip = !LAST && check_stop && frame_stopped(frames[f]) ? 1 : 0;
             if (g.skip) g.H = 0;  // no pixel of the tile is evaluated or summed
@@ -1605,6 +1611,7 @@ static cudaError_t launch_pipe_as(const FrameArgs *d_frames, int n, int total_ti
 cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles, int win_max, bool same, bool last,
                                int nst, int rows, int tile_h, int ctas_per_sm, int grid, int *err, int check_stop,
                                cudaStream_t s) {
+    if (total_tiles < 1) return cudaSuccess;
     if (grid > total_tiles) grid = total_tiles;
     if (grid < 1) grid = 1;
     if (nst < 3) nst = 3;
@@ -1633,6 +1640,350 @@ cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles
                     : launch_pipe_as<true, false, 3, 1>(d_frames, n, total_tiles, win_max, nst, grid, smem, err, check_stop, s);
     return wide ? launch_pipe_as<false, false, 4, 1>(d_frames, n, total_tiles, win_max, nst, grid, smem, err, check_stop, s)
                 : launch_pipe_as<false, false, 3, 1>(d_frames, n, total_tiles, win_max, nst, grid, smem, err, check_stop, s);
+}
+
+// ---------------------------------------------------------------------------
+// One pass over 16x16 blocks, a warp per block (frames whose S is a multiple
+// of 16: a block lies in one cell)
+// ---------------------------------------------------------------------------
+//
+// The tile kernel above shares a tile between the warps of a CTA: headers,
+// stage reuse, two sets of private sums and their flush are handed between
+// warps, which took 57 of its 141 instructions per pixel, and its warps span
+// two cells, so that every pixel's sums go through shared atomics. Here each
+// warp works alone on a run of neighbouring blocks: lane 0 copies the next
+// block's features (16x16x3) and its nine centre records into the warp's own
+// two stages, one mbarrier each, and no warp waits for another.
+//
+// All lanes share the nine candidates (broadcast loads at fixed offsets). Lane
+// l holds the pixel pairs at columns 2 * (l % 8) of rows l / 8 + 4 i: its loads
+// are 256 contiguous bytes per warp. Pixels that stay with their own cell, the
+// most frequent winner, add up in registers and across the warp; the others go
+// to the warp's bins in shared memory (see FrameBins). Running 64-bit totals
+// of the nine cells stay in the lanes' registers while the run moves along a
+// row, shifted by one cell at a time: only the three cells left behind go to
+// global memory, so a block costs 18 atomic lanes, not 54.
+namespace {
+constexpr int kBlk = 16;
+constexpr int kBlkThreads = 256, kBlkWarps = kBlkThreads / 32;
+constexpr int kBlkStages = 2;
+constexpr int kBlkFeat = 3 * kBlk * kBlk * 4;   // bytes of a stage's features
+constexpr int kBlkCen = 9 * kCtabRec * 4;       // and of its centre records
+constexpr int kBlkStage = (kBlkFeat + kBlkCen + 127) & ~127;
+constexpr int kBlkBinWords = 160;               // word q of candidate t, copy c: q * 40 + t * 4 + c
+
+// A block: frame, cell, first pixel, extent inside the image, cell column.
+struct __align__(16) BlockHdr {
+    int f, k, x0, y0;
+    int wl, hl, cx, cy;
+};
+
+// What a warp keeps in shared memory rather than in registers (the candidate
+// loop needs those): the frame its blocks come from, and the lanes' totals.
+struct __align__(16) BlockState {
+    int f, W, ns_c, vec;
+    float fs, w;
+    int32_t *out;
+    unsigned long long *acc;
+    int k, cx, y0, have;  // the block the totals belong to (have: there is one)
+    longlong2 total[27];
+};
+constexpr int kBlkHdrs = 64;  // of a warp: two runs of 32, made by its lanes together
+
+constexpr size_t blocks_smem_bytes() {
+    return (size_t)kBlkWarps * (kBlkStages * (kBlkStage + 8) + kBlkHdrs * sizeof(BlockHdr) + sizeof(BlockState) + 2 * kBlkBinWords * 4) + 128;
+}
+}  // namespace
+
+template <bool LAST>
+__global__ void __launch_bounds__(kBlkThreads, 2)
+    k_assign_blocks(const FrameArgs *frames, int n_frames, int total_blocks, int *err, int check_stop) {
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    unsigned char *const smem =
+        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~(uintptr_t)127);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *const stages = smem + (size_t)warp * kBlkStages * kBlkStage;
+    unsigned *const bins =
+        reinterpret_cast<unsigned *>(smem + (size_t)kBlkWarps * kBlkStages * kBlkStage) + warp * 2 * kBlkBinWords;
+    BlockHdr *const hdr = reinterpret_cast<BlockHdr *>(bins + (kBlkWarps - warp) * 2 * kBlkBinWords) + warp * kBlkHdrs;
+    BlockState *const me = reinterpret_cast<BlockState *>(hdr + (kBlkWarps - warp) * kBlkHdrs) + warp;
+    uint64_t *const full = reinterpret_cast<uint64_t *>(me + kBlkWarps - warp) + warp * kBlkStages;
+
+    // This warp's run of the batch's blocks.
+    const long long nw = (long long)gridDim.x * kBlkWarps, iw = (long long)blockIdx.x * kBlkWarps + warp;
+    const int b0 = (int)(total_blocks * iw / nw), n_blk = (int)(total_blocks * (iw + 1) / nw) - b0;
+    if (lane == 0) {
+        for (int q = 0; q < kBlkStages; ++q) mbar_init(&full[q], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int i = lane; i < 2 * kBlkBinWords; i += 32) bins[i] = 0u;
+    // Headers of blocks j0 .. j0 + 31 of the run, one per lane.
+    auto make_headers = [&](int j0) {
+        BlockHdr h;
+        h.f = -1;
+        if (j0 + lane < n_blk) {
+            const int b = b0 + j0 + lane;
+            h.f = find_frame<kBlockBase>(frames, n_frames, b);
+            const FrameArgs &a = frames[h.f];
+            const int local = b - a.block_base, by = local / a.blocks_x;
+            h.x0 = (local - by * a.blocks_x) * kBlk;
+            h.y0 = by * kBlk;
+            h.cx = div_s(h.x0, a.s_mul, a.S);
+            h.cy = div_s(h.y0, a.s_mul, a.S);
+            h.k = h.cy * a.ns_c + h.cx;
+            h.wl = min(kBlk, a.W - h.x0);
+            h.hl = min(kBlk, a.H - h.y0);
+            if (!LAST && check_stop && frame_stopped(a)) h.wl = 0;  // nothing to sum, no copy
+        }
+        hdr[(j0 + lane) % kBlkHdrs] = h;
+    };
+    make_headers(0);
+    if (lane == 0) {
+        me->f = -1;
+        me->have = 0;
+    }
+    __syncwarp();
+    // One lane: copy block j into stage j % kBlkStages.
+    auto produce = [&](int j) {
+        const BlockHdr &h = hdr[j % kBlkHdrs];
+        uint64_t *const bar = &full[j % kBlkStages];
+        if (h.wl == 0) {
+            mbar_arrive(bar);
+            return;
+        }
+        const FrameArgs &a = frames[h.f];
+        unsigned char *const st = stages + (size_t)(j % kBlkStages) * kBlkStage;
+        mbar_expect_tx(bar, kBlkFeat + kBlkCen);
+        tma_load_3d(st, &a.feat_map16, h.x0, h.y0, 0, bar);
+        tma_load_2d(st + kBlkFeat, &a.ctab_map9, h.cx * kCtabRec, h.cy, bar);
+    };
+    // (fault injection: copies are not to be issued)
+    const bool no_copies = *reinterpret_cast<volatile int *>(&g_abort_copies) != 0;
+    bool ok = true;
+    if (lane == 0 && !no_copies)
+        for (int j = 0; j < kBlkStages && j < n_blk; ++j) produce(j);
+
+    const int row = lane >> 3, col = 2 * (lane & 7);
+    // Running totals: lane 3 * t + part (t < 9) keeps two of the six sums of the
+    // cell at candidate t's place around the last block's cell.
+    const int part = lane - lane / 3 * 3, rt = lane / 3;
+    auto flush = [&](int k) {  // the lane's totals, around cell k, to the global sums
+        const longlong2 r = me->total[lane];
+        if ((r.x | r.y) != 0) {
+            unsigned long long *g = me->acc + (size_t)(k + (rt / 3 - 1) * me->ns_c + rt % 3 - 1) * 6 + 2 * part;
+            atomicAdd(g, (unsigned long long)r.x);
+            atomicAdd(g + 1, (unsigned long long)r.y);
+        }
+    };
+
+    int j = 0, par = 0;  // par: the bins' set
+    for (; j < n_blk; ++j) {
+        const int q = j % kBlkStages;
+        if (!__all_sync(kFull, mbar_wait(&full[q], (j / kBlkStages) & 1))) {
+            ok = false;
+            break;
+        }
+        const BlockHdr h = hdr[j % kBlkHdrs];
+        if (j % 32 == 0) make_headers(j + 32);  // (their slots held blocks j - 32 ..; the next __syncwarp is before their use)
+        if (h.wl == 0) {  // a stopped frame's block
+            __syncwarp();
+            if (lane == 0 && j + kBlkStages < n_blk && !no_copies) produce(j + kBlkStages);
+            continue;
+        }
+        if (h.f != me->f) {  // (all lanes read it before lane 0 writes)
+            if (!LAST && me->have && lane < 27) flush(me->k);
+            __syncwarp();
+            if (lane == 0) {
+                me->have = 0;
+                const FrameArgs &a = frames[h.f];
+                me->f = h.f;
+                me->W = a.W;
+                me->ns_c = a.ns_c;
+                me->vec = a.assign_vec;
+                me->fs = a.fix_scale;
+                me->w = a.w;
+                me->out = a.assign_out;
+                me->acc = reinterpret_cast<unsigned long long *>(a.acc);
+            }
+            if (!LAST && lane < 27) me->total[lane] = make_longlong2(0, 0);
+            __syncwarp();
+        }
+        const float w = me->w;
+        const unsigned long long ww = pack2(w, w);
+        const unsigned char *const st = stages + (size_t)q * kBlkStage;
+        const float *const feat = reinterpret_cast<const float *>(st);
+        const float *const cen = reinterpret_cast<const float *>(st + kBlkFeat);
+        unsigned long long l[4], a[4], b[4], fy[4];
+        const float fx = (float)(h.x0 + col);
+        const unsigned long long x = pack2(fx, fx + 1.0f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float *const p = feat + (row + 4 * i) * kBlk + col;
+            l[i] = *reinterpret_cast<const unsigned long long *>(p);
+            a[i] = *reinterpret_cast<const unsigned long long *>(p + kBlk * kBlk);
+            b[i] = *reinterpret_cast<const unsigned long long *>(p + 2 * kBlk * kBlk);
+            const float y = (float)(h.y0 + row + 4 * i);
+            fy[i] = pack2(y, y);
+        }
+        // Eq. (1), with the operations of the tile kernel
+        float bk[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) bk[i][0] = bk[i][1] = __int_as_float(0x7F800000);
+#pragma unroll
+        for (int t0 = 0; t0 < 9; t0 += 2) {
+            const int nt = t0 < 8 ? 2 : 1;
+            float kk[2][4][2];
+#pragma unroll
+            for (int u = 0; u < nt; ++u) {
+                const float *rp = cen + (t0 + u) * kCtabRec;
+                const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(rp);
+                const ulonglong2 bx = *reinterpret_cast<const ulonglong2 *>(rp + 4);
+                const unsigned long long yy = *reinterpret_cast<const unsigned long long *>(rp + 8);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const unsigned long long ddy = sub2(yy, fy[i]);
+                    eval_keys(la, bx, mul2(ddy, ddy), ww, l[i], a[i], b[i], x, c_tags[t0 + u], kk[u][i][0],
+                              kk[u][i][1]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int v = 0; v < 2; ++v)
+                    bk[i][v] = nt == 2 ? fmin3_nan(bk[i][v], kk[0][i][v], kk[1][i][v]) : fmin_nan(bk[i][v], kk[0][i][v]);
+        }
+        // Every read of the stage is done: the next block goes there.
+        __syncwarp();
+        if (lane == 0 && j + kBlkStages < n_blk && !no_copies) produce(j + kBlkStages);
+        int t[4][2];  // winning candidate, -1 outside the image
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+                t[i][v] = row + 4 * i < h.hl && col + v < h.wl ? (int)(__float_as_uint(bk[i][v]) & 15u) : -1;
+        if constexpr (LAST) {
+            const int W = me->W, ns_c = me->ns_c, vec = me->vec;
+            int32_t *const out = me->out;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                int32_t *const o = out + (size_t)(h.y0 + row + 4 * i) * W + h.x0 + col;
+                int lab[2];
+#pragma unroll
+                for (int v = 0; v < 2; ++v)
+                    lab[v] = h.k - ns_c - 1 + t[i][v] + (int)__umulhi((unsigned)t[i][v], 0x55555556u) * (ns_c - 3);
+                if (vec && t[i][1] >= 0) {
+                    *reinterpret_cast<int2 *>(o) = make_int2(lab[0], lab[1]);
+                } else {
+                    if (t[i][0] >= 0) o[0] = lab[0];
+                    if (t[i][1] >= 0) o[1] = lab[1];
+                }
+            }
+        } else {
+            const float fs = me->fs;
+            unsigned own[4] = {0u, 0u, 0u, 0u};
+            unsigned *const set = bins + par * kBlkBinWords;
+            par ^= 1;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                unsigned v[2][4];
+                float f0, f1;
+                unpack2(l[i], f0, f1);
+                fix_round2_biased(f0, f1, fs, v[0][0], v[1][0]);
+                unpack2(a[i], f0, f1);
+                fix_round2_biased(f0, f1, fs, v[0][1], v[1][1]);
+                unpack2(b[i], f0, f1);
+                fix_round2_biased(f0, f1, fs, v[0][2], v[1][2]);
+                // x and y from the block's corner and the count: 11 + 11 + 10
+                // bits, enough for its 256 pixels
+                v[0][3] = (unsigned)col + ((unsigned)(row + 4 * i) << 11) + (1u << 22);
+                v[1][3] = v[0][3] + 1u;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (t[i][u] == 4) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) own[c] += v[u][c];
+                    } else if (t[i][u] >= 0) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) atomicAdd(&set[c * 40 + t[i][u] * 4 + (lane & 3)], v[u][c]);
+                    }
+                }
+            }
+            {
+                // the other set, read for the last block, is cleared for the next
+                uint4 *const z = reinterpret_cast<uint4 *>(bins + par * kBlkBinWords);
+                z[lane] = make_uint4(0u, 0u, 0u, 0u);
+                if (lane < 8) z[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) own[c] = __reduce_add_sync(kFull, own[c]);
+            __syncwarp();
+            if (lane < 27) {
+                // The totals follow the block: one cell to the right, the left
+                // column is complete; anything else but the same cell, all nine.
+                const bool row_same = h.y0 == me->y0, right = row_same && h.cx == me->cx + 1,
+                           same = !me->have || (row_same && h.cx == me->cx);
+                longlong2 r = me->total[lane];
+                if (!same) {
+                    if (!right || rt % 3 == 0) flush(me->k);
+                    r = right && rt % 3 < 2 ? me->total[lane + 3] : make_longlong2(0, 0);
+                }
+                auto word = [&](int c) {  // the four copies' sum (own: the warp's)
+                    if (rt == 4) return c == 0 ? own[0] : c == 1 ? own[1] : c == 2 ? own[2] : own[3];
+                    const uint4 v = *reinterpret_cast<const uint4 *>(set + c * 40 + rt * 4);
+                    return v.x + v.y + v.z + v.w;
+                };
+                const unsigned xyn = word(3), cnt = xyn >> 22, bias = cnt * kFixBias;
+                if (part == 0) {
+                    r.x += (int)(word(0) - bias);
+                    r.y += (int)(word(1) - bias);
+                } else if (part == 1) {
+                    r.x += (int)(word(2) - bias);
+                    r.y += (long long)(xyn & 0x7FFu) + (long long)cnt * h.x0;
+                } else {
+                    r.x += (long long)((xyn >> 11) & 0x7FFu) + (long long)cnt * h.y0;
+                    r.y += (long long)cnt;
+                }
+                __syncwarp(0x7FFFFFFu);  // (totals read before they are replaced)
+                me->total[lane] = r;
+                if (lane == 0) {
+                    me->k = h.k;
+                    me->cx = h.cx;
+                    me->y0 = h.y0;
+                    me->have = 1;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (!LAST && ok && me->have && lane < 27) flush(me->k);
+    if (lane == 0 && !ok) atomicOr(err, 1);
+    // After a wait that timed out: the copies still in flight land (bounded)
+    // before the CTA exits, so none targets freed shared memory.
+    if (lane == 0 && !ok && !no_copies)
+        for (int q = j; q < min(n_blk, j + kBlkStages); ++q) mbar_wait(&full[q % kBlkStages], (q / kBlkStages) & 1);
+}
+
+int assign_blocks_occupancy() {
+    int o[2] = {0, 0};
+    const int smem = (int)blocks_smem_bytes();
+    if (cudaFuncSetAttribute(k_assign_blocks<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaFuncSetAttribute(k_assign_blocks<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[0], k_assign_blocks<false>, kBlkThreads, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[1], k_assign_blocks<true>, kBlkThreads, smem) != cudaSuccess)
+        return 0;
+    return std::min(o[0], o[1]);
+}
+
+cudaError_t launch_assign_blocks(const FrameArgs *d_frames, int n, int total_blocks, bool last, int grid, int *err,
+                                 int check_stop, cudaStream_t s) {
+    if (total_blocks < 1) return cudaSuccess;
+    grid = std::max(1, std::min(grid, (total_blocks + kBlkWarps - 1) / kBlkWarps));
+    auto kern = last ? k_assign_blocks<true> : k_assign_blocks<false>;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)blocks_smem_bytes());
+    if (e != cudaSuccess) return e;
+    kern<<<grid, kBlkThreads, blocks_smem_bytes(), s>>>(d_frames, n, total_blocks, err, check_stop);
+    return cudaGetLastError();
 }
 
 // Cooperative launch (every CTA resident at once: the fused kernel's CTAs
