@@ -79,74 +79,109 @@ __device__ __forceinline__ float sqrt_fast(float v) {
 // 9 slots of the pixel's cell window the Eq. (1) distance D/100 to the
 // grid-initialised centre of that cell (2.0 off the grid), zero padding.
 // ---------------------------------------------------------------------------
+//
+// A block covers 128 columns of kPrepRows rows. The grid centres its pixels
+// see are converted once into shared memory; a thread walks down its column
+// and keeps its nine centres in registers while the rows stay in one cell row.
+// (One row per block, centres read back for every pixel: 125 us for four
+// 1920x1080 images, bound by the blocks' start-up latency and the shared
+// loads.)
+constexpr int kPrepRows = 8;
+__host__ __device__ constexpr int prep_cols(int S) { return 127 / S + 4; }            // cell columns a block sees
+__host__ __device__ constexpr int prep_rows(int S) { return (kPrepRows - 1) / S + 4; }  // and cell rows
+
 __global__ void __launch_bounds__(128) k_net_prep(ConvConsts cc, const uint8_t *rgb, const uint8_t *const *table,
                                                   int W, int H, int C, int S, float w, __nv_bfloat16 *x0) {
-    // A block covers 128 pixels of one row; the grid centres of the cells its
-    // pixels see (three cell rows, the covered cell columns +- 1) are
-    // converted once into shared memory instead of once per pixel and slot.
-    constexpr int kMaxCols = 128 + 3;
-    __shared__ float4 cen_lab[3][kMaxCols];  // L, a, b, x of a grid centre
-    __shared__ float cen_y[3][kMaxCols];     // y (< 0: off the grid)
-    const int x0p = blockIdx.x * blockDim.x, y = blockIdx.y, b = blockIdx.z;
+    extern __shared__ __align__(16) unsigned char prep_smem[];
+    __shared__ float lut[256];
+    const int cols_max = prep_cols(S);
+    float4 *const cen_lab = reinterpret_cast<float4 *>(prep_smem);  // L, a, b, x of a grid centre
+    float *const cen_y = reinterpret_cast<float *>(cen_lab + prep_rows(S) * cols_max);  // y (< 0: off the grid)
+    const int x0p = blockIdx.x * 128, y0 = blockIdx.y * kPrepRows, b = blockIdx.z;
     const size_t img = (size_t)b * H * W;
     // image b: entry b of the pointer table, else the b-th of a contiguous stack
     const uint8_t *const src = table ? table[b] : rgb + img * C;
     const int ns_c = (W + S - 1) / S, ns_r = (H + S - 1) / S;
-    const int cy = y / S, cx_lo = x0p / S - 1;
-    const int cx_hi = min(x0p + (int)blockDim.x - 1, W - 1) / S + 1;
-    const int ncols = cx_hi - cx_lo + 1;
-    for (int i = threadIdx.x; i < 3 * ncols; i += blockDim.x) {
+    const int x = x0p + threadIdx.x, y_end = min(y0 + kPrepRows, H);
+    uint8_t px[kPrepRows][3];  // this thread's pixels, in flight during the set-up
+#pragma unroll
+    for (int r = 0; r < kPrepRows; ++r) {
+        const bool in = x < W && y0 + r < y_end;
+        const uint8_t *p = src + ((size_t)(y0 + r) * W + x) * C;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) px[r][c] = in ? __ldg(p + c) : (uint8_t)0;
+    }
+    for (int i = threadIdx.x; i < 256; i += 128) lut[i] = g_lut_net[i];
+    __syncthreads();
+    const int cy_lo = y0 / S - 1, cy_hi = (y_end - 1) / S + 1, cx_lo = x0p / S - 1;
+    const int ncols = min(x0p + 127, W - 1) / S + 1 - cx_lo + 1;
+    for (int i = threadIdx.x; i < (cy_hi - cy_lo + 1) * ncols; i += 128) {
         const int r = i / ncols, c = i - r * ncols;
-        const int nx = cx_lo + c, ny = cy + r - 1;
+        const int nx = cx_lo + c, ny = cy_lo + r, e = r * cols_max + c;
         if (nx >= 0 && nx < ns_c && ny >= 0 && ny < ns_r) {
             // grid initialisation of Sec. 3: midpoint of the in-image cell, colour under it
             const int xf = nx * S, xl = min((nx + 1) * S, W) - 1, yf = ny * S, yl = min((ny + 1) * S, H) - 1;
             const uint8_t *q = src + ((size_t)((yf + yl) >> 1) * W + ((xf + xl) >> 1)) * C;
             float l, a2, b2;
-            convert_pixel(cc, q[0], q[1], q[2], g_lut_net, l, a2, b2);
-            cen_lab[r][c] = make_float4(l, a2, b2, 0.5f * (float)(xf + xl));
-            cen_y[r][c] = 0.5f * (float)(yf + yl);
+            convert_pixel(cc, q[0], q[1], q[2], lut, l, a2, b2);
+            cen_lab[e] = make_float4(l, a2, b2, 0.5f * (float)(xf + xl));
+            cen_y[e] = 0.5f * (float)(yf + yl);
         } else {
-            cen_lab[r][c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            cen_y[r][c] = -1.0f;
+            cen_lab[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            cen_y[e] = -1.0f;
         }
     }
     __syncthreads();
-    const int x = x0p + threadIdx.x;
     if (x >= W) return;
-    const size_t px = img + (size_t)y * W + x;
-    const uint8_t *p = src + ((size_t)y * W + x) * C;
-    float f0, f1, f2;
-    convert_pixel(cc, p[0], p[1], p[2], g_lut_net, f0, f1, f2);
     const int cx = x / S;
-    const float inv_s = 1.0f / (float)S;
-    float ch[16];
-    ch[0] = f0 * 0.01f;
-    ch[1] = f1 * (1.0f / 128.0f);
-    ch[2] = f2 * (1.0f / 128.0f);
-    ch[3] = (float)(x - cx * S) * inv_s;
-    ch[4] = (float)(y - cy * S) * inv_s;
-    const float fx = (float)x, fy = (float)y;
+    const float inv_s = 1.0f / (float)S, fx = (float)x, chx = (float)(x - cx * S) * inv_s;
+    int cy = y0 / S, y_next = y0;  // the cell row, and the row where its centres are loaded
+    float el[9], ea[9], eb[9], dx[9], ey[9];
 #pragma unroll
-    for (int t = 0; t < 9; ++t) {
-        const int col = cx + t % 3 - 1 - cx_lo;
-        const float4 e = cen_lab[t / 3][col];
-        const float ey = cen_y[t / 3][col];
-        float d = 2.0f;
-        if (ey >= 0.0f) {
-            const float dl = e.x - f0, da = e.y - f1, db = e.z - f2;
-            const float dx = e.w - fx, dy = ey - fy;
-            d = (sqrt_fast(fmaf(dl, dl, fmaf(da, da, db * db))) + w * sqrt_fast(fmaf(dx, dx, dy * dy))) * 0.01f;
+    for (int r = 0; r < kPrepRows; ++r) {
+        const int y = y0 + r;
+        if (y >= y_end) break;
+        if (y == y_next) {
+            cy = y / S;
+            y_next = (cy + 1) * S;
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const int e = (cy + t / 3 - 1 - cy_lo) * cols_max + cx + t % 3 - 1 - cx_lo;
+                const float4 v = cen_lab[e];
+                el[t] = v.x;
+                ea[t] = v.y;
+                eb[t] = v.z;
+                dx[t] = v.w - fx;
+                ey[t] = cen_y[e];
+            }
         }
-        ch[5 + t] = d;
-    }
-    ch[14] = ch[15] = 0.0f;
-    uint32_t out[8];
+        float f0, f1, f2;
+        convert_pixel(cc, px[r][0], px[r][1], px[r][2], lut, f0, f1, f2);
+        float ch[16];
+        ch[0] = f0 * 0.01f;
+        ch[1] = f1 * (1.0f / 128.0f);
+        ch[2] = f2 * (1.0f / 128.0f);
+        ch[3] = chx;
+        ch[4] = (float)(y - cy * S) * inv_s;
+        const float fy = (float)y;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) out[i] = pack_bf16(ch[2 * i], ch[2 * i + 1]);
-    uint4 *dst = reinterpret_cast<uint4 *>(x0 + px * 16);
-    dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-    dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        for (int t = 0; t < 9; ++t) {
+            float d = 2.0f;
+            if (ey[t] >= 0.0f) {
+                const float dl = el[t] - f0, da = ea[t] - f1, db = eb[t] - f2;
+                const float dy = ey[t] - fy;
+                d = (sqrt_fast(fmaf(dl, dl, fmaf(da, da, db * db))) + w * sqrt_fast(fmaf(dx[t], dx[t], dy * dy))) * 0.01f;
+            }
+            ch[5 + t] = d;
+        }
+        ch[14] = ch[15] = 0.0f;
+        uint32_t out[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) out[i] = pack_bf16(ch[2 * i], ch[2 * i + 1]);
+        uint4 *dst = reinterpret_cast<uint4 *>(x0 + (img + (size_t)y * W + x) * 16);
+        dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
+        dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -416,54 +451,44 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
     };
 
     if (warp == PRODUCER) {
-        // ---- producer: 12 tensor-map copies (4 quarters x 3 rows) per stage ----
-        if (lane == 0) {
-            int s = 0;
-            unsigned u = 0;       // completed rounds of the ring
-            unsigned issued = 0;  // bit s: a copy was issued into stage s
-            unsigned lastpar = 0; // bit s: parity of that copy's completion
-            Stepper w(4 * blockIdx.x, 4 * G, segs_x, (unsigned)H);
-            for (unsigned t = blockIdx.x; t < total; t += G, w.advance()) {
-                if (u > 0 && !tc_wait_ab(&empty[s], (u - 1) & 1u, abort)) {
-                    fail();
-                    break;
-                }
-                const unsigned b = tc_smem(&full[s]);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(BOX) : "memory");
-                const unsigned dst0 = tc_smem(in_s + s * BOX);
-                int sx = (int)w.a, y = (int)w.b, img = (int)w.c;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    // (past the last segment: the rows of an image outside the
-                    // batch, or zeros; their results are not stored)
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) {
-                        asm volatile(
-                            "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
-                            "{%2, %3, %4, %5}], [%6];" ::"r"(dst0 + (unsigned)((dy * kTcIn + 32 * q) * ROWB)),
-                            "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(0), "r"(sx * kTcSeg - 1), "r"(y + dy - 1),
-                            "r"(img), "r"(b)
-                            : "memory");
-                    }
-                    if (++sx == (int)segs_x) {
-                        sx = 0;
-                        if (++y == H) {
-                            y = 0;
-                            ++img;
-                        }
-                    }
-                }
-                issued |= 1u << s;
-                lastpar = (lastpar & ~(1u << s)) | ((u & 1u) << s);
-                if (++s == NS) {
-                    s = 0;
-                    ++u;
-                }
+        // ---- producer: 12 tensor-map copies (4 quarters x 3 rows) per stage,
+        // one per lane: issued one after another by one lane they kept the
+        // kernel waiting ----
+        const int q = lane & 3, dy = lane >> 2;  // lanes 0 .. 11
+        Stepper w(4 * blockIdx.x + q, 4 * G, segs_x, (unsigned)H);
+        int s = 0;
+        unsigned u = 0;       // completed rounds of the ring
+        unsigned issued = 0;  // bit s: a copy was issued into stage s
+        unsigned lastpar = 0; // bit s: parity of that copy's completion
+        for (unsigned t = blockIdx.x; t < total; t += G, w.advance()) {
+            if (u > 0 && !__all_sync(0xffffffffu, tc_wait_ab(&empty[s], (u - 1) & 1u, abort))) {
+                if (lane == 0) fail();
+                break;
             }
-            // every copy lands before the shared memory is released
+            const unsigned b = tc_smem(&full[s]);
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(BOX) : "memory");
+            __syncwarp();
+            // (past the last segment: rows of an image outside the batch, or
+            // zeros; their results are not stored)
+            if (lane < 12)
+                asm volatile(
+                    "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
+                    "{%2, %3, %4, %5}], [%6];" ::"r"(tc_smem(in_s + s * BOX) + (unsigned)((dy * kTcIn + 32 * q) * ROWB)),
+                    "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(0), "r"((int)w.a * kTcSeg - 1), "r"((int)w.b + dy - 1),
+                    "r"((int)w.c), "r"(b)
+                    : "memory");
+            issued |= 1u << s;
+            lastpar = (lastpar & ~(1u << s)) | ((u & 1u) << s);
+            if (++s == NS) {
+                s = 0;
+                ++u;
+            }
+        }
+        // every copy lands before the shared memory is released
+        if (lane == 0)
             for (int k = 0; k < NS; ++k)
                 if (issued & (1u << k)) tc_wait(&full[k], (lastpar >> k) & 1u);
-        }
     } else if (warp == ISSUER) {
         // ---- MMA issuer ----
         if (lane == 0) {
@@ -605,13 +630,13 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                 }
                 __syncwarp();
             } else {
-                const int x = xw + lane;
-                if (lane < n_out) {
-                    const size_t px = row0 + x;
-                    if constexpr (LABELS) {
+                static_assert(!RELU, "logits have no activation");
+                if constexpr (LABELS) {
+                    if (lane < n_out) {
                         // argmax of the valid slots' logits (first maximum in
                         // slot order), as the stand-alone label kernel on
                         // stored logits
+                        const int x = xw + lane;
                         const int cx = x / S, cy = y / S, ns_c = (W + S - 1) / S, ns_r = (H + S - 1) / S;
                         float mx = -INFINITY;
                         int arg = 4;
@@ -622,17 +647,15 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
                                 arg = q;
                             }
                         }
-                        static_cast<int32_t *>(out)[px] = (cy + arg / 3 - 1) * ns_c + cx + arg % 3 - 1;
-                    } else {
-                        float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(out) + px * COUT + c0);
+                        static_cast<int32_t *>(out)[row0 + x] = (cy + arg / 3 - 1) * ns_c + cx + arg % 3 - 1;
+                    }
+                } else {
+                    // (through shared memory, whole pixels per store instruction:
+                    // 304 us against 206 for four 1920x1080 images)
+                    if (lane < n_out) {
+                        float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(out) + (row0 + xw + lane) * COUT + c0);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            float4 f = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                            if (RELU) {
-                                f.x = fmaxf(f.x, 0.0f); f.y = fmaxf(f.y, 0.0f); f.z = fmaxf(f.z, 0.0f); f.w = fmaxf(f.w, 0.0f);
-                            }
-                            o[q] = f;
-                        }
+                        for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                     }
                 }
             }
@@ -1133,8 +1156,10 @@ cudaError_t conv_fwd(const slic_net_ctx *nc, int l, const __nv_bfloat16 *wf, con
     const CUtensorMap &m = nc->in_map[l];
     if (l == 0) return conv_fwd_tc<16, 32, true, false, false, 4>(m, wf, b, out, W, H, n, nc->S, nc->tc_err, nc->sms, s);
     if (l < 3) return conv_fwd_tc<32, 32, true, false, false, 3>(m, wf, b, out, W, H, n, nc->S, nc->tc_err, nc->sms, s);
+    // (labels: two stages, three CTAs per SM, 164 us for four 1920x1080 images
+    // against 195 with three and two; logits store 16 times as much: 225 and 206)
     if (labels)
-        return conv_fwd_tc<32, 16, false, false, true, 3>(m, wf, b, out, W, H, n, nc->S, nc->tc_err, nc->sms, s);
+        return conv_fwd_tc<32, 16, false, false, true, 2>(m, wf, b, out, W, H, n, nc->S, nc->tc_err, nc->sms, s);
     return conv_fwd_tc<32, 16, false, true, false, 3>(m, wf, b, out, W, H, n, nc->S, nc->tc_err, nc->sms, s);
 }
 
@@ -1143,8 +1168,9 @@ cudaError_t conv_fwd(const slic_net_ctx *nc, int l, const __nv_bfloat16 *wf, con
 slic_status forward_all(slic_net_ctx *n, int batch, const uint8_t *d_images, cudaStream_t s,
                         int32_t *labels_out = nullptr, const uint8_t *const *d_table = nullptr, int C = 3,
                         float *logits = nullptr) {
-    const dim3 pg((n->W + 127) / 128, n->H, batch);
-    k_net_prep<<<pg, 128, 0, s>>>(n->conv, d_images, d_table, n->W, n->H, C, n->S, n->m / (float)n->S, n->act[0]);
+    const dim3 pg((n->W + 127) / 128, (n->H + kPrepRows - 1) / kPrepRows, batch);
+    const size_t psm = (size_t)prep_rows(n->S) * prep_cols(n->S) * (sizeof(float4) + sizeof(float));
+    k_net_prep<<<pg, 128, psm, s>>>(n->conv, d_images, d_table, n->W, n->H, C, n->S, n->m / (float)n->S, n->act[0]);
     cudaError_t e = cudaGetLastError();
     for (int l = 0; l < kLayers && e == cudaSuccess; ++l) {
         void *out = l < 3 ? static_cast<void *>(n->act[l + 1])
