@@ -1406,11 +1406,21 @@ slic_status slic_net_get_params(slic_net n, int which, float *h_out, size_t coun
         return nfail(n, SLIC_ERR_INVALID, "bad arguments (count must equal slic_net_param_count)");
     cudaError_t e = cudaDeviceSynchronize();
     size_t off = 0;
+    // every gradient lies in one buffer: one copy, not two per layer
+    std::vector<float> all(which ? kWeights + kBiases : 0);
+    if (which && e == cudaSuccess)
+        e = cudaMemcpy(all.data(), n->grads, sizeof(float) * all.size(), cudaMemcpyDeviceToHost);
     for (int l = 0; l < kLayers && e == cudaSuccess; ++l) {
-        std::vector<float> hw(wcount(l)), hb(kCoutPad[l]);
-        e = cudaMemcpy(hw.data(), which ? n->wg[l] : n->w[l], sizeof(float) * hw.size(), cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(hb.data(), which ? n->bg[l] : n->b[l], sizeof(float) * hb.size(), cudaMemcpyDeviceToHost);
+        std::vector<float> hw(which ? 0 : wcount(l)), hb(which ? 0 : kCoutPad[l]);
+        if (which) {
+            hw.assign(all.begin() + (n->wg[l] - n->grads), all.begin() + (n->wg[l] - n->grads) + wcount(l));
+            hb.assign(all.begin() + (n->bg[l] - n->grads), all.begin() + (n->bg[l] - n->grads) + kCoutPad[l]);
+        } else {
+            e = cudaMemcpy(hw.data(), n->w[l], sizeof(float) * hw.size(), cudaMemcpyDeviceToHost);
+            if (e == cudaSuccess)
+                e = cudaMemcpy(hb.data(), n->b[l], sizeof(float) * hb.size(), cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) break;
+        }
         for (int tap = 0; tap < 9; ++tap)
             for (int ci = 0; ci < kCinReal[l]; ++ci)
                 for (int co = 0; co < kCoutReal[l]; ++co)
