@@ -46,9 +46,9 @@ struct slic_batch_ctx {
     bool any_conv = false;            // some frame has a stopping threshold
     int total_tiles = 0, total_centres = 0, total_rows = 0, max_w = 0, win_max = 0;
     int total_tiles64 = 0, win_max64 = 0;  // the same for 32x64 tiles
-    // Passes with one row group per warp: frames whose S is a multiple of 16
-    // run over 16x16 blocks (k_assign_blocks), the others over tiles
-    int total_blocks = 0, total_rest = 0, block_occ = 0;
+    // Passes of the pipelined path: frames whose S is a multiple of 16 run over
+    // 16x16 blocks (k_assign_blocks), the others over tiles
+    int total_blocks = 0, total_rest = 0, total_rest64 = 0, block_occ = 0;
     int total_chunks = 0;    // update chunks of all frames (fused passes)
     bool fused = false;      // the passes before the last in one cooperative launch
     // Groups: the frames run as `groups` runs of consecutive frames (split
@@ -334,6 +334,7 @@ cudaError_t upload_tables(slic_batch_ctx *b, int k, cudaStream_t s) {
             a.chunk_base -= a0.chunk_base;
             a.block_base -= a0.block_base;
             a.rest_base -= a0.rest_base;
+            a.rest_base64 -= a0.rest_base64;
             gt[f] = a;
         }
     }
@@ -514,17 +515,20 @@ slic_status slic_batch_create(const slic_params *params, int n_frames, slic_batc
         if (b->pipe && !encode_maps(a)) b->pipe = false;  // then every pass uses k_assign_batch
     }
     {
-        // Blocks or 32x32 tiles, per frame, with one row group: at other S a
-        // 16x16 block does not lie in one cell.
+        // Blocks or tiles, per frame: at other S a 16x16 block does not lie in
+        // one cell. 32 x 1080p, S = 16, middle pass: 417 us over blocks, 432
+        // over 32x64 tiles, 549 over 32x32 tiles with one row group.
         b->block_occ = b->pipe ? assign_blocks_occupancy() : 0;
         for (FrameArgs &a : b->frames) {
             a.block_base = b->total_blocks;
             a.rest_base = b->total_rest;
+            a.rest_base64 = b->total_rest64;
             if (b->block_occ > 0 && a.S % 16 == 0) {
                 a.blocks_x = (a.W + 15) / 16;
                 b->total_blocks += a.blocks_x * ((a.H + 15) / 16);
             } else {
                 b->total_rest += a.n_tiles;
+                b->total_rest64 += a.n_tiles64;
             }
         }
     }
@@ -601,14 +605,14 @@ namespace {
 // (bases counted from its first frame) and its totals.
 struct Span {
     const FrameArgs *frames;
-    int n, tiles, tiles64, centres, rows, units, chunks, blocks, rest;
+    int n, tiles, tiles64, centres, rows, units, chunks, blocks, rest, rest64;
 };
 
 // Group g of the batch (g < 0: the whole batch, with its own table).
 Span span_of(const slic_batch_ctx *b, int g) {
     if (g < 0)
         return Span{b->d_frames, b->n, b->total_tiles, b->total_tiles64, b->total_centres, b->total_rows,
-                    b->total_units, b->total_chunks, b->total_blocks, b->total_rest};
+                    b->total_units, b->total_chunks, b->total_blocks, b->total_rest, b->total_rest64};
     const int f0 = b->group_first[g], f1 = b->group_first[g + 1];
     const FrameArgs &a = b->frames[f0];
     const bool end = f1 == b->n;
@@ -621,7 +625,8 @@ Span span_of(const slic_batch_ctx *b, int g) {
                 (end ? b->total_units : z->strip_base) - a.strip_base,
                 (end ? b->total_chunks : z->chunk_base) - a.chunk_base,
                 (end ? b->total_blocks : z->block_base) - a.block_base,
-                (end ? b->total_rest : z->rest_base) - a.rest_base};
+                (end ? b->total_rest : z->rest_base) - a.rest_base,
+                (end ? b->total_rest64 : z->rest_base64) - a.rest_base64};
 }
 
 // Every stage of a segmentation of the span's frames, enqueued on s: the
@@ -689,14 +694,17 @@ cudaError_t enqueue_span(slic_batch_ctx *b, const Span &sp, cudaStream_t s, bool
             if (!b->pipe)
                 return launch_assign_batch(sp.frames, sp.n, sp.tiles, b->win_max, b->same, pass == 0 && !warm, last,
                                            b->smem, grid, s);
-            if (b->rows == 2)
-                return launch_assign_pipe(sp.frames, sp.n, tiles_th, win_th, b->same, last, b->stages, b->rows,
-                                          b->tile_h, pipe_per_sm, grid_pipe, b->d_err, b->any_conv ? 1 : 0, s);
-            if (sp.blocks > 0 && sp.rest > 0) ++n_launch;  // (two launches)
-            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, last, grid_for(b, b->block_occ), b->d_err,
+            const int rest = b->tile_h == 64 ? sp.rest64 : sp.rest;
+            if (sp.blocks > 0 && rest > 0) ++n_launch;  // (two launches)
+            // Blocks: every CTA that fits (2 per SM, 417 us; 1 per SM, 602 us),
+            // but as many as asked for while frame groups share the GPU
+            // (10-iteration step with 4 groups: 4.69 ms at 1 per SM and group,
+            // 4.79 ms at 2)
+            const int grid_blocks = whole ? b->block_occ * b->sms : grid_for(b, b->block_occ);
+            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, last, grid_blocks, b->d_err,
                                                  b->any_conv ? 1 : 0, s);
             if (r == cudaSuccess)
-                r = launch_assign_pipe(sp.frames, sp.n, sp.rest, win_th, b->same, last, b->stages, b->rows, b->tile_h,
+                r = launch_assign_pipe(sp.frames, sp.n, rest, win_th, b->same, last, b->stages, b->rows, b->tile_h,
                                        pipe_per_sm, grid_pipe, b->d_err, b->any_conv ? 1 : 0, s);
             return r;
         };

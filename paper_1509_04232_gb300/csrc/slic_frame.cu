@@ -309,16 +309,17 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
             }
             const float4 *const u_la = f_la + ((size_t)ul * NP + i0) * 32 + lane;
             const float2 *const u_b = f_b + ((size_t)ul * NP + i0) * 32 + lane;
-            unsigned long long l[M], aa[M], b[M], x[M], fy[M];
+            unsigned long long l[M], aa[M], b[M], x[M];
+            float fy[M];
 #pragma unroll
             for (int i = 0; i < M; ++i) {
                 const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(u_la + 32 * i);
                 l[i] = la.x;
                 aa[i] = la.y;
                 b[i] = *reinterpret_cast<const unsigned long long *>(u_b + 32 * i);
-                const float fx = (float)(n.x0 + col[i]), fyi = (float)(n.y0 + row[i]);
+                const float fx = (float)(n.x0 + col[i]);
                 x[i] = pack2(fx, fx + 1.0f);
-                fy[i] = pack2(fyi, fyi);
+                fy[i] = (float)(n.y0 + row[i]);
             }
             // Eq. (1), candidates two at a time as in the pipelined kernel
             float bk[M][2];
@@ -333,11 +334,11 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
                     const float *rp = ctab + 4 * n.rec[t0 + q];
                     const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(rp);
                     const ulonglong2 bx = *reinterpret_cast<const ulonglong2 *>(rp + 4);
-                    const unsigned long long yy = *reinterpret_cast<const unsigned long long *>(rp + 8);
+                    const float yy = rp[8];
 #pragma unroll
                     for (int i = 0; i < M; ++i) {
-                        const unsigned long long ddy = sub2(yy, fy[i]);
-                        eval_keys(la, bx, mul2(ddy, ddy), ww, l[i], aa[i], b[i], XS ? x[0] : x[i], c_tags[t0 + q],
+                        const float ddy = __fsub_rn(yy, fy[i]), ddy2 = __fmul_rn(ddy, ddy);
+                        eval_keys(la, bx, pack2(ddy2, ddy2), ww, l[i], aa[i], b[i], XS ? x[0] : x[i], c_tags[t0 + q],
                                   kk[q][i][0], kk[q][i][1]);
                     }
                 }

@@ -156,11 +156,11 @@ struct FrameArgs {
     // batch's list of chunks
     int n_tiles, n_tiles64, n_chunks;
     int chunk_base;
-    // Split of a pass with one row group per warp (see k_assign_blocks): 16x16
-    // blocks of the frame per row and its first one in the batch's list (frames
-    // whose S is a multiple of 16), and its first 32x32 tile in the list of the
+    // Split of a pass's launches (see k_assign_blocks): 16x16 blocks of the
+    // frame per row and its first one in the batch's list (frames whose S is a
+    // multiple of 16), and its first 32x32 / 32x64 tile in the list of the
     // other frames' tiles. A frame has no entry in the list it is not in.
-    int blocks_x, block_base, rest_base;
+    int blocks_x, block_base, rest_base, rest_base64;
 };
 constexpr int kUpdateChunk = 256;  // centres per update work item of the fused assignment
 

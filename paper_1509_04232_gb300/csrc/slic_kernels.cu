@@ -44,7 +44,7 @@ __device__ __forceinline__ int div_s(int x, unsigned s_mul, int S) {
 // Index of the frame whose [base, next base) range holds `idx` (frames are
 // sorted by base; base of frame 0 is 0).
 enum BaseField {
-    kTileBase, kCentreBase, kRowBase, kStripBase, kTileBase64, kChunkBase, kBlockBase, kRestBase
+    kTileBase, kCentreBase, kRowBase, kStripBase, kTileBase64, kChunkBase, kBlockBase, kRestBase, kRestBase64
 };
 template <BaseField F>
 __device__ __forceinline__ int base_of(const FrameArgs &a) {
@@ -55,6 +55,7 @@ __device__ __forceinline__ int base_of(const FrameArgs &a) {
            : F == kTileBase64 ? a.tile_base64
            : F == kBlockBase ? a.block_base
            : F == kRestBase ? a.rest_base
+           : F == kRestBase64 ? a.rest_base64
                               : a.chunk_base;
 }
 template <BaseField F>
@@ -1147,8 +1148,8 @@ __device__ __forceinline__ void assign_pipe_body(const FrameArgs *frames, int n_
             if (use > 0 && !mbar_wait(&empty[q], (use - 1) & 1)) return false;
             // A producer thread's tiles come in increasing order: its frame
             // index only moves forward.
-            // (one row group: only the frames that k_assign_blocks leaves)
-            constexpr BaseField kBase = TH == 64 ? kTileBase64 : ROWS == 2 ? kTileBase : kRestBase;
+            // (only the frames that k_assign_blocks leaves)
+            constexpr BaseField kBase = TH == 64 ? kRestBase64 : kRestBase;
             while (pf + 1 < n_frames && base_of<kBase>(frames[pf + 1]) <= t) ++pf;
             const int f = pf;
             TileGeom g = tile_geom<TH>(frames[f], t - base_of<kBase>(frames[f]));
@@ -1672,6 +1673,14 @@ constexpr int kBlkCen = 9 * kCtabRec * 4;       // and of its centre records
 constexpr int kBlkStage = (kBlkFeat + kBlkCen + 127) & ~127;
 constexpr int kBlkBinWords = 160;               // word q of candidate t, copy c: q * 40 + t * 4 + c
 
+// Shared-memory loads that stay where they are written.
+__device__ __forceinline__ void lds_u64x2(ulonglong2 &v, const float *p) {
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(smem_addr(p)));
+}
+__device__ __forceinline__ void lds_f32(float &v, const float *p) {
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(smem_addr(p)));
+}
+
 // A block: frame, cell, first pixel, extent inside the image, cell column.
 struct __align__(16) BlockHdr {
     int f, k, x0, y0;
@@ -1685,7 +1694,7 @@ struct __align__(16) BlockState {
     float fs, w;
     int32_t *out;
     unsigned long long *acc;
-    int k, cx, y0, have;  // the block the totals belong to (have: there is one)
+    int k, pad[3];  // the cell the totals are around, -1: none
     longlong2 total[27];
 };
 constexpr int kBlkHdrs = 64;  // of a warp: two runs of 32, made by its lanes together
@@ -1740,7 +1749,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
     make_headers(0);
     if (lane == 0) {
         me->f = -1;
-        me->have = 0;
+        me->k = -1;
     }
     __syncwarp();
     // One lane: copy block j into stage j % kBlkStages.
@@ -1791,10 +1800,10 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
             continue;
         }
         if (h.f != me->f) {  // (all lanes read it before lane 0 writes)
-            if (!LAST && me->have && lane < 27) flush(me->k);
+            if (!LAST && me->k >= 0 && lane < 27) flush(me->k);
             __syncwarp();
             if (lane == 0) {
-                me->have = 0;
+                me->k = -1;
                 const FrameArgs &a = frames[h.f];
                 me->f = h.f;
                 me->W = a.W;
@@ -1813,8 +1822,9 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
         const unsigned char *const st = stages + (size_t)q * kBlkStage;
         const float *const feat = reinterpret_cast<const float *>(st);
         const float *const cen = reinterpret_cast<const float *>(st + kBlkFeat);
-        unsigned long long l[4], a[4], b[4], fy[4];
-        const float fx = (float)(h.x0 + col);
+        unsigned long long l[4], a[4], b[4];
+        float fy[4];
+        const float fx = (float)(h.x0 + col), fy0 = (float)(h.y0 + row);  // (whole numbers: the sums below are exact)
         const unsigned long long x = pack2(fx, fx + 1.0f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -1822,27 +1832,36 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
             l[i] = *reinterpret_cast<const unsigned long long *>(p);
             a[i] = *reinterpret_cast<const unsigned long long *>(p + kBlk * kBlk);
             b[i] = *reinterpret_cast<const unsigned long long *>(p + 2 * kBlk * kBlk);
-            const float y = (float)(h.y0 + row + 4 * i);
-            fy[i] = pack2(y, y);
+            fy[i] = fy0 + (float)(4 * i);
         }
-        // Eq. (1), with the operations of the tile kernel
+        // Eq. (1), with the operations of the tile kernel (the row's distance
+        // once per pair: both halves are equal). A candidate's record is loaded
+        // while the one before it is evaluated, in this order: left to itself
+        // the compiler loads each where it is needed (438 -> 417 us per pass,
+        // with the scalar row distance).
         float bk[4][2];
 #pragma unroll
         for (int i = 0; i < 4; ++i) bk[i][0] = bk[i][1] = __int_as_float(0x7F800000);
+ulonglong2 nla = *reinterpret_cast<const ulonglong2 *>(cen), nbx = *reinterpret_cast<const ulonglong2 *>(cen + 4);
+        float nyy = cen[8];
 #pragma unroll
         for (int t0 = 0; t0 < 9; t0 += 2) {
             const int nt = t0 < 8 ? 2 : 1;
             float kk[2][4][2];
 #pragma unroll
             for (int u = 0; u < nt; ++u) {
-                const float *rp = cen + (t0 + u) * kCtabRec;
-                const ulonglong2 la = *reinterpret_cast<const ulonglong2 *>(rp);
-                const ulonglong2 bx = *reinterpret_cast<const ulonglong2 *>(rp + 4);
-                const unsigned long long yy = *reinterpret_cast<const unsigned long long *>(rp + 8);
+                const ulonglong2 la = nla, bx = nbx;
+                const float yy = nyy;
+                if (t0 + u < 8) {
+                    const float *rp = cen + (t0 + u + 1) * kCtabRec;
+                    lds_u64x2(nla, rp);
+                    lds_u64x2(nbx, rp + 4);
+                    lds_f32(nyy, rp + 8);
+                }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const unsigned long long ddy = sub2(yy, fy[i]);
-                    eval_keys(la, bx, mul2(ddy, ddy), ww, l[i], a[i], b[i], x, c_tags[t0 + u], kk[u][i][0],
+                    const float ddy = __fsub_rn(yy, fy[i]), ddy2 = __fmul_rn(ddy, ddy);
+                    eval_keys(la, bx, pack2(ddy2, ddy2), ww, l[i], a[i], b[i], x, c_tags[t0 + u], kk[u][i][0],
                               kk[u][i][1]);
                 }
             }
@@ -1856,22 +1875,29 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
         __syncwarp();
         if (lane == 0 && j + kBlkStages < n_blk && !no_copies) produce(j + kBlkStages);
         int t[4][2];  // winning candidate, -1 outside the image
+        const bool whole = h.wl + h.hl == 2 * kBlk;  // (the warp's)
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int v = 0; v < 2; ++v)
-                t[i][v] = row + 4 * i < h.hl && col + v < h.wl ? (int)(__float_as_uint(bk[i][v]) & 15u) : -1;
-        if constexpr (LAST) {
-            const int W = me->W, ns_c = me->ns_c, vec = me->vec;
-            int32_t *const out = me->out;
+            for (int v = 0; v < 2; ++v) t[i][v] = (int)(__float_as_uint(bk[i][v]) & 15u);
+        if (!whole) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                int32_t *const o = out + (size_t)(h.y0 + row + 4 * i) * W + h.x0 + col;
-                int lab[2];
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int v = 0; v < 2; ++v)
-                    lab[v] = h.k - ns_c - 1 + t[i][v] + (int)__umulhi((unsigned)t[i][v], 0x55555556u) * (ns_c - 3);
-                if (vec && t[i][1] >= 0) {
+                    if (row + 4 * i >= h.hl || col + v >= h.wl) t[i][v] = -1;
+        }
+        if constexpr (LAST) {
+            const int W = me->W, ns_c = me->ns_c, base = h.k - ns_c - 1, skip = ns_c - 3;
+            int32_t *o = me->out + (size_t)(h.y0 + row) * W + h.x0 + col;
+            const bool fast = whole && me->vec;
+#pragma unroll
+            for (int i = 0; i < 4; ++i, o += 4 * (size_t)W) {
+                int lab[2];
+#pragma unroll
+                for (int v = 0; v < 2; ++v)  // t / 3 rows of cells down
+                    lab[v] = base + t[i][v] + (int)__umulhi((unsigned)t[i][v], 0x55555556u) * skip;
+                if (fast) {
                     *reinterpret_cast<int2 *>(o) = make_int2(lab[0], lab[1]);
                 } else {
                     if (t[i][0] >= 0) o[0] = lab[0];
@@ -1916,46 +1942,38 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) own[c] = __reduce_add_sync(kFull, own[c]);
+            if (lane < 4)  // the own cell's words into its place among the bins
+                set[lane * 40 + 16] = lane == 0 ? own[0] : lane == 1 ? own[1] : lane == 2 ? own[2] : own[3];
             __syncwarp();
             if (lane < 27) {
                 // The totals follow the block: one cell to the right, the left
                 // column is complete; anything else but the same cell, all nine.
-                const bool row_same = h.y0 == me->y0, right = row_same && h.cx == me->cx + 1,
-                           same = !me->have || (row_same && h.cx == me->cx);
                 longlong2 r = me->total[lane];
-                if (!same) {
-                    if (!right || rt % 3 == 0) flush(me->k);
+                const int lk = me->k;  // (-1: no totals)
+                if (h.k != lk) {
+                    const bool right = h.k == lk + 1 && h.cx > 0;
+                    if (lk >= 0 && (!right || rt % 3 == 0)) flush(lk);
                     r = right && rt % 3 < 2 ? me->total[lane + 3] : make_longlong2(0, 0);
                 }
-                auto word = [&](int c) {  // the four copies' sum (own: the warp's)
-                    if (rt == 4) return c == 0 ? own[0] : c == 1 ? own[1] : c == 2 ? own[2] : own[3];
+                auto word = [&](int c) {  // the four copies' sum
                     const uint4 v = *reinterpret_cast<const uint4 *>(set + c * 40 + rt * 4);
                     return v.x + v.y + v.z + v.w;
                 };
+                // part 0: l, a; 1: b, x; 2: y, count
                 const unsigned xyn = word(3), cnt = xyn >> 22, bias = cnt * kFixBias;
-                if (part == 0) {
-                    r.x += (int)(word(0) - bias);
-                    r.y += (int)(word(1) - bias);
-                } else if (part == 1) {
-                    r.x += (int)(word(2) - bias);
-                    r.y += (long long)(xyn & 0x7FFu) + (long long)cnt * h.x0;
-                } else {
-                    r.x += (long long)((xyn >> 11) & 0x7FFu) + (long long)cnt * h.y0;
-                    r.y += (long long)cnt;
-                }
+                const int c0 = (int)(word(part == 0 ? 0 : 2) - bias), c1 = (int)(word(1) - bias);
+                const long long xs = (long long)(xyn & 0x7FFu) + (long long)cnt * h.x0,
+                                ys = (long long)((xyn >> 11) & 0x7FFu) + (long long)cnt * h.y0;
+                r.x += part < 2 ? (long long)c0 : ys;
+                r.y += part == 0 ? (long long)c1 : part == 1 ? xs : (long long)cnt;
                 __syncwarp(0x7FFFFFFu);  // (totals read before they are replaced)
                 me->total[lane] = r;
-                if (lane == 0) {
-                    me->k = h.k;
-                    me->cx = h.cx;
-                    me->y0 = h.y0;
-                    me->have = 1;
-                }
+                if (lane == 0) me->k = h.k;
             }
         }
     }
     __syncwarp();
-    if (!LAST && ok && me->have && lane < 27) flush(me->k);
+    if (!LAST && ok && me->k >= 0 && lane < 27) flush(me->k);
     if (lane == 0 && !ok) atomicOr(err, 1);
     // After a wait that timed out: the copies still in flight land (bounded)
     // before the CTA exits, so none targets freed shared memory.
