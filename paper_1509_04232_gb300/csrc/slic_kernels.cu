@@ -2855,13 +2855,43 @@ __global__ void __launch_bounds__(kCclThreads) k_ccl_relabel(CclFrames fr, int G
     const int ty = local / tiles_x, tx = local - ty * tiles_x;
     const int x0 = tx * kCclTile, y0 = ty * kCclTile;
     const int tw = min(kCclTile, f.W - x0), th = min(kCclTile, f.H - y0);
-    for (int i = threadIdx.x; i < kCclTile * kCclTile; i += kCclThreads) {
-        const int lx = i & (kCclTile - 1), ly = i / kCclTile;
-        if (lx >= tw || ly >= th) continue;
-        const int p = (y0 + ly) * f.W + x0 + lx;
-        int L = parent[f.base + p];
-        if ((unsigned)L >= (unsigned)G) L = f.base;  // (only after a walk gave up)
-        f.out[p] = labels_of[L];
+    // Four pixels per access where rows allow it, every parent loaded before the
+    // labels are gathered and those before any store (one pixel at a time, each
+    // waiting for two loads in turn, took 58 us for 8 x 1080p, 20 us of traffic)
+    constexpr int kRows = kCclThreads / (kCclTile / 4), kIter = kCclTile / kRows;
+    const int lx = 4 * (threadIdx.x % (kCclTile / 4)), ly0 = threadIdx.x / (kCclTile / 4);
+    const bool vec = ((f.W | f.base) & 3) == 0 && ((uintptr_t)f.out & 15) == 0 && ((uintptr_t)parent & 15) == 0 &&
+                     lx + 3 < tw;
+    int L[kIter][4];
+#pragma unroll
+    for (int r = 0; r < kIter; ++r) {
+        const int ly = ly0 + r * kRows, p = (y0 + ly) * f.W + x0 + lx;
+        if (vec && ly < th) {
+            const int4 v = *reinterpret_cast<const int4 *>(parent + f.base + p);
+            L[r][0] = v.x; L[r][1] = v.y; L[r][2] = v.z; L[r][3] = v.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) L[r][q] = ly < th && lx + q < tw ? parent[f.base + p + q] : f.base;
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kIter; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if ((unsigned)L[r][q] >= (unsigned)G) L[r][q] = f.base;  // (only after a walk gave up)
+            L[r][q] = labels_of[L[r][q]];
+        }
+#pragma unroll
+    for (int r = 0; r < kIter; ++r) {
+        const int ly = ly0 + r * kRows, p = (y0 + ly) * f.W + x0 + lx;
+        if (ly >= th) continue;
+        if (vec) {
+            *reinterpret_cast<int4 *>(f.out + p) = make_int4(L[r][0], L[r][1], L[r][2], L[r][3]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (lx + q < tw) f.out[p + q] = L[r][q];
+        }
     }
 }
 
