@@ -2604,32 +2604,61 @@ __global__ void __launch_bounds__(kCclThreads) k_ccl_local(CclFrames fr, int *pa
         par[i] = ly * kCclTile + (31 - __clz(starts));
     }
     __syncthreads();
-    for (int ly = warp + (warp == 0 ? kRowsPerPass : 0); ly < th; ly += kRowsPerPass) {
-        if (!col_ok) continue;
+    // Vertical links. A run's first link needs no union: no other link
+    // changes the run's start yet, so it simply takes the parent of the pixel
+    // above it (smaller indices, one writer). The few other links, of runs
+    // that join two runs above, are unions once every first link is made.
+    volatile int *const vp = par;
+    unsigned more = 0;  // bit of each of this lane's rows with such a link
+    for (int ly = warp; ly < th; ly += kRowsPerPass) {  // (whole warps)
+        if (ly == 0) continue;
         const int i = ly * kCclTile + lane;
-        const int32_t v = lab[i];
-        if (lab[i - kCclTile] != v) continue;
-        if (lane > 0 && lab[i - 1] == v && lab[i - kCclTile - 1] == v) continue;
-        ccl_union_s(par, i, i - kCclTile, err);
+        const int32_t v = lab[i], left = lane > 0 ? lab[i - 1] : 0;
+        const bool same_left = lane > 0 && left == v;
+        const bool link = col_ok && lab[i - kCclTile] == v && !(same_left && lab[i - kCclTile - 1] == v);
+        const unsigned starts = __ballot_sync(kFull, !same_left), links = __ballot_sync(kFull, link);
+        const int s = 31 - __clz(starts & (kFull >> (31 - lane)));
+        if (link) {
+            if ((links & ((1u << lane) - 1u)) >> s)
+                more |= 1u << (ly / kRowsPerPass);
+            else
+                vp[ly * kCclTile + s] = vp[i - kCclTile];
+        }
     }
     __syncthreads();
-    // Roots are always run starts (a link goes from a root to a root), so
-    // only the starts need a walk: each adds its run's length to its root's
-    // size, and the run's pixels take its root (no parent points at a pixel
-    // that is not a run start, so those entries can change freely).
+    // The first links make chains of one row per step. Rounds of "my parent's
+    // parent is my parent" halve them: straight-line code for every pixel, in
+    // place of a walk per run whose loops ran as long as the longest of a warp.
+    auto halve = [&](int rounds) {
+        for (int q = 0; q < rounds; ++q) {
+#pragma unroll
+            for (int r = 0; r < kCclTile / kRowsPerPass; ++r) {
+                const int i = (r * kRowsPerPass + warp) * kCclTile + lane, p = vp[i];
+                const int g = vp[p];
+                if (g != p) vp[i] = g;
+            }
+            __syncthreads();
+        }
+    };
+    halve(3);
+    for (int ly = warp; __any_sync(kFull, more != 0); ly += kRowsPerPass, more >>= 1)
+        if (more & 1u) ccl_union_s(par, ly * kCclTile + lane, (ly - 1) * kCclTile + lane, err);
+    __syncthreads();
+    halve(2);
+    // What is left of a longer chain is walked. Each run's first pixel adds the
+    // run's length to its root's size.
     for (int ly = warp; ly < th; ly += kRowsPerPass) {
         const int i = ly * kCclTile + lane;
+        int r = vp[i];
+        if (vp[r] != r) r = ccl_find_s(par, r, err);
         const int32_t v = lab[i];
         const bool start = col_ok && (lane == 0 || lab[i - 1] != v);
         const unsigned st = __ballot_sync(kFull, start);
-        int r = i;
         if (start) {
-            r = ccl_find_s(par, i, err);
             const unsigned after = st & ~(kFull >> (31 - lane));
             atomicAdd(&cnt[r], (after ? __ffs(after) - 1 : tw) - lane);
         }
-        r = __shfl_sync(kFull, r, 31 - __clz(st & (kFull >> (31 - lane))));
-        if (col_ok) par[i] = r;
+        if (col_ok) vp[i] = r;
     }
     __syncthreads();
     // Parents out; the tile's roots go into the list with one global atomic
