@@ -1842,7 +1842,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
         float bk[4][2];
 #pragma unroll
         for (int i = 0; i < 4; ++i) bk[i][0] = bk[i][1] = __int_as_float(0x7F800000);
-ulonglong2 nla = *reinterpret_cast<const ulonglong2 *>(cen), nbx = *reinterpret_cast<const ulonglong2 *>(cen + 4);
+        ulonglong2 nla = *reinterpret_cast<const ulonglong2 *>(cen), nbx = *reinterpret_cast<const ulonglong2 *>(cen + 4);
         float nyy = cen[8];
 #pragma unroll
         for (int t0 = 0; t0 < 9; t0 += 2) {
