@@ -738,9 +738,13 @@ extern "C" slic_status slic_segment_noalloc(const slic_params *params, const uin
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         plan_resident(p.width, p.height, S, ns_c, ns_r, sms, feat_b, &plan)) {
         int *const words = reinterpret_cast<int *>(ctrl);
-        e = launch_resident(resident_args(a, p.iterations, p.enforce_connectivity == 1, lbl_tmp,
-                                          reinterpret_cast<long long *>(base), words + 1, words),
-                            plan, s);
+        // (calls that overlapped against the rules may have left the barrier
+        // counters of the shared array anywhere)
+        e = cudaMemsetAsync(words + 1, 0, 2 * sizeof(int), s);
+        if (e == cudaSuccess)
+            e = launch_resident(resident_args(a, p.iterations, p.enforce_connectivity == 1, lbl_tmp,
+                                              reinterpret_cast<long long *>(base), words + 1, words),
+                                plan, s);
         done = e == cudaSuccess;
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             cudaGetLastError();

@@ -1,0 +1,135 @@
+"""Edges of the batched block pass, of the label sums and of the network's
+weight gradients: remainders, the smallest sizes, and the sizes where a launch
+splits its work differently."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import net_oracle as NO
+from paper_1509_04232_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _img(W, H, seed, channels=3):
+    import torch
+    return torch.from_numpy(synth.voronoi_frame(W, H, 60, 8.0, seed, channels=channels)).cuda()
+
+
+# (frames as (W, H, S, options), iterations, launch shape, groups). S a multiple
+# of 16 runs over blocks, other S over tiles, both in one batch.
+BLOCKS = [
+    ([(16, 16, 16, {}), (17, 15, 16, {}), (1, 1, 16, {}), (31, 33, 16, {})], 3, None, 1),
+    ([(640, 360, 16, {}), (333, 257, 32, {}), (500, 90, 48, {}), (97, 400, 64, {})], 4, (0, 3, 2, 64), 2),
+    ([(320, 240, 16, {}), (320, 240, 8, {}), (200, 100, 32, {}), (211, 130, 13, {}), (64, 64, 16, {})], 3, None, 3),
+    ([(320, 240, 32, dict(in_channels=4)), (322, 243, 8, {}), (401, 300, 16, dict(color_space=1))], 2, (1, 3, 2, 64), 1),
+    ([(300, 200, 16, dict(convergence=0.5)), (300, 200, 16, {}), (170, 200, 32, dict(convergence=1.0))], 6, None, 1),
+    ([(40, 600, 16, dict(perturb_seeds=True)), (2000, 20, 16, dict(color_space=2))], 2, (2, 4, 2, 32), 2),
+]
+
+
+@pytest.mark.parametrize("frames,iterations,shape,groups", BLOCKS)
+def test_blocks_equal_launch_per_stage(slic_gpu, frames, iterations, shape, groups):
+    """Every frame of the batch is bit-identical to the single frame run stage
+    by stage (a handle whose per-launch timers are on)."""
+    import torch
+    bs = slic_gpu.BatchSegmenter([dict(width=W, height=H, S=S, **kw) for W, H, S, kw in frames], iterations=iterations)
+    if shape:
+        bs.set_tuning(*shape)
+    bs.set_groups(groups)
+    imgs = [_img(W, H, 300 + k, kw.get("in_channels", 3)) for k, (W, H, S, kw) in enumerate(frames)]
+    bs.bind(imgs)
+    for _ in range(2):
+        labels, centres = bs.segment()
+        bs.status()
+    ran = bs.iterations_run
+    for k, (W, H, S, kw) in enumerate(frames):
+        seg = slic_gpu.Segmenter(W, H, S=S, iterations=iterations, **kw)
+        slic_gpu.slic_profile_enable(seg.handle, True)
+        want = seg.segment(imgs[k])
+        assert torch.equal(labels[k], want[0]) and torch.equal(centres[k], want[1]), k
+        assert ran[k] == seg.iterations_run
+
+
+@pytest.mark.parametrize("W,H,S,kind", [(64, 8, 8, "noise"), (65, 9, 4, "noise"), (130, 70, 16, "blocks"),
+                                        (333, 57, 13, "slots"), (3, 2, 2, "noise"), (256, 128, 2, "noise")])
+def test_label_sums(slic_gpu, W, H, S, kind):
+    """slic_update from label maps with few and with very many labels per tile
+    (more than its table holds), runs, and labels outside [0, K): counts exact,
+    means within the centre tolerance 1e-4 max(1, |ref|)."""
+    import torch
+    seg = slic_gpu.Segmenter(W, H, S=S)
+    K = seg.K_eff
+    rng = np.random.default_rng(W * H)
+    y, x = np.mgrid[0:H, 0:W]
+    if kind == "blocks":
+        lab = (y // S) * seg.ns_c + x // S
+    elif kind == "slots":
+        lab = np.clip(y // S + rng.integers(-1, 2, (H, W)), 0, seg.ns_r - 1) * seg.ns_c
+        lab += np.clip(x // S + rng.integers(-1, 2, (H, W)), 0, seg.ns_c - 1)
+    else:
+        lab = rng.integers(-1, K + 1, (H, W))
+    feat = rng.uniform(-128, 128, (3, H, W)).astype(np.float32)
+    start = rng.uniform(0, 50, (K, 6)).astype(np.float32)
+    got = seg.update(torch.from_numpy(feat).cuda(), torch.from_numpy(lab.astype(np.int32)).cuda(),
+                     torch.from_numpy(start).cuda()).cpu().numpy()
+    ok = (lab >= 0) & (lab < K)
+    n = np.bincount(lab[ok], minlength=K)
+    np.testing.assert_array_equal(got[:, 5], n)
+    for c, v in enumerate([*feat.astype(np.float64), x.astype(np.float64), y.astype(np.float64)]):
+        ref = np.where(n > 0, np.bincount(lab[ok], weights=v[ok], minlength=K) / np.maximum(n, 1), start[:, c])
+        assert np.all(np.abs(got[:, c] - ref) <= 1e-4 * np.maximum(1.0, np.abs(ref)))
+
+
+def _away_from_zero(seed):
+    """Parameters that keep every hidden pre-activation away from zero: the odd
+    channels' biases at +2, the even ones' at -2 (dead channels). At so few
+    pixels one ReLU derivative that differs between two roundings of a value
+    near zero would be a large part of an element."""
+    params = NO.init_params(seed)
+    for w, b in params[:3]:
+        b += np.where(np.arange(len(b)) % 2, 2.0, -2.0).astype(np.float32)
+        w *= 0.1
+    return params
+
+
+@pytest.mark.parametrize("n,W,H", [(1, 64, 2), (3, 65, 3), (2, 30, 1), (2, 31, 5), (1, 129, 7), (2, 72, 4)])
+def test_gradients_at_the_edges(slic_gpu, n, W, H):
+    """Weight and bias gradients where rows leave half a row pair, columns a
+    part of a 64-pixel stage or of a 30-pixel segment, and the batch is below
+    the network's largest: the element-wise bound of the gradient test,
+    2^-6 |g| + 2^-8 T + 2^-14 T1 (test_gpu_net.py derives it), at parameters
+    that meet its premise (no ReLU derivative in doubt). Dead channels'
+    gradients are zero exactly."""
+    import torch
+    import test_gpu_net as N
+    from paper_1509_04232_gb300.warmstart import WarmStartNet
+    S = 8
+    net = WarmStartNet(W, H, S, max_batch=n + 1, seed=11)
+    net.set_params(np.concatenate([np.concatenate([w.ravel(), b]) for w, b in _away_from_zero(11)]).astype(np.float32))
+    host = np.stack([synth.voronoi_frame(W, H, 12, 8.0, 700 + i) for i in range(n)])
+    valid = NO.slot_mask(H, W, S)
+    rng = np.random.default_rng(5)
+    target = np.array([[[rng.choice(np.flatnonzero(valid[y, x])) for x in range(W)] for y in range(H)]
+                       for _ in range(n)], np.uint8)
+    net.gradients(torch.from_numpy(host).cuda(), torch.from_numpy(target).cuda())
+    torch.cuda.synchronize()
+    net.status()
+    got, params = N._split(net.grads()), N._split(net.params())
+    ref = [[np.zeros_like(v) for v in p] for p in params]
+    t0 = [[np.zeros_like(v) for v in p] for p in params]
+    t1 = [[np.zeros_like(v) for v in p] for p in params]
+    for i in range(n):
+        x0 = NO.input_channels(oracle.convert(host[i]), S, 10.0)
+        assert min(np.abs(z).min() for _, _, z in NO.forward(x0, params)[1][:3]) > 0.5
+        _, g, dzs = NO.backward(x0, params, target[i].astype(np.int64), valid, bf16=True, bf16_grad=True,
+                                return_dz=True)
+        for l, m in enumerate(N._term_magnitudes(dzs, params)):
+            for k in range(2):
+                ref[l][k] += g[l][k] / n
+                t0[l][k] += m[k] / n
+                t1[l][k] += m[2 + k] / n
+    for l in range(4):
+        for k in range(2):
+            bound = 2.0 ** -6 * np.abs(ref[l][k]) + 2.0 ** -8 * t0[l][k] + 2.0 ** -14 * t1[l][k]
+            assert np.all(np.abs(got[l][k] - ref[l][k]) <= bound), (l, k)
