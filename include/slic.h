@@ -187,7 +187,7 @@ slic_status slic_launch_count(slic_handle h, long long *count);
    records a CUDA event pair around every assignment-kernel launch it
    enqueues, on the launching stream (inside a stream capture these become
    event-record nodes that every replay of the graph re-records).
-   (while enabled, slic_segment launches every stage by itself).
+   While enabled, slic_segment launches every stage by itself.
    slic_profile_read waits for those events and returns the summed duration
    (ms) of the recorded pairs and their number; it does not reset them. */
 slic_status slic_profile_enable(slic_handle h, int enable);
@@ -256,8 +256,12 @@ slic_status slic_batch_segment(slic_batch b, void *stream);
 slic_status slic_batch_segment_host(slic_batch b, const uint8_t *const *host_images, int32_t *const *host_labels,
                                     float *const *host_centres, void *stream);
 
-/* Launch shape of the persistent assignment kernels: resident CTAs per SM
-   (0 = as many as fit, capped by each kernel's occupancy), the number of
+/* Launch shape of the persistent assignment kernels. Frames whose S is a
+   multiple of 16 run over 16x16-pixel blocks, one warp each, unless fused
+   passes are set (slic_batch_set_fused); the shape below is that of all
+   other frames. ctas_per_sm holds for both, for blocks only while frame
+   groups (slic_batch_set_groups) run side by side (else as many as fit).
+   Resident CTAs per SM (0 = as many as fit, capped by each kernel's occupancy), the number of
    TMA pipeline stages (3 or 4; 0 keeps the current value, default 4 where it
    fits), the row groups per warp (1: 256 threads, 4 pixels per thread;
    2: 128 threads per 32 tile rows, 8 pixels per thread, only when every
@@ -383,8 +387,9 @@ slic_status slic_segment_noalloc(const slic_params *params, const uint8_t *d_ima
 
 /* Wait for the current device, then report whether a bounded loop of the
    allocation-free path (component connectivity, enforce_connectivity = 2, or
-   a grid barrier of the one-launch segmentation) gave up since the last check on this device (SLIC_ERR_TIMEOUT: those
-   labels are incomplete). Clears the flag. */
+   a grid barrier of the one-launch segmentation) gave up since the last check
+   on this device (SLIC_ERR_TIMEOUT: those labels are incomplete). Clears the
+   flag. */
 slic_status slic_noalloc_status_check(void);
 
 /* ---- Fault injection, for tests of failure detection ----------------------

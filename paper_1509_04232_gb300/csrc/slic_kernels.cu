@@ -2122,10 +2122,10 @@ __global__ void k_update_batch(const FrameArgs *frames, int n, int total, int it
 // memory, keyed by label, and adds each entry to the global sums once; labels
 // beyond the table's probes go to the global sums directly. Colours are summed
 // as two 16-bit halves of their fixed-point value (at most 512 of each: exact
-// for any value), x and y from the tile's corner. Aggregating the lanes of a
-// warp label by label instead, with six global atomics each, took 153 us for
-// four 1920x1080 label maps of the network, whose labels mix the nine cells of
-// a window (18 us for one 1280x720 SLIC map).
+// for any value), x and y from the tile's corner. 76 us for four 1920x1080 label
+// maps of the network, whose labels mix the nine cells of a window, bound by the
+// shared atomics; 13 us for one 1280x720 SLIC map. Aggregating the lanes of a
+// warp label by label, with six global atomics each, took 153 and 18 us.
 namespace {
 constexpr int kSumW = 64, kSumH = 8, kSumThreads = 128;  // 4 pixels per thread
 constexpr int kSumSlots = 64, kSumProbes = 8;
@@ -2725,7 +2725,8 @@ __global__ void __launch_bounds__(2 * kCclTile) k_ccl_border(CclFrames fr, int *
 
 // The root stages follow a few dependent loads per root. Each thread takes
 // kRootsPer roots side by side, the same step of all of them in flight: one at a
-// time, a stage took 20 to 35 us for the 0.8 million roots of 8 x 1080p frames.
+// time, a stage took 20 to 35 us for the 0.8 million roots of 8 x 1080p frames
+// (all of them: 1075 -> 1057 us per 5-iteration batch).
 namespace {
 constexpr int kRootsPer = 4;
 }
@@ -2971,8 +2972,8 @@ __global__ void __launch_bounds__(kCclThreads) k_ccl_relabel(CclFrames fr, int G
     const int x0 = tx * kCclTile, y0 = ty * kCclTile;
     const int tw = min(kCclTile, f.W - x0), th = min(kCclTile, f.H - y0);
     // Four pixels per access where rows allow it, every parent loaded before the
-    // labels are gathered and those before any store (one pixel at a time, each
-    // waiting for two loads in turn, took 58 us for 8 x 1080p, 20 us of traffic)
+    // labels are gathered and those before any store: 27 us for 8 x 1080p, 20 us
+    // of them traffic (one pixel at a time, each waiting for two loads in turn: 58)
     constexpr int kRows = kCclThreads / (kCclTile / 4), kIter = kCclTile / kRows;
     const int lx = 4 * (threadIdx.x % (kCclTile / 4)), ly0 = threadIdx.x / (kCclTile / 4);
     const bool vec = ((f.W | f.base) & 3) == 0 && ((uintptr_t)f.out & 15) == 0 && ((uintptr_t)parent & 15) == 0 &&

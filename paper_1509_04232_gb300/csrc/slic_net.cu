@@ -83,9 +83,10 @@ __device__ __forceinline__ float sqrt_fast(float v) {
 // A block covers 128 columns of kPrepRows rows. The grid centres its pixels
 // see are converted once into shared memory; a thread walks down its column
 // and keeps its nine centres in registers while the rows stay in one cell row.
-// (One row per block, centres read back for every pixel: 125 us for four
-// 1920x1080 images, bound by the blocks' start-up latency and the shared
-// loads.)
+// 102 us for four 1920x1080 images, 43 of them the traffic of its 35 B/px, the
+// rest nine square roots and the packing per pixel. One row per block, centres
+// read back for every pixel: 125 us, bound by the blocks' start-up latency and
+// the shared loads.
 constexpr int kPrepRows = 8;
 __host__ __device__ constexpr int prep_cols(int S) { return 127 / S + 4; }            // cell columns a block sees
 __host__ __device__ constexpr int prep_rows(int S) { return (kPrepRows - 1) / S + 4; }  // and cell rows
@@ -702,9 +703,10 @@ __global__ void __launch_bounds__((tc_epi_warps(COUT) + 2) * 32) k_conv_fwd_tc(
 // One thread copies into a ring of kWgStages stages, one issues the MMAs, four
 // warps store the sums. Per stage (128 pixels) 12 MMAs of about 48 cycles (6 KB
 // of operands each at 128 B/clk) would take 32 us for 2.1 Mpx, the copies'
-// 208 B/px from L2 about 45 us. Staging K-major operands by transposing rows
-// through shared memory took 310 us per 32 -> 32 layer; MN-major planes of 8
-// channels filled by 16-byte cp.async 133 us (bound by the loads in flight).
+// 208 B/px from L2 about 45 us; a 32 -> 32 layer takes 49 us (DRAM at 67 % of
+// its peak). Staging K-major operands by transposing rows through shared memory
+// took 310 us; MN-major planes of 8 channels filled by 16-byte cp.async 133 us
+// (bound by the loads in flight).
 // ---------------------------------------------------------------------------
 constexpr int kWgK = 64;      // pixels (columns) of a stage
 constexpr int kWgCols = 72;   // input columns copied: kWgK + 2, rounded up to whole swizzle patterns (8 pixels)
@@ -898,8 +900,9 @@ __global__ void __launch_bounds__(256) k_reduce_partials(const float *partial, i
 
 // The last layer's bias gradient (the sums of the stored dL/dlogits) on the
 // way. One pass over 97 B/px by a grid sized for the device, 16-byte loads,
-// and one atomic per sum and block: a thread per pixel with scalar loads and
-// two atomics per warp to the same words took 226 us for 2.1 Mpx.
+// and one atomic per sum and block: 44 us for 2.1 Mpx, most of them DRAM's. A
+// thread per pixel with scalar loads and two atomics per warp to the same words
+// took 226 us.
 __global__ void __launch_bounds__(256) k_softmax_ce(const float *logits, const uint8_t *target, int W, int H, int n_img,
                                                     int S, float inv_total, __nv_bfloat16 *dz, float *stats,
                                                     float *db) {
