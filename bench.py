@@ -14,7 +14,7 @@ Prints ONE JSON line (rank 0). Keys beyond the base contract:
   quality       the agreement-vs-iterations curves of both methods, their
                 iteration counts at 99 % and frames/s there, the network's
                 training and its forward against the bf16 tensor roofline
-  roofline      the dominant kernel (the pipelined assignment pass) against
+  roofline      the dominant kernel (the middle assignment pass) against
                 its bound (the square-root pipe), with its HBM view
   cpu_baseline  the FP64 CPU oracle timed on a bounded sample over all host
                 cores (one process per core), with a one-core figure beside it
@@ -349,12 +349,12 @@ def run_ours(args):
     # --- dominant kernel: event-timed replays of the plain step ---
     # Each replay records one event pair per assignment launch. One launch
     # per pass: pass order 0..n, and passes 1..n-1 run the dominant kernel
-    # (the pipelined middle pass, k_assign_pipe<0,1,MINB,ROWS,TILE_H>: MINB
-    # = 2 for 32x64 tiles, 4 for the 32x32 two-row-group build and for the
-    # one-row 64-register build the autotuner picks at 4 CTAs per SM, else
-    # 3). Fused passes: the fused launch (passes 0..n-1 with their updates,
-    # k_assign_multi<1,MINB,ROWS,TILE_H>) and the last pass; the fused launch
-    # is the dominant kernel, with n passes' work. With the timers on, the
+    # (the middle pass over 16x16 blocks, k_assign_blocks<0>: S is a multiple
+    # of 16). Fused passes: the fused launch (passes 0..n-1 with their
+    # updates, k_assign_multi<1,MINB,ROWS,TILE_H>: MINB = 2 for 32x64 tiles, 4
+    # for the 32x32 two-row-group build and for the one-row 64-register build
+    # the autotuner picks at 4 CTAs per SM, else 3) and the last pass; the
+    # fused launch is the dominant kernel, with n passes' work. With the timers on, the
     # batch runs as one group of frames (concurrent groups would share the
     # GPU during a launch, so its duration would not be its own).
     pb = bs if method["name"] == "plain" else _plain_batch(pkg, frames, n_plain, dev, tuning)
@@ -369,7 +369,7 @@ def run_ours(args):
     minb = 2 if tile_h == 64 else (4 if (rows == 2 or occ_alone >= 4) else 3)
     fused_dom = bool(fused) and n_plain >= 1
     kname = (f"k_assign_multi<1,{minb},{rows},{tile_h}>" if fused_dom else
-             f"k_assign_pipe<0,1,{minb},{rows},{tile_h}>")
+             "k_assign_blocks<0>")
     passes_per_launch = n_plain if fused_dom else 1
     mid = []
     for _ in range(max(3, min(args.steps, 10))):
@@ -522,7 +522,7 @@ def run_ours(args):
                          "unit": "Tsqrt/s", "achieved": achieved_tops, "peak": xu_peak, "frac": achieved_tops / xu_peak,
                          "peak_source": f"16 MUFU lanes/clk/SM x {sms} SMs x max SM clock (recipe unit counts)",
                          "traffic": traffic, "avg_launch_us": mid_ms * 1e3, "launches_timed": len(mid),
-                         "measured_as": f"one frame group at full occupancy ({occ_alone} CTAs/SM); the step runs "
+                         "measured_as": f"one frame group at full occupancy ({occ_alone if fused_dom else 2} CTAs/SM); the step runs "
                                         f"{groups} group(s) concurrently at {ctas_per_sm} CTAs/SM each",
                          "in_step": {"achieved": in_step_tops,
                                      "frac": in_step_tops / xu_peak if in_step_tops else None,
@@ -579,7 +579,7 @@ def single_frame_latency(args, pkg, stream, dev, image):
         t = np.array([evs[k].elapsed_time(evs[k + 1]) for k in range(reps)])
         out[name] = {"ms_p50": float(np.percentile(t, 50)), "ms_p99": float(np.percentile(t, 99)),
                      "frames_per_s": 1e3 / float(np.mean(t)), "K_eff": seg.K_eff, "iterations": ITERS,
-                     "launches_per_frame": per_frame}
+                     "stages_per_frame": per_frame}  # (one launch runs them all)
         seg.close()
     return out
 
