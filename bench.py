@@ -349,7 +349,7 @@ def run_ours(args):
     # --- dominant kernel: event-timed replays of the plain step ---
     # Each replay records one event pair per assignment launch. One launch
     # per pass: pass order 0..n, and passes 1..n-1 run the dominant kernel
-    # (the middle pass over 16x16 blocks, k_assign_blocks<0>: S is a multiple
+    # (the middle pass over 16x16 blocks, k_assign_blocks<0,1>: S is a multiple
     # of 16). Fused passes: the fused launch (passes 0..n-1 with their
     # updates, k_assign_multi<1,MINB,ROWS,TILE_H>: MINB = 2 for 32x64 tiles, 4
     # for the 32x32 two-row-group build and for the one-row 64-register build
@@ -369,7 +369,7 @@ def run_ours(args):
     minb = 2 if tile_h == 64 else (4 if (rows == 2 or occ_alone >= 4) else 3)
     fused_dom = bool(fused) and n_plain >= 1
     kname = (f"k_assign_multi<1,{minb},{rows},{tile_h}>" if fused_dom else
-             "k_assign_blocks<0>")
+             "k_assign_blocks<0,1>")
     passes_per_launch = n_plain if fused_dom else 1
     mid = []
     for _ in range(max(3, min(args.steps, 10))):

@@ -256,8 +256,8 @@ slic_status slic_batch_segment(slic_batch b, void *stream);
 slic_status slic_batch_segment_host(slic_batch b, const uint8_t *const *host_images, int32_t *const *host_labels,
                                     float *const *host_centres, void *stream);
 
-/* Launch shape of the persistent assignment kernels. Frames whose S is a
-   multiple of 16 run over 16x16-pixel blocks, one warp each, unless fused
+/* Launch shape of the persistent assignment kernels. Frames whose S is 8 or
+   a multiple of 16 run over 16x16-pixel blocks, one warp each, unless fused
    passes are set (slic_batch_set_fused); the shape below is that of all
    other frames. ctas_per_sm holds for both, for blocks only while frame
    groups (slic_batch_set_groups) run side by side (else as many as fit).

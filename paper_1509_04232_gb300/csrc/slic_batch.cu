@@ -46,9 +46,9 @@ struct slic_batch_ctx {
     bool any_conv = false;            // some frame has a stopping threshold
     int total_tiles = 0, total_centres = 0, total_rows = 0, max_w = 0, win_max = 0;
     int total_tiles64 = 0, win_max64 = 0;  // the same for 32x64 tiles
-    // Passes of the pipelined path: frames whose S is a multiple of 16 run over
-    // 16x16 blocks (k_assign_blocks), the others over tiles
-    int total_blocks = 0, total_rest = 0, total_rest64 = 0, block_occ = 0;
+    // Passes of the pipelined path: frames whose S is 8 or a multiple of 16 run
+    // over 16x16 blocks (k_assign_blocks), the others over tiles
+    int total_blocks = 0, total_blocks8 = 0, total_rest = 0, total_rest64 = 0, block_occ = 0;
     int total_chunks = 0;    // update chunks of all frames (fused passes)
     bool fused = false;      // the passes before the last in one cooperative launch
     // Groups: the frames run as `groups` runs of consecutive frames (split
@@ -152,13 +152,13 @@ bool encode_maps(FrameArgs &a) {
     // 32x64 tiles: a box twice as high, and the taller window of centres
     const cuuint32_t fbox64[3] = {(cuuint32_t)kTileW, (cuuint32_t)(2 * kTileH), 3};
     const cuuint32_t cbox64[2] = {(cuuint32_t)a.box_w * kCtabRec, (cuuint32_t)a.box_h64};
-    // 16x16 blocks and the 3x3 records around a cell
+    // 16x16 blocks and the records around their cells
     const cuuint32_t fbox16[3] = {16, 16, 3};
-    const cuuint32_t cbox9[2] = {3 * kCtabRec, 3};
+    const cuuint32_t side = a.S == 8 ? 4 : 3, cbox_blk[2] = {side * kCtabRec, side};
     if (enc(&a.feat_map16, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.feat, fdim, fstride, fbox16, ones,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-        enc(&a.ctab_map9, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.ctab, cdim, cstride, cbox9, ones,
+        enc(&a.ctab_map_blk, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.ctab, cdim, cstride, cbox_blk, ones,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
@@ -333,6 +333,7 @@ cudaError_t upload_tables(slic_batch_ctx *b, int k, cudaStream_t s) {
             a.strip_base -= a0.strip_base;
             a.chunk_base -= a0.chunk_base;
             a.block_base -= a0.block_base;
+            a.block8_base -= a0.block8_base;
             a.rest_base -= a0.rest_base;
             a.rest_base64 -= a0.rest_base64;
             gt[f] = a;
@@ -515,17 +516,18 @@ slic_status slic_batch_create(const slic_params *params, int n_frames, slic_batc
         if (b->pipe && !encode_maps(a)) b->pipe = false;  // then every pass uses k_assign_batch
     }
     {
-        // Blocks or tiles, per frame: at other S a 16x16 block does not lie in
-        // one cell. 32 x 1080p, S = 16, middle pass: 417 us over blocks, 432
+        // Blocks or tiles, per frame: at other S a 16x16 block is not made of
+        // whole cells nor part of one. 32 x 1080p, S = 16, middle pass: 417 us over blocks, 432
         // over 32x64 tiles, 549 over 32x32 tiles with one row group.
         b->block_occ = b->pipe ? assign_blocks_occupancy() : 0;
         for (FrameArgs &a : b->frames) {
             a.block_base = b->total_blocks;
+            a.block8_base = b->total_blocks8;
             a.rest_base = b->total_rest;
             a.rest_base64 = b->total_rest64;
-            if (b->block_occ > 0 && a.S % 16 == 0) {
+            if (b->block_occ > 0 && (a.S % 16 == 0 || a.S == 8)) {
                 a.blocks_x = (a.W + 15) / 16;
-                b->total_blocks += a.blocks_x * ((a.H + 15) / 16);
+                (a.S == 8 ? b->total_blocks8 : b->total_blocks) += a.blocks_x * ((a.H + 15) / 16);
             } else {
                 b->total_rest += a.n_tiles;
                 b->total_rest64 += a.n_tiles64;
@@ -605,14 +607,14 @@ namespace {
 // (bases counted from its first frame) and its totals.
 struct Span {
     const FrameArgs *frames;
-    int n, tiles, tiles64, centres, rows, units, chunks, blocks, rest, rest64;
+    int n, tiles, tiles64, centres, rows, units, chunks, blocks, blocks8, rest, rest64;
 };
 
 // Group g of the batch (g < 0: the whole batch, with its own table).
 Span span_of(const slic_batch_ctx *b, int g) {
     if (g < 0)
         return Span{b->d_frames, b->n, b->total_tiles, b->total_tiles64, b->total_centres, b->total_rows,
-                    b->total_units, b->total_chunks, b->total_blocks, b->total_rest, b->total_rest64};
+                    b->total_units, b->total_chunks, b->total_blocks, b->total_blocks8, b->total_rest, b->total_rest64};
     const int f0 = b->group_first[g], f1 = b->group_first[g + 1];
     const FrameArgs &a = b->frames[f0];
     const bool end = f1 == b->n;
@@ -625,6 +627,7 @@ Span span_of(const slic_batch_ctx *b, int g) {
                 (end ? b->total_units : z->strip_base) - a.strip_base,
                 (end ? b->total_chunks : z->chunk_base) - a.chunk_base,
                 (end ? b->total_blocks : z->block_base) - a.block_base,
+                (end ? b->total_blocks8 : z->block8_base) - a.block8_base,
                 (end ? b->total_rest : z->rest_base) - a.rest_base,
                 (end ? b->total_rest64 : z->rest_base64) - a.rest_base64};
 }
@@ -695,13 +698,13 @@ cudaError_t enqueue_span(slic_batch_ctx *b, const Span &sp, cudaStream_t s, bool
                 return launch_assign_batch(sp.frames, sp.n, sp.tiles, b->win_max, b->same, pass == 0 && !warm, last,
                                            b->smem, grid, s);
             const int rest = b->tile_h == 64 ? sp.rest64 : sp.rest;
-            if (sp.blocks > 0 && rest > 0) ++n_launch;  // (two launches)
+            n_launch += std::max(0, (sp.blocks > 0) + (sp.blocks8 > 0) + (rest > 0) - 1);  // (one launch each)
             // Blocks: every CTA that fits (2 per SM, 417 us; 1 per SM, 602 us),
             // but as many as asked for while frame groups share the GPU
             // (10-iteration step with 4 groups: 4.69 ms at 1 per SM and group,
             // 4.79 ms at 2)
             const int grid_blocks = whole ? b->block_occ * b->sms : grid_for(b, b->block_occ);
-            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, last, grid_blocks, b->d_err,
+            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, sp.blocks8, last, grid_blocks, b->d_err,
                                                  b->any_conv ? 1 : 0, s);
             if (r == cudaSuccess)
                 r = launch_assign_pipe(sp.frames, sp.n, rest, win_th, b->same, last, b->stages, b->rows, b->tile_h,

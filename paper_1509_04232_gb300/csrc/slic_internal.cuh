@@ -117,7 +117,7 @@ struct FrameArgs {
     CUtensorMap feat_map64; // the same for 32x64 tiles: box 32x64x3, and
     CUtensorMap ctab_map64; // box box_w*kCtabRec x box_h64
     CUtensorMap feat_map16; // for 16x16 blocks: box 16x16x3, and the
-    CUtensorMap ctab_map9;  // 3x3 records around a cell
+    CUtensorMap ctab_map_blk;  // the records around a block's cells: 3x3, or 4x4 (S = 8)
     ConvConsts conv;
     const uint8_t *rgb;     // [H][W][C]
     float *feat;            // 3 planes [H][P]; plane stride H*P
@@ -158,9 +158,10 @@ struct FrameArgs {
     int chunk_base;
     // Split of a pass's launches (see k_assign_blocks): 16x16 blocks of the
     // frame per row and its first one in the batch's list (frames whose S is a
-    // multiple of 16), and its first 32x32 / 32x64 tile in the list of the
-    // other frames' tiles. A frame has no entry in the list it is not in.
-    int blocks_x, block_base, rest_base, rest_base64;
+    // multiple of 16; those with S = 8 have a list of their own), and its first
+    // 32x32 / 32x64 tile in the list of the other frames' tiles. A frame has no
+    // entry in the lists it is not in.
+    int blocks_x, block_base, block8_base, rest_base, rest_base64;
 };
 constexpr int kUpdateChunk = 256;  // centres per update work item of the fused assignment
 
@@ -227,10 +228,11 @@ cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles
                                int nst, int rows, int tile_h, int ctas_per_sm, int grid, int *err, int check_stop,
                                cudaStream_t s);
 // The same pass over 16x16 blocks, a warp per block, for the frames whose S is
-// a multiple of 16 (total_blocks of them in all); launch_assign_pipe then
-// takes the tiles of the rest. Resident CTAs per SM of its kernels.
-cudaError_t launch_assign_blocks(const FrameArgs *d_frames, int n, int total_blocks, bool last, int grid, int *err,
-                                 int check_stop, cudaStream_t s);
+// a multiple of 16 (total_blocks of them in all) or 8 (total_blocks8, a launch
+// of their own); launch_assign_pipe then takes the tiles of the rest. Resident
+// CTAs per SM of its kernels.
+cudaError_t launch_assign_blocks(const FrameArgs *d_frames, int n, int total_blocks, int total_blocks8, bool last,
+                                 int grid, int *err, int check_stop, cudaStream_t s);
 int assign_blocks_occupancy();
 // Fused multi-pass form of the tile kernel, one cooperative launch: passes
 // 0 .. passes-1 with the update after each (updates 1 .. passes), ordered

@@ -44,7 +44,7 @@ __device__ __forceinline__ int div_s(int x, unsigned s_mul, int S) {
 // Index of the frame whose [base, next base) range holds `idx` (frames are
 // sorted by base; base of frame 0 is 0).
 enum BaseField {
-    kTileBase, kCentreBase, kRowBase, kStripBase, kTileBase64, kChunkBase, kBlockBase, kRestBase, kRestBase64
+    kTileBase, kCentreBase, kRowBase, kStripBase, kTileBase64, kChunkBase, kBlockBase, kBlock8Base, kRestBase, kRestBase64
 };
 template <BaseField F>
 __device__ __forceinline__ int base_of(const FrameArgs &a) {
@@ -54,6 +54,7 @@ __device__ __forceinline__ int base_of(const FrameArgs &a) {
            : F == kStripBase ? a.strip_base
            : F == kTileBase64 ? a.tile_base64
            : F == kBlockBase ? a.block_base
+           : F == kBlock8Base ? a.block8_base
            : F == kRestBase ? a.rest_base
            : F == kRestBase64 ? a.rest_base64
                               : a.chunk_base;
@@ -1645,7 +1646,7 @@ cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles
 
 // ---------------------------------------------------------------------------
 // One pass over 16x16 blocks, a warp per block (frames whose S is a multiple
-// of 16: a block lies in one cell)
+// of 16: a block lies in one cell; or 8: in 2x2)
 // ---------------------------------------------------------------------------
 //
 // The tile kernel above shares a tile between the warps of a CTA: headers,
@@ -1664,14 +1665,25 @@ cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles
 // of the nine cells stay in the lanes' registers while the run moves along a
 // row, shifted by one cell at a time: only the three cells left behind go to
 // global memory, so a block costs 18 atomic lanes, not 54.
+//
+// CS = 2: frames with S = 8, a block of 2x2 cells. Eight lanes take a cell
+// (columns 2 * (l % 4), rows l / 4 % 2 + 2 i of it): a lane's pixels share one
+// window of 3x3 records among the block's 4x4, at its own base address.
 namespace {
 constexpr int kBlk = 16;
 constexpr int kBlkThreads = 256, kBlkWarps = kBlkThreads / 32;
 constexpr int kBlkStages = 2;
 constexpr int kBlkFeat = 3 * kBlk * kBlk * 4;   // bytes of a stage's features
-constexpr int kBlkCen = 9 * kCtabRec * 4;       // and of its centre records
-constexpr int kBlkStage = (kBlkFeat + kBlkCen + 127) & ~127;
-constexpr int kBlkBinWords = 160;               // word q of candidate t, copy c: q * 40 + t * 4 + c
+// CS cells a side: a window of side * side cells around the block's.
+template <int CS>
+struct BlkGeo {
+    static constexpr int side = CS + 2, cells = side * side;
+    static constexpr int cen = cells * kCtabRec * 4;  // bytes of a stage's centre records
+    static constexpr int stage = (kBlkFeat + cen + 127) & ~127;
+    static constexpr int q = CS == 1 ? 40 : 64;       // bins: word c of cell t, copy k: c * q + t * 4 + k
+    static constexpr int bins = 4 * q;
+    static constexpr int ents = 3 * cells;            // running totals: two of a cell's six sums each
+};
 
 // Shared-memory loads that stay where they are written.
 __device__ __forceinline__ void lds_u64x2(ulonglong2 &v, const float *p) {
@@ -1689,24 +1701,30 @@ struct __align__(16) BlockHdr {
 
 // What a warp keeps in shared memory rather than in registers (the candidate
 // loop needs those): the frame its blocks come from, and the lanes' totals.
+template <int CS>
 struct __align__(16) BlockState {
     int f, W, ns_c, vec;
     float fs, w;
     int32_t *out;
     unsigned long long *acc;
     int k, pad[3];  // the cell the totals are around, -1: none
-    longlong2 total[27];
+    longlong2 total[BlkGeo<CS>::ents];
 };
 constexpr int kBlkHdrs = 64;  // of a warp: two runs of 32, made by its lanes together
 
+template <int CS>
 constexpr size_t blocks_smem_bytes() {
-    return (size_t)kBlkWarps * (kBlkStages * (kBlkStage + 8) + kBlkHdrs * sizeof(BlockHdr) + sizeof(BlockState) + 2 * kBlkBinWords * 4) + 128;
+    return (size_t)kBlkWarps * (kBlkStages * (BlkGeo<CS>::stage + 8) + kBlkHdrs * sizeof(BlockHdr) +
+                                sizeof(BlockState<CS>) + 2 * BlkGeo<CS>::bins * 4) + 128;
 }
 }  // namespace
 
-template <bool LAST>
+template <bool LAST, int CS>
 __global__ void __launch_bounds__(kBlkThreads, 2)
     k_assign_blocks(const FrameArgs *frames, int n_frames, int total_blocks, int *err, int check_stop) {
+    using Geo = BlkGeo<CS>;
+    constexpr int kBlkStage = Geo::stage, kBlkBinWords = Geo::bins, kSide = Geo::side, kQ = Geo::q;
+    constexpr int kEnts = Geo::ents;
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     unsigned char *const smem =
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~(uintptr_t)127);
@@ -1715,7 +1733,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
     unsigned *const bins =
         reinterpret_cast<unsigned *>(smem + (size_t)kBlkWarps * kBlkStages * kBlkStage) + warp * 2 * kBlkBinWords;
     BlockHdr *const hdr = reinterpret_cast<BlockHdr *>(bins + (kBlkWarps - warp) * 2 * kBlkBinWords) + warp * kBlkHdrs;
-    BlockState *const me = reinterpret_cast<BlockState *>(hdr + (kBlkWarps - warp) * kBlkHdrs) + warp;
+    BlockState<CS> *const me = reinterpret_cast<BlockState<CS> *>(hdr + (kBlkWarps - warp) * kBlkHdrs) + warp;
     uint64_t *const full = reinterpret_cast<uint64_t *>(me + kBlkWarps - warp) + warp * kBlkStages;
 
     // This warp's run of the batch's blocks.
@@ -1732,9 +1750,9 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
         h.f = -1;
         if (j0 + lane < n_blk) {
             const int b = b0 + j0 + lane;
-            h.f = find_frame<kBlockBase>(frames, n_frames, b);
+            h.f = find_frame<CS == 1 ? kBlockBase : kBlock8Base>(frames, n_frames, b);
             const FrameArgs &a = frames[h.f];
-            const int local = b - a.block_base, by = local / a.blocks_x;
+            const int local = b - (CS == 1 ? a.block_base : a.block8_base), by = local / a.blocks_x;
             h.x0 = (local - by * a.blocks_x) * kBlk;
             h.y0 = by * kBlk;
             h.cx = div_s(h.x0, a.s_mul, a.S);
@@ -1762,9 +1780,9 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
         }
         const FrameArgs &a = frames[h.f];
         unsigned char *const st = stages + (size_t)(j % kBlkStages) * kBlkStage;
-        mbar_expect_tx(bar, kBlkFeat + kBlkCen);
+        mbar_expect_tx(bar, kBlkFeat + Geo::cen);
         tma_load_3d(st, &a.feat_map16, h.x0, h.y0, 0, bar);
-        tma_load_2d(st + kBlkFeat, &a.ctab_map9, h.cx * kCtabRec, h.cy, bar);
+        tma_load_2d(st + kBlkFeat, &a.ctab_map_blk, h.cx * kCtabRec, h.cy, bar);
     };
     // (fault injection: copies are not to be issued)
     const bool no_copies = *reinterpret_cast<volatile int *>(&g_abort_copies) != 0;
@@ -1772,17 +1790,26 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
     if (lane == 0 && !no_copies)
         for (int j = 0; j < kBlkStages && j < n_blk; ++j) produce(j);
 
-    const int row = lane >> 3, col = 2 * (lane & 7);
-    // Running totals: lane 3 * t + part (t < 9) keeps two of the six sums of the
-    // cell at candidate t's place around the last block's cell.
-    const int part = lane - lane / 3 * 3, rt = lane / 3;
-    auto flush = [&](int k) {  // the lane's totals, around cell k, to the global sums
-        const longlong2 r = me->total[lane];
+    // The lane's pixels: pairs at column col of rows row + kStep * i, in the
+    // block's cell (qx, qy); win: that cell's window in the block's.
+    constexpr int kStep = CS == 1 ? 4 : 2;
+    const int qx = CS == 1 ? 0 : (lane >> 3) & 1, qy = CS == 1 ? 0 : lane >> 4, win = qy * kSide + qx;
+    const int row = CS == 1 ? lane >> 3 : 8 * qy + ((lane >> 2) & 1), col = CS == 1 ? 2 * (lane & 7) : 8 * qx + 2 * (lane & 3);
+    // Running totals: entry 3 * t + part keeps two of the six sums of the cell
+    // at place t of the window around the last block. A lane looks after entry
+    // lane and, of 48, entry lane + 32.
+    const int part = lane - lane / 3 * 3, rt = lane / 3, rt1 = (lane + 32) / 3, part1 = lane + 32 - rt1 * 3;
+    auto flush = [&](int e, int t, int p, int k) {  // entry e, around cell k, to the global sums
+        const longlong2 r = me->total[e];
         if ((r.x | r.y) != 0) {
-            unsigned long long *g = me->acc + (size_t)(k + (rt / 3 - 1) * me->ns_c + rt % 3 - 1) * 6 + 2 * part;
+            unsigned long long *g = me->acc + (size_t)(k + (t / kSide - 1) * me->ns_c + t % kSide - 1) * 6 + 2 * p;
             atomicAdd(g, (unsigned long long)r.x);
             atomicAdd(g + 1, (unsigned long long)r.y);
         }
+    };
+    auto flush_all = [&](int k) {
+        if (CS == 2 || lane < kEnts) flush(lane, rt, part, k);
+        if (CS == 2 && lane < kEnts - 32) flush(lane + 32, rt1, part1, k);
     };
 
     int j = 0, par = 0;  // par: the bins' set
@@ -1800,7 +1827,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
             continue;
         }
         if (h.f != me->f) {  // (all lanes read it before lane 0 writes)
-            if (!LAST && me->k >= 0 && lane < 27) flush(me->k);
+            if (!LAST && me->k >= 0) flush_all(me->k);
             __syncwarp();
             if (lane == 0) {
                 me->k = -1;
@@ -1814,25 +1841,27 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
                 me->out = a.assign_out;
                 me->acc = reinterpret_cast<unsigned long long *>(a.acc);
             }
-            if (!LAST && lane < 27) me->total[lane] = make_longlong2(0, 0);
+            if (!LAST && lane < kEnts) me->total[lane] = make_longlong2(0, 0);
+            if (!LAST && CS == 2 && lane < kEnts - 32) me->total[lane + 32] = make_longlong2(0, 0);
             __syncwarp();
         }
         const float w = me->w;
         const unsigned long long ww = pack2(w, w);
         const unsigned char *const st = stages + (size_t)q * kBlkStage;
         const float *const feat = reinterpret_cast<const float *>(st);
-        const float *const cen = reinterpret_cast<const float *>(st + kBlkFeat);
+        const float *const cen = CS == 1 ? reinterpret_cast<const float *>(st + kBlkFeat)
+                                         : reinterpret_cast<const float *>(st + kBlkFeat) + win * kCtabRec;
         unsigned long long l[4], a[4], b[4];
         float fy[4];
         const float fx = (float)(h.x0 + col), fy0 = (float)(h.y0 + row);  // (whole numbers: the sums below are exact)
         const unsigned long long x = pack2(fx, fx + 1.0f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const float *const p = feat + (row + 4 * i) * kBlk + col;
+            const float *const p = feat + (row + kStep * i) * kBlk + col;
             l[i] = *reinterpret_cast<const unsigned long long *>(p);
             a[i] = *reinterpret_cast<const unsigned long long *>(p + kBlk * kBlk);
             b[i] = *reinterpret_cast<const unsigned long long *>(p + 2 * kBlk * kBlk);
-            fy[i] = fy0 + (float)(4 * i);
+            fy[i] = fy0 + (float)(kStep * i);
         }
         // Eq. (1), with the operations of the tile kernel (the row's distance
         // once per pair: both halves are equal). A candidate's record is loaded
@@ -1853,7 +1882,8 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
                 const ulonglong2 la = nla, bx = nbx;
                 const float yy = nyy;
                 if (t0 + u < 8) {
-                    const float *rp = cen + (t0 + u + 1) * kCtabRec;
+                    const int nx = t0 + u + 1;
+                    const float *rp = cen + (nx / 3 * kSide + nx % 3) * kCtabRec;
                     lds_u64x2(nla, rp);
                     lds_u64x2(nbx, rp + 4);
                     lds_f32(nyy, rp + 8);
@@ -1885,14 +1915,14 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int v = 0; v < 2; ++v)
-                    if (row + 4 * i >= h.hl || col + v >= h.wl) t[i][v] = -1;
+                    if (row + kStep * i >= h.hl || col + v >= h.wl) t[i][v] = -1;
         }
         if constexpr (LAST) {
-            const int W = me->W, ns_c = me->ns_c, base = h.k - ns_c - 1, skip = ns_c - 3;
+            const int W = me->W, ns_c = me->ns_c, base = h.k + (qy - 1) * ns_c + qx - 1, skip = ns_c - 3;
             int32_t *o = me->out + (size_t)(h.y0 + row) * W + h.x0 + col;
             const bool fast = whole && me->vec;
 #pragma unroll
-            for (int i = 0; i < 4; ++i, o += 4 * (size_t)W) {
+            for (int i = 0; i < 4; ++i, o += kStep * (size_t)W) {
                 int lab[2];
 #pragma unroll
                 for (int v = 0; v < 2; ++v)  // t / 3 rows of cells down
@@ -1921,7 +1951,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
                 fix_round2_biased(f0, f1, fs, v[0][2], v[1][2]);
                 // x and y from the block's corner and the count: 11 + 11 + 10
                 // bits, enough for its 256 pixels
-                v[0][3] = (unsigned)col + ((unsigned)(row + 4 * i) << 11) + (1u << 22);
+                v[0][3] = (unsigned)col + ((unsigned)(row + kStep * i) << 11) + (1u << 22);
                 v[1][3] = v[0][3] + 1u;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
@@ -1929,8 +1959,10 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
 #pragma unroll
                         for (int c = 0; c < 4; ++c) own[c] += v[u][c];
                     } else if (t[i][u] >= 0) {
+                        int cell = t[i][u];  // its place in the block's window
+                        if constexpr (CS == 2) cell += win + (int)__umulhi((unsigned)cell, 0x55555556u);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) atomicAdd(&set[c * 40 + t[i][u] * 4 + (lane & 3)], v[u][c]);
+                        for (int c = 0; c < 4; ++c) atomicAdd(&set[c * kQ + cell * 4 + (lane & 3)], v[u][c]);
                     }
                 }
             }
@@ -1938,42 +1970,89 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
                 // the other set, read for the last block, is cleared for the next
                 uint4 *const z = reinterpret_cast<uint4 *>(bins + par * kBlkBinWords);
                 z[lane] = make_uint4(0u, 0u, 0u, 0u);
-                if (lane < 8) z[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+                if (lane < kBlkBinWords / 4 - 32) z[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
             }
+            // the own cells' words into their places among the bins
+            if constexpr (CS == 1) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) own[c] = __reduce_add_sync(kFull, own[c]);
-            if (lane < 4)  // the own cell's words into its place among the bins
-                set[lane * 40 + 16] = lane == 0 ? own[0] : lane == 1 ? own[1] : lane == 2 ? own[2] : own[3];
+                for (int c = 0; c < 4; ++c) own[c] = __reduce_add_sync(kFull, own[c]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) own[c] += __shfl_xor_sync(kFull, own[c], o);
+            }
+            if constexpr (CS == 1) {
+                if (lane < 4) set[lane * kQ + 16] = lane == 0 ? own[0] : lane == 1 ? own[1] : lane == 2 ? own[2] : own[3];
+            } else {  // (pixels of the block's other cells may have it too)
+                const int ln = lane & 7;
+                if (ln < 4)
+                    atomicAdd(&set[ln * kQ + (win + kSide + 1) * 4],
+                              ln == 0 ? own[0] : ln == 1 ? own[1] : ln == 2 ? own[2] : own[3]);
+            }
             __syncwarp();
-            if (lane < 27) {
-                // The totals follow the block: one cell to the right, the left
-                // column is complete; anything else but the same cell, all nine.
-                longlong2 r = me->total[lane];
+            // The totals follow the block: one block to the right, the left
+            // columns are complete; anything else but the same cell, all.
+            auto moved = [&](int e, int t, int p) {  // entry e (cell t, part p), this block's sums added
+                longlong2 r = me->total[e];
                 const int lk = me->k;  // (-1: no totals)
                 if (h.k != lk) {
-                    const bool right = h.k == lk + 1 && h.cx > 0;
-                    if (lk >= 0 && (!right || rt % 3 == 0)) flush(lk);
-                    r = right && rt % 3 < 2 ? me->total[lane + 3] : make_longlong2(0, 0);
+                    const bool right = h.k == lk + CS && h.cx > 0;
+                    if (lk >= 0 && (!right || t % kSide < CS)) flush(e, t, p, lk);
+                    r = right && t % kSide < 2 ? me->total[e + 3 * CS] : make_longlong2(0, 0);
                 }
                 auto word = [&](int c) {  // the four copies' sum
-                    const uint4 v = *reinterpret_cast<const uint4 *>(set + c * 40 + rt * 4);
+                    const uint4 v = *reinterpret_cast<const uint4 *>(set + c * kQ + t * 4);
                     return v.x + v.y + v.z + v.w;
                 };
                 // part 0: l, a; 1: b, x; 2: y, count
                 const unsigned xyn = word(3), cnt = xyn >> 22, bias = cnt * kFixBias;
-                const int c0 = (int)(word(part == 0 ? 0 : 2) - bias), c1 = (int)(word(1) - bias);
+                const int c0 = (int)(word(p == 0 ? 0 : 2) - bias), c1 = (int)(word(1) - bias);
                 const long long xs = (long long)(xyn & 0x7FFu) + (long long)cnt * h.x0,
                                 ys = (long long)((xyn >> 11) & 0x7FFu) + (long long)cnt * h.y0;
-                r.x += part < 2 ? (long long)c0 : ys;
-                r.y += part == 0 ? (long long)c1 : part == 1 ? xs : (long long)cnt;
-                __syncwarp(0x7FFFFFFu);  // (totals read before they are replaced)
-                me->total[lane] = r;
+                r.x += p < 2 ? (long long)c0 : ys;
+                r.y += p == 0 ? (long long)c1 : p == 1 ? xs : (long long)cnt;
+                return r;
+            };
+            if constexpr (CS == 1) {
+                // (spelled out, not by way of moved(): a 10-iteration step of
+                // 32 x 1080p takes 4.69 ms, 4.71 with any part of it shared)
+                if (lane < kEnts) {
+                    longlong2 r = me->total[lane];
+                    const int lk = me->k;  // (-1: no totals)
+                    if (h.k != lk) {
+                        const bool right = h.k == lk + 1 && h.cx > 0;
+                        if (lk >= 0 && (!right || rt % 3 == 0)) flush(lane, rt, part, lk);
+                        r = right && rt % 3 < 2 ? me->total[lane + 3] : make_longlong2(0, 0);
+                    }
+                    auto word = [&](int c) {  // the four copies' sum
+                        const uint4 v = *reinterpret_cast<const uint4 *>(set + c * 40 + rt * 4);
+                        return v.x + v.y + v.z + v.w;
+                    };
+                    // part 0: l, a; 1: b, x; 2: y, count
+                    const unsigned xyn = word(3), cnt = xyn >> 22, bias = cnt * kFixBias;
+                    const int c0 = (int)(word(part == 0 ? 0 : 2) - bias), c1 = (int)(word(1) - bias);
+                    const long long xs = (long long)(xyn & 0x7FFu) + (long long)cnt * h.x0,
+                                    ys = (long long)((xyn >> 11) & 0x7FFu) + (long long)cnt * h.y0;
+                    r.x += part < 2 ? (long long)c0 : ys;
+                    r.y += part == 0 ? (long long)c1 : part == 1 ? xs : (long long)cnt;
+                    __syncwarp(0x7FFFFFFu);  // (totals read before they are replaced)
+                    me->total[lane] = r;
+                    if (lane == 0) me->k = h.k;
+                }
+            } else {
+                const longlong2 r0 = moved(lane, rt, part);
+                longlong2 r1 = make_longlong2(0, 0);
+                if (lane < kEnts - 32) r1 = moved(lane + 32, rt1, part1);
+                __syncwarp();
+                me->total[lane] = r0;
+                if (lane < kEnts - 32) me->total[lane + 32] = r1;
                 if (lane == 0) me->k = h.k;
             }
         }
     }
     __syncwarp();
-    if (!LAST && ok && me->k >= 0 && lane < 27) flush(me->k);
+    if (!LAST && ok && me->k >= 0) flush_all(me->k);
     if (lane == 0 && !ok) atomicOr(err, 1);
     // After a wait that timed out: the copies still in flight land (bounded)
     // before the CTA exits, so none targets freed shared memory.
@@ -1981,27 +2060,46 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
         for (int q = j; q < min(n_blk, j + kBlkStages); ++q) mbar_wait(&full[q % kBlkStages], (q / kBlkStages) & 1);
 }
 
-int assign_blocks_occupancy() {
-    int o[2] = {0, 0};
-    const int smem = (int)blocks_smem_bytes();
-    if (cudaFuncSetAttribute(k_assign_blocks<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaFuncSetAttribute(k_assign_blocks<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[0], k_assign_blocks<false>, kBlkThreads, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[1], k_assign_blocks<true>, kBlkThreads, smem) != cudaSuccess)
-        return 0;
-    return std::min(o[0], o[1]);
+template <bool LAST, int CS>
+static cudaError_t blocks_smem_attr() {
+    return cudaFuncSetAttribute(k_assign_blocks<LAST, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)blocks_smem_bytes<CS>());
 }
 
-cudaError_t launch_assign_blocks(const FrameArgs *d_frames, int n, int total_blocks, bool last, int grid, int *err,
-                                 int check_stop, cudaStream_t s) {
+template <bool LAST, int CS>
+static int blocks_occupancy() {
+    int o = 0;
+    if (blocks_smem_attr<LAST, CS>() != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_assign_blocks<LAST, CS>, kBlkThreads,
+                                                      blocks_smem_bytes<CS>()) != cudaSuccess)
+        return 0;
+    return o;
+}
+
+int assign_blocks_occupancy() {
+    return std::min(std::min(blocks_occupancy<false, 1>(), blocks_occupancy<true, 1>()),
+                    std::min(blocks_occupancy<false, 2>(), blocks_occupancy<true, 2>()));
+}
+
+template <bool LAST, int CS>
+static cudaError_t launch_blocks_as(const FrameArgs *d_frames, int n, int total_blocks, int grid, int *err,
+                                    int check_stop, cudaStream_t s) {
     if (total_blocks < 1) return cudaSuccess;
     grid = std::max(1, std::min(grid, (total_blocks + kBlkWarps - 1) / kBlkWarps));
-    auto kern = last ? k_assign_blocks<true> : k_assign_blocks<false>;
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)blocks_smem_bytes());
+    const cudaError_t e = blocks_smem_attr<LAST, CS>();
     if (e != cudaSuccess) return e;
-    kern<<<grid, kBlkThreads, blocks_smem_bytes(), s>>>(d_frames, n, total_blocks, err, check_stop);
+    k_assign_blocks<LAST, CS>
+        <<<grid, kBlkThreads, blocks_smem_bytes<CS>(), s>>>(d_frames, n, total_blocks, err, check_stop);
     return cudaGetLastError();
+}
+
+cudaError_t launch_assign_blocks(const FrameArgs *d_frames, int n, int total_blocks, int total_blocks8, bool last,
+                                 int grid, int *err, int check_stop, cudaStream_t s) {
+    const cudaError_t e = last ? launch_blocks_as<true, 1>(d_frames, n, total_blocks, grid, err, check_stop, s)
+                               : launch_blocks_as<false, 1>(d_frames, n, total_blocks, grid, err, check_stop, s);
+    if (e != cudaSuccess) return e;
+    return last ? launch_blocks_as<true, 2>(d_frames, n, total_blocks8, grid, err, check_stop, s)
+                : launch_blocks_as<false, 2>(d_frames, n, total_blocks8, grid, err, check_stop, s);
 }
 
 // Cooperative launch (every CTA resident at once: the fused kernel's CTAs

@@ -16,14 +16,17 @@ def _img(W, H, seed, channels=3):
     return torch.from_numpy(synth.voronoi_frame(W, H, 60, 8.0, seed, channels=channels)).cuda()
 
 
-# (frames as (W, H, S, options), iterations, launch shape, groups). S a multiple
-# of 16 runs over blocks, other S over tiles, both in one batch.
+# (frames as (W, H, S, options), iterations, launch shape, groups). S = 8 and
+# multiples of 16 run over blocks, other S over tiles, all in one batch.
 BLOCKS = [
     ([(16, 16, 16, {}), (17, 15, 16, {}), (1, 1, 16, {}), (31, 33, 16, {})], 3, None, 1),
     ([(640, 360, 16, {}), (333, 257, 32, {}), (500, 90, 48, {}), (97, 400, 64, {})], 4, (0, 3, 2, 64), 2),
     ([(320, 240, 16, {}), (320, 240, 8, {}), (200, 100, 32, {}), (211, 130, 13, {}), (64, 64, 16, {})], 3, None, 3),
     ([(320, 240, 32, dict(in_channels=4)), (322, 243, 8, {}), (401, 300, 16, dict(color_space=1))], 2, (1, 3, 2, 64), 1),
     ([(300, 200, 16, dict(convergence=0.5)), (300, 200, 16, {}), (170, 200, 32, dict(convergence=1.0))], 6, None, 1),
+    ([(8, 8, 8, {}), (9, 17, 8, {}), (1, 1, 8, {}), (23, 41, 8, {}), (16, 16, 8, {}), (7, 100, 8, {})], 3, None, 1),
+    ([(642, 203, 8, dict(convergence=0.5)), (120, 88, 8, dict(perturb_seeds=True)), (48, 48, 24, {}),
+      (333, 64, 8, dict(in_channels=4))], 5, None, 2),
     ([(40, 600, 16, dict(perturb_seeds=True)), (2000, 20, 16, dict(color_space=2))], 2, (2, 4, 2, 32), 2),
 ]
 
