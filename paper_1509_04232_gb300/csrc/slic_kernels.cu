@@ -2620,6 +2620,19 @@ __device__ __forceinline__ int ccl_find_s(int *par, int i, int *err) {
     atomicOr(err, 2);
     return i;
 }
+// The root of i without a store, for a stage in which every entry has an owner
+// that writes its root.
+__device__ __forceinline__ int ccl_root_s(const int *par, int i, int *err) {
+    const volatile int *vp = par;
+    const unsigned lim = g_ccl_steps;
+    for (unsigned n = 0; n < lim; ++n) {
+        const int p = vp[i];
+        if (p == i) return i;
+        i = p;
+    }
+    atomicOr(err, 2);
+    return i;
+}
 __device__ __forceinline__ void ccl_union_s(int *par, int a, int b, int *err) {
     const unsigned lim = g_ccl_steps;
     for (unsigned n = 0; n < lim; ++n) {
@@ -2744,12 +2757,13 @@ __global__ void __launch_bounds__(kCclThreads) k_ccl_local(CclFrames fr, int *pa
         if (more & 1u) ccl_union_s(par, ly * kCclTile + lane, (ly - 1) * kCclTile + lane, err);
     __syncthreads();
     halve(2);
-    // What is left of a longer chain is walked. Each run's first pixel adds the
-    // run's length to its root's size.
+    // What is left of a longer chain is walked, without halving: a walk that
+    // stored a grandparent could overwrite the root that the entry's owner had
+    // stored meanwhile, and that pixel's parent would then be no root. Each
+    // run's first pixel adds the run's length to its root's size.
     for (int ly = warp; ly < th; ly += kRowsPerPass) {
         const int i = ly * kCclTile + lane;
-        int r = vp[i];
-        if (vp[r] != r) r = ccl_find_s(par, r, err);
+        const int r = ccl_root_s(par, vp[i], err);
         const int32_t v = lab[i];
         const bool start = col_ok && (lane == 0 || lab[i - 1] != v);
         const unsigned st = __ballot_sync(kFull, start);

@@ -250,6 +250,42 @@ def test_components_stage_matches_oracle(slic_gpu, W, H, S, kind):
     assert got.max() == n - 1
 
 
+def _winding(H, W, kind, seed):
+    """Label maps whose segments wind through a tile: long chains of links."""
+    y, x = np.mgrid[0:H, 0:W]
+    if kind == "snake":      # one path per label, down a column and up the next
+        lab = np.where(x % 2 == 0, 0, 1 + (x // 2) % 2)
+        lab[(y % 32 == np.where(x // 2 % 2 == 0, 31, 0)) & (x % 2 == 1)] = 0
+    elif kind == "spiral":   # nested square rings of each 32x32 tile, cut open at one corner
+        ring = np.minimum(np.minimum(x % 32, 31 - x % 32), np.minimum(y % 32, 31 - y % 32))
+        lab = ring % 2
+        lab[(ring % 2 == 1) & (y % 32 == ring) & (x % 32 == ring + 1)] = 0
+    elif kind == "comb":     # teeth joined at the bottom of a tile
+        lab = np.where((x % 2 == 0) | (y % 32 >= 30), 0, 1 + x // 2 % 3)
+    elif kind == "stairs":   # one-pixel diagonal steps, each row a run of its own
+        lab = (x + y) // 2 % 3
+    else:
+        lab = np.random.default_rng(seed).integers(0, 2, (H, W))
+    return np.ascontiguousarray(lab.astype(np.int32))
+
+
+@pytest.mark.parametrize("kind", ["snake", "spiral", "comb", "stairs", "noise"])
+@pytest.mark.parametrize("W,H", [(32, 32), (96, 64), (333, 127)])
+def test_components_of_winding_segments(slic_gpu, W, H, kind):
+    """Winding segments leave chains of links for the tile stage's last walk,
+    which runs beside the stores of the roots: equal to the oracle, and the
+    same on every repetition."""
+    lab = _winding(H, W, kind, W + H)
+    S = 4
+    seg = slic_gpu.Segmenter(W, H, S=S, enforce_connectivity=2)
+    want, _ = oracle.connectivity_components(lab, S * S // 4)
+    dev = _t(lab)
+    for _ in range(50):
+        got = _np(seg.connectivity_components(dev))
+        np.testing.assert_array_equal(got, want)
+    seg.status()
+
+
 def test_components_whole_run_and_paths(slic_gpu):
     """A whole run in mode 2 equals the oracle's relabelling of the same
     run's pre-connectivity labels; the batch and the allocation-free paths
