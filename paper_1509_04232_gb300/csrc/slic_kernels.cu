@@ -1828,6 +1828,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2)
             continue;
         }
         if (h.f != me->f) {  // (all lanes read it before lane 0 writes)
+            __syncwarp();    // (lane 0's store to me->k for the last block; the vote above orders no memory)
             if (!LAST && me->k >= 0) flush_all(me->k);
             __syncwarp();
             if (lane == 0) {

@@ -54,6 +54,25 @@ def test_blocks_equal_launch_per_stage(slic_gpu, frames, iterations, shape, grou
         assert ran[k] == seg.iterations_run
 
 
+def test_blocks_of_many_frames_per_warp(slic_gpu):
+    """Hundreds of small frames: a warp's run of blocks crosses from frame to
+    frame, where its totals go out and its state changes. Every copy of a frame
+    is bit-identical to the single frame, on every repetition."""
+    import torch
+    kinds = [(48, 48, 16), (70, 33, 16), (40, 24, 8), (17, 90, 8), (96, 40, 32), (16, 16, 16)]
+    n = 600
+    imgs = [_img(W, H, 900 + k) for k, (W, H, _) in enumerate(kinds)]
+    want = [slic_gpu.Segmenter(W, H, S=S, iterations=3).segment(imgs[k]) for k, (W, H, S) in enumerate(kinds)]
+    of = [f % len(kinds) for f in range(n)]
+    bs = slic_gpu.BatchSegmenter([dict(width=kinds[k][0], height=kinds[k][1], S=kinds[k][2]) for k in of], iterations=3)
+    bs.bind([imgs[k] for k in of])
+    for _ in range(5):
+        labels, centres = bs.segment()
+        bs.status()
+        for f, k in enumerate(of):
+            assert torch.equal(labels[f], want[k][0]) and torch.equal(centres[f], want[k][1]), f
+
+
 @pytest.mark.parametrize("W,H,S,kind", [(64, 8, 8, "noise"), (65, 9, 4, "noise"), (130, 70, 16, "blocks"),
                                         (333, 57, 13, "slots"), (3, 2, 2, "noise"), (256, 128, 2, "noise")])
 def test_label_sums(slic_gpu, W, H, S, kind):
