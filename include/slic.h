@@ -144,7 +144,10 @@ slic_status slic_iterations_run(slic_handle h, int *out);
 
 /* Use d_init [K_eff][6] (e.g. the previous video frame's centres) instead of
    the grid initialisation on the next slic_segment call. The buffer is read
-   when that call's work runs. Pass NULL to disarm. */
+   when that call's work runs. Pass NULL to disarm. Values beyond 1e17, and
+   NaN, take part in the distances as +-1e17 (NaN as -1e17), so that every
+   pixel gets a label of the grid; a centre that no pixel chose is returned as
+   it was given. */
 slic_status slic_set_init_centres(slic_handle h, const float *d_init);
 
 /* Sec. 3 "Image space conversion" only: d_features float [3][height][width]. */

@@ -165,7 +165,7 @@ FrameArgs frame_args(slic_ctx *h, const uint8_t *rgb, float *feat, int P, const 
     a.S = h->S;
     a.ns_c = h->ns_c;
     a.ns_r = h->ns_r;
-    a.w = h->p.m / (float)h->S;
+    a.w = spatial_weight(h->p.m, h->S);
     a.s_mul = h->S <= 2048 ? (unsigned)((0x100000000ULL + (unsigned)h->S - 1) / (unsigned)h->S) : 0u;
     a.tiles_x = (h->p.width + kTileW - 1) / kTileW;
     a.win_max = assign_max_window(h->S, h->ns_c, h->ns_r);
@@ -715,7 +715,7 @@ extern "C" slic_status slic_segment_noalloc(const slic_params *params, const uin
     a.S = S;
     a.ns_c = ns_c;
     a.ns_r = ns_r;
-    a.w = p.m / (float)S;
+    a.w = spatial_weight(p.m, S);
     a.win_max = win;
     a.direct_acc = assign_direct_acc(win) ? 1 : 0;
     a.rgb_vec = ((p.width & 3) == 0 && ((uintptr_t)d_image & 15) == 0) ? 1 : 0;

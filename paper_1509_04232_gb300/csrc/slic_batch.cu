@@ -394,7 +394,7 @@ slic_status slic_batch_create(const slic_params *params, int n_frames, slic_batc
         a.S = S;
         a.ns_c = (p.width + S - 1) / S;
         a.ns_r = (p.height + S - 1) / S;
-        a.w = p.m / (float)S;
+        a.w = spatial_weight(p.m, S);
         a.fix_scale = p.color_space == SLIC_RGB ? 1.0f : kFixScaleFrac;
         a.s_mul = S <= 2048 ? (unsigned)((0x100000000ULL + (unsigned)S - 1) / (unsigned)S) : 0u;
         a.tiles_x = (p.width + kTileW - 1) / kTileW;

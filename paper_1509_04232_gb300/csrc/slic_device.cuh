@@ -14,12 +14,29 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
+// Cells off the grid have a sentinel centre, kSentinel in every coordinate, so
+// that the candidate loops need no bounds checks. It has to lose to every centre
+// of the grid: a pixel that chose it would count in a cell that does not exist.
+// A centre that the caller gives may be anything, NaN included, so its record
+// holds it within +-kFarCentre (NaN: -kFarCentre), and the weight of the spatial
+// distance is at most kMaxWeight: every D is then finite, and the sentinels'
+// ten times any other. (Outputs keep the values that the caller gave.)
+constexpr float kSentinel = 1e18f, kFarCentre = 1e17f;
+__device__ __forceinline__ float near_centre(float v) { return fminf(fmaxf(v, -kFarCentre), kFarCentre); }
+
 // One record of the padded centre table: each field twice (see kCtabRec).
 __device__ __forceinline__ void write_ctab(float *t, const float *c) {
     float4 *t4 = reinterpret_cast<float4 *>(t);
     t4[0] = make_float4(c[0], c[0], c[1], c[1]);
     t4[1] = make_float4(c[2], c[2], c[3], c[3]);
     t4[2] = make_float4(c[4], c[4], c[5], 0.0f);
+}
+// The record of a centre that may be the caller's.
+__device__ __forceinline__ void write_ctab_near(float *t, const float *c) {
+    float n[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) n[i] = i < 5 ? near_centre(c[i]) : c[i];
+    write_ctab(t, n);
 }
 
 // Candidate tags 0..8 (scan position in the 3x3 window) for the keys

@@ -140,11 +140,14 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
     // Initial centres of the window.
     for (int e = tid; e <= sent; e += kFrThreads) {
         const int seg = e / win, j = e - seg * win, k = k0 + (seg - 1) * ns_c - 1 + j;
-        float rec[6] = {1e18f, 1e18f, 1e18f, 1e18f, 1e18f, 0.0f};
+        float rec[6] = {kSentinel, kSentinel, kSentinel, kSentinel, kSentinel, 0.0f};
         if (e < sent && j < nk + 2 && k >= 0 && k < K) {
             if (a.init) {
 #pragma unroll
-                for (int i = 0; i < 6; ++i) rec[i] = a.init[(size_t)k * 6 + i];
+                for (int i = 0; i < 6; ++i) {
+                    const float v = a.init[(size_t)k * 6 + i];
+                    rec[i] = i < 5 ? near_centre(v) : v;
+                }
             } else {
                 int px, py;
                 init_centre_position(k, W, H, S, ns_c, rec[3], rec[4], px, py);
@@ -471,7 +474,9 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
         // The centres the labels were assigned against.
         for (int i = tid; i < (ko1 - ko0) * 6; i += kFrThreads) {
             const int k = ko0 + i / 6, q = i % 6;
-            a.centres[(size_t)k * 6 + q] = ctab[(size_t)(win + k - k0 + 1) * kCtabRec + 2 * q];
+            float v = ctab[(size_t)(win + k - k0 + 1) * kCtabRec + 2 * q];
+            if (fabsf(v) == kFarCentre && a.init) v = a.init[(size_t)k * 6 + q];  // (held there: as it was given)
+            a.centres[(size_t)k * 6 + q] = v;
         }
         if (a.connect) {
             arrive();

@@ -108,6 +108,16 @@ struct ConvState {
 };
 constexpr float kResidScale = 65536.0f;
 
+// The weight m / S of the spatial distance in Eq. (1). Above kMaxWeight D would
+// overflow (see kSentinel). No colour distance counts at all there, so halving
+// the weight scales every D exactly and changes no comparison.
+constexpr float kMaxWeight = 73786976294838206464.0f;  // 2^66
+inline float spatial_weight(float m, int S) {
+    float w = m / (float)S;
+    while (w > kMaxWeight) w *= 0.5f;
+    return w;
+}
+
 // One frame's geometry and buffers as seen by the kernels (a kernel
 // parameter for single-frame launches, an entry of a device-side table for
 // batched ones).

@@ -31,7 +31,6 @@ __device__ float g_lut[256];  // sRGB byte -> linear, filled by the host
 namespace {
 
 constexpr int kWarps = kThreads / 32;
-constexpr float kSentinel = 1e18f;
 constexpr size_t kPrivateAccLimit = 64 * 1024;
 
 
@@ -158,7 +157,7 @@ __global__ void k_init_batch(const FrameArgs *frames, int n, int total) {
     if (k == 0) reset_conv(a.cstate);
     if (a.ctab) {
         const int r = k / a.ns_c, c = k - (k / a.ns_c) * a.ns_c;
-        write_ctab(a.ctab + ((size_t)(r + 1) * (a.ns_c + 2) + c + 1) * kCtabRec, a.centres_out + (size_t)k * 6);
+        write_ctab_near(a.ctab + ((size_t)(r + 1) * (a.ns_c + 2) + c + 1) * kCtabRec, a.centres_out + (size_t)k * 6);
     }
 }
 
@@ -176,7 +175,7 @@ __global__ void k_fill_ring(const FrameArgs *frames, int n, int max_ring) {
         else { const int j = i - 2 * cw; r = 1 + (j >> 1); c = (j & 1) ? cw - 1 : 0; }
         float4 *t = reinterpret_cast<float4 *>(a.ctab + ((size_t)r * cw + c) * kCtabRec);
 #pragma unroll
-        for (int q = 0; q < kCtabRec / 4; ++q) t[q] = make_float4(1e18f, 1e18f, 1e18f, 1e18f);
+        for (int q = 0; q < kCtabRec / 4; ++q) t[q] = make_float4(kSentinel, kSentinel, kSentinel, kSentinel);
     }
 }
 
@@ -362,16 +361,16 @@ __device__ __forceinline__ void assign_tile(const FrameArgs &fa, int tx0, int ty
         }
     }
 
-    // Out-of-grid window cells hold a sentinel centre whose D is ~1e18, so
-    // the candidate loop needs no bounds checks (the own cell is always
-    // valid and always beats it).
+    // Out-of-grid window cells hold a sentinel centre (kSentinel), so the
+    // candidate loop needs no bounds checks (the own cell is always valid and
+    // always beats it).
     for (int i = tid; i < nwin; i += kThreads) {
         const int qy = i / wnx;
         const int cy = wy0 + qy, cx = wx0 + i - qy * wnx;
         if (cx >= 0 && cx < ns_c && cy >= 0 && cy < ns_r) {
             const float *ck = fa.centres + ((size_t)cy * ns_c + cx) * 6;
-            cA[i] = make_float4(ck[0], ck[1], ck[2], ck[3]);
-            cY[i] = ck[4];
+            cA[i] = make_float4(near_centre(ck[0]), near_centre(ck[1]), near_centre(ck[2]), near_centre(ck[3]));
+            cY[i] = near_centre(ck[4]);
         } else {
             cA[i] = make_float4(kSentinel, kSentinel, kSentinel, kSentinel);
             cY[i] = kSentinel;
@@ -889,7 +888,8 @@ __device__ __forceinline__ float update_centre(long long *ak, const float *ci, f
     float move = 0.0f;
     if (n > 0) {
         const float fn = (float)n;
-        const float x0 = want_move ? __ldcg(ci + 3) : 0.0f, y0 = want_move ? __ldcg(ci + 4) : 0.0f;
+        const float x0 = want_move ? near_centre(__ldcg(ci + 3)) : 0.0f,
+                    y0 = want_move ? near_centre(__ldcg(ci + 4)) : 0.0f;
         co[0] = __fdiv_rn((float)s01.x * fix_inv, fn);
         co[1] = __fdiv_rn((float)s01.y * fix_inv, fn);
         co[2] = __fdiv_rn((float)s23.x * fix_inv, fn);
@@ -984,7 +984,7 @@ __device__ __forceinline__ void update_chunk(const FrameArgs &a, int c0, int cn,
                 move = update_centre(a.acc + k, a.centres_out + k, a.centres_out + k, 1.0f / a.fix_scale,
                                      a.conv_eps > 0.0f);
                 const int r = kk / a.ns_c, c = kk - r * a.ns_c;
-                write_ctab(a.ctab + ((size_t)(r + 1) * (a.ns_c + 2) + c + 1) * kCtabRec, a.centres_out + k);
+                write_ctab_near(a.ctab + ((size_t)(r + 1) * (a.ns_c + 2) + c + 1) * kCtabRec, a.centres_out + k);
             }
         }
         // (a frame stops for all its centres: a warp of valid lanes is all
@@ -2204,7 +2204,7 @@ __global__ void k_update_batch(const FrameArgs *frames, int n, int total, int it
                                  a.conv_eps > 0.0f);
             if (a.ctab) {
                 const int r = kk / a.ns_c, c = kk - r * a.ns_c;
-                write_ctab(a.ctab + ((size_t)(r + 1) * (a.ns_c + 2) + c + 1) * kCtabRec, a.centres_out + k);
+                write_ctab_near(a.ctab + ((size_t)(r + 1) * (a.ns_c + 2) + c + 1) * kCtabRec, a.centres_out + k);
             }
         }
     }

@@ -73,6 +73,70 @@ def test_blocks_of_many_frames_per_warp(slic_gpu):
             assert torch.equal(labels[f], want[k][0]) and torch.equal(centres[f], want[k][1]), f
 
 
+def _start_centres(seg, kind):
+    """Initial centres that the grid's sentinel centres (1e18) can beat: all of
+    them, or those around the first and the last cell."""
+    import torch
+    value = dict(nan=float("nan"), inf=float("inf"), far=3e18, overflow=1e30, corner=float("nan"))[kind]
+    c = torch.rand(seg.K_eff, 6, device="cuda") * 20
+    if kind != "corner":
+        c[:] = value
+    else:
+        g = c.view(seg.ns_r, seg.ns_c, 6)
+        g[:2, :2] = value
+        g[-2:, -2:] = value
+    return c
+
+
+@pytest.mark.parametrize("kind", ["nan", "inf", "far", "overflow", "corner", "m"])
+def test_labels_and_sums_stay_in_the_grid(slic_gpu, kind):
+    """Centres from the caller that are not finite or further off than the
+    sentinels around the grid, and an m whose distances would overflow: every
+    path gives every pixel a label of the grid, counts every pixel once, leaves
+    a neighbouring frame of the batch alone, and agrees with the others."""
+    import torch
+    geo = [(100, 61, 16), (75, 50, 8), (90, 70, 13), (121, 96, 24), (64, 48, 32), (50, 33, 3), (130, 40, 40)]
+    m = 3e38 if kind == "m" else 10.0
+    imgs = [_img(W, H, 40 + k) for k, (W, H, _) in enumerate(geo)]
+    for iterations in (0, 1):
+        kw = dict(m=m, iterations=iterations, enforce_connectivity=0)
+        want, start = [], []
+        for (W, H, S), img in zip(geo, imgs):
+            one = slic_gpu.Segmenter(W, H, S=S, **kw)
+            per = slic_gpu.Segmenter(W, H, S=S, **kw)
+            slic_gpu.slic_profile_enable(per.handle, True)  # (a launch per stage)
+            init = None if kind == "m" else _start_centres(per, kind)
+            l, c = per.segment(img, init_centres=init)
+            assert int(l.min()) >= 0 and int(l.max()) < per.K_eff
+            if iterations:
+                assert int(c[:, 5].sum()) == W * H
+            l1, c1 = one.segment(img, init_centres=init)
+            assert torch.equal(l1, l) and torch.equal(c1.view(torch.int32), c.view(torch.int32))
+            want.append((l, c))
+            start.append(init)
+        ordinary = slic_gpu.Segmenter(80, 48, S=16, iterations=iterations, enforce_connectivity=0)
+        good = _img(80, 48, 7)
+        want_good = ordinary.segment(good)
+        for shape in ([0], [1, 2, 0], [3, 4], [3], [6], [5, 2]):  # blocks, tiles, two row groups, small S
+            frames, ims, inits, refs = [], [], [], []
+            for k in shape:
+                frames += [dict(width=80, height=48, S=16), dict(width=geo[k][0], height=geo[k][1], S=geo[k][2], m=m)]
+                ims += [good, imgs[k]]
+                inits += [None, start[k]]
+                refs += [want_good, want[k]]
+            bs = slic_gpu.BatchSegmenter(frames, iterations=iterations, enforce_connectivity=0)
+            bs.bind(ims, init_centres=inits)
+            same8 = all(f["S"] % 8 == 0 for f in frames)
+            for tune, fused in ([((0, 3, 1, 32), False), ((0, 3, 1, 32), True)] +
+                                ([((0, 3, 2, 32), False), ((0, 3, 2, 64), False), ((0, 3, 2, 64), True)] if same8 else [])):
+                bs.set_tuning(*tune, fused=fused)
+                labels, centres = bs.segment()
+                bs.status()
+                for f, (l, c) in enumerate(refs):
+                    assert torch.equal(labels[f], l), (shape, tune, fused, f)
+                    assert torch.equal(centres[f].view(torch.int32), c.view(torch.int32)), (shape, tune, fused, f)
+
+
 @pytest.mark.parametrize("W,H,S,kind", [(64, 8, 8, "noise"), (65, 9, 4, "noise"), (130, 70, 16, "blocks"),
                                         (333, 57, 13, "slots"), (3, 2, 2, "noise"), (256, 128, 2, "noise")])
 def test_label_sums(slic_gpu, W, H, S, kind):
