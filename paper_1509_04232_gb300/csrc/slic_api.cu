@@ -29,7 +29,7 @@ struct slic_ctx {
     int32_t *lbl_tmp = nullptr;   // [H][W] connectivity ping-pong
     ConvState *cstate = nullptr;  // stopping-test state of the current run
     int *ccl = nullptr;           // component connectivity scratch (mode 2), and its error flag
-    int *ccl_err = nullptr;       // [0] the flag, [1..2] the barrier counters of the one-launch path
+    int *ccl_err = nullptr;       // [0] the flag, [1] the barrier counter of the one-launch path
     ResidentPlan plan{};          // the one-launch path (grid 0: not for this geometry)
     float fix_scale = 0.0f;
     size_t smem_max = 0;
@@ -307,8 +307,8 @@ slic_status slic_create(const slic_params *params, slic_handle *out) {
         dev_alloc(&h->acc, sizeof(long long) * 6 * (size_t)h->K) != cudaSuccess ||
         dev_alloc(&h->lbl_tmp, sizeof(int32_t) * npix) != cudaSuccess ||
         dev_alloc(&h->cstate, sizeof(ConvState)) != cudaSuccess ||
-        cudaMemset(h->cstate, 0, sizeof(ConvState)) != cudaSuccess || dev_alloc(&h->ccl_err, 3 * sizeof(int)) != cudaSuccess ||
-        cudaMemset(h->ccl_err, 0, 3 * sizeof(int)) != cudaSuccess ||
+        cudaMemset(h->cstate, 0, sizeof(ConvState)) != cudaSuccess || dev_alloc(&h->ccl_err, 2 * sizeof(int)) != cudaSuccess ||
+        cudaMemset(h->ccl_err, 0, 2 * sizeof(int)) != cudaSuccess ||
         (p.enforce_connectivity == 2 && dev_alloc(&h->ccl, sizeof(int) * ccl_scratch_ints((long long)npix)) != cudaSuccess)) {
         cudaGetLastError();
         cudaFree(h->feat);
@@ -738,13 +738,9 @@ extern "C" slic_status slic_segment_noalloc(const slic_params *params, const uin
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         plan_resident(p.width, p.height, S, ns_c, ns_r, sms, feat_b, &plan)) {
         int *const words = reinterpret_cast<int *>(ctrl);
-        // (calls that overlapped against the rules may have left the barrier
-        // counters of the shared array anywhere)
-        e = cudaMemsetAsync(words + 1, 0, 2 * sizeof(int), s);
-        if (e == cudaSuccess)
-            e = launch_resident(resident_args(a, p.iterations, p.enforce_connectivity == 1, lbl_tmp,
-                                              reinterpret_cast<long long *>(base), words + 1, words),
-                                plan, s);
+        e = launch_resident(resident_args(a, p.iterations, p.enforce_connectivity == 1, lbl_tmp,
+                                          reinterpret_cast<long long *>(base), words + 1, words),
+                            plan, s);
         done = e == cudaSuccess;
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             cudaGetLastError();

@@ -297,7 +297,7 @@ struct ResidentFrame {
     int32_t *labels, *lbl_tmp;
     long long *acc;         // three sets of [K][6] sums
     ConvState *cstate;
-    int *ctrl;              // two barrier counters, zero before the first launch
+    int *ctrl;              // the barrier counter
     int *err;               // bit 4: a barrier gave up
     int W, H, C, S, ns_c, ns_r, K, iterations, perturb, connect, labels_vec, labels_vec2;
     float w, fix_scale, eps;

@@ -79,3 +79,48 @@ def test_one_launch_replays_in_a_graph_and_in_place(slic_gpu):
     want = seg.segment(img, init_centres=start)
     got = seg.segment(img, centres=centres, init_centres=centres)
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+def _captured_nodes(call, stream):
+    """Node types of the graph that `call` is captured into on `stream`, and the graph's launch."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+    graph, n = ctypes.c_void_p(), ctypes.c_size_t()
+    ok = lambda r: r == 0 or pytest.fail(f"driver call failed: {r}")  # noqa: E731
+    s = ctypes.c_void_p(stream.cuda_stream)
+    ok(cu.cuStreamBeginCapture_v2(s, 1))  # (thread-local mode)
+    call()
+    ok(cu.cuStreamEndCapture(s, ctypes.byref(graph)))
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    kinds = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        kinds.append(kind.value)
+    ok(cu.cuGraphDestroy(graph))
+    return kinds
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_the_barrier_counter_is_cleared_for_every_launch(slic_gpu, noalloc):
+    """A call of either entry point is the clear of the barrier counter and the
+    one kernel: no launch relies on what the one before it has left."""
+    import torch
+    kernel, memset = 0, 2  # CU_GRAPH_NODE_TYPE_KERNEL, CU_GRAPH_NODE_TYPE_MEMSET
+    img = _frame(320, 240, 3, 5)
+    seg = slic_gpu.Segmenter(320, 240, S=16, iterations=3)
+    want = seg.segment(img)
+    labels, centres = torch.empty_like(want[0]), torch.empty_like(want[1])
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    if noalloc:
+        run = lambda: slic_gpu.slic_segment_noalloc(seg.params, img.data_ptr(), labels.data_ptr(),  # noqa: E731
+                                                    centres.data_ptr(), stream.cuda_stream)
+    else:
+        run = lambda: seg.segment(img, labels, centres, stream=stream)  # noqa: E731
+    run()
+    torch.cuda.synchronize()
+    assert torch.equal(labels, want[0]) and torch.equal(centres, want[1])
+    assert sorted(_captured_nodes(run, stream)) == [kernel, memset]
