@@ -414,12 +414,19 @@ slic_status slic_noalloc_status_check(void);
                               out after about a second per launch and
                               slic_batch_status reports SLIC_ERR_TIMEOUT.
                               0 clears.
-   The device words apply to the current device. SLIC_ERR_INVALID for an
+     SLIC_FAULT_BARRIER_LIMIT the grid barrier of the one-launch segmentation
+                              gives up after `value` polls instead of 2^22 (0
+                              restores it): every CTA then leaves, and
+                              slic_status_check or slic_noalloc_status_check
+                              reports SLIC_ERR_TIMEOUT. Applies to launches
+                              enqueued from now on.
+   The device words (walk limit, copies) apply to the current device. SLIC_ERR_INVALID for an
    unknown kind or a negative value. */
 typedef enum {
     SLIC_FAULT_ALLOC = 1,
     SLIC_FAULT_WALK_LIMIT = 2,
-    SLIC_FAULT_ABORT_COPIES = 3
+    SLIC_FAULT_ABORT_COPIES = 3,
+    SLIC_FAULT_BARRIER_LIMIT = 4
 } slic_fault;
 slic_status slic_fault_inject(int kind, long long value);
 

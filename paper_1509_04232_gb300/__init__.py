@@ -11,6 +11,7 @@ from __future__ import annotations
 
 from ._binding import (SLIC_CIELAB, SLIC_ERR_CUDA, SLIC_ERR_INVALID, SLIC_ERR_NOMEM,  # noqa: F401
                        SLIC_ERR_STATE, SLIC_ERR_TIMEOUT, SLIC_FAULT_ABORT_COPIES, SLIC_FAULT_ALLOC,
+                       SLIC_FAULT_BARRIER_LIMIT,
                        SLIC_FAULT_WALK_LIMIT, SLIC_OK, SLIC_RGB, SLIC_XYZ, SlicError, library_path, slic_assign,
                        slic_fault_inject, slic_noalloc_status_check,
                        slic_batch_autotune, slic_batch_create, slic_batch_destroy, slic_batch_info,

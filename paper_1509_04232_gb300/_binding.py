@@ -16,7 +16,7 @@ from . import build as _build
 
 SLIC_OK, SLIC_ERR_INVALID, SLIC_ERR_NOMEM, SLIC_ERR_CUDA, SLIC_ERR_TIMEOUT, SLIC_ERR_STATE = 0, -1, -2, -3, -4, -5
 SLIC_CIELAB, SLIC_RGB, SLIC_XYZ = 0, 1, 2
-SLIC_FAULT_ALLOC, SLIC_FAULT_WALK_LIMIT, SLIC_FAULT_ABORT_COPIES = 1, 2, 3
+SLIC_FAULT_ALLOC, SLIC_FAULT_WALK_LIMIT, SLIC_FAULT_ABORT_COPIES, SLIC_FAULT_BARRIER_LIMIT = 1, 2, 3, 4
 
 _STATUS_NAMES = {0: "SLIC_OK", -1: "SLIC_ERR_INVALID", -2: "SLIC_ERR_NOMEM", -3: "SLIC_ERR_CUDA",
                  -4: "SLIC_ERR_TIMEOUT", -5: "SLIC_ERR_STATE"}

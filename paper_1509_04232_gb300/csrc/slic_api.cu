@@ -177,6 +177,11 @@ FrameArgs frame_args(slic_ctx *h, const uint8_t *rgb, float *feat, int P, const 
     return a;
 }
 
+// Polls of the one-launch path's grid barrier, over a second by default
+// (lowered only by fault injection, to make the barrier give up in tests).
+constexpr unsigned kBarrierPolls = 1u << 22;
+std::atomic<unsigned> g_barrier_polls{kBarrierPolls};
+
 // The same frame for the one-launch path.
 ResidentFrame resident_args(const FrameArgs &a, int iterations, bool connect, int32_t *lbl_tmp, long long *acc,
                             int *ctrl, int *err) {
@@ -190,6 +195,7 @@ ResidentFrame resident_args(const FrameArgs &a, int iterations, bool connect, in
     r.cstate = a.cstate;
     r.ctrl = ctrl;
     r.err = err;
+    r.polls = g_barrier_polls.load();
     r.W = a.W;
     r.H = a.H;
     r.C = a.C;
@@ -599,6 +605,10 @@ slic_status slic_fault_inject(int kind, long long value) {
     case SLIC_FAULT_ABORT_COPIES:
         abort_copies = value != 0;
         break;
+    case SLIC_FAULT_BARRIER_LIMIT:
+        if (value > (long long)kBarrierPolls) return fail(nullptr, SLIC_ERR_INVALID, "barrier limit above the default");
+        g_barrier_polls.store(value ? (unsigned)value : kBarrierPolls);
+        return SLIC_OK;
     default:
         return fail(nullptr, SLIC_ERR_INVALID, "unknown fault kind");
     }

@@ -37,7 +37,6 @@ constexpr int kFrWarps = kFrThreads / 32;
 // mostly pick the same candidate, and with one copy an atomic instruction
 // took 8 passes over shared memory (ncu), a quarter of the launch.
 constexpr int kFrBinWords = 160;
-constexpr unsigned kFrPolls = 1u << 22;     // of the grid barrier: over a second
 constexpr int kFrMaxSmem = 227 * 1024;
 
 // A unit's first pixel and extent (wl x hl pixels, clipped to its cell and the
@@ -94,9 +93,9 @@ __global__ void __launch_bounds__(kFrThreads, 1) k_frame(const __grid_constant__
         if (tid == 0) {
             const int target = barriers * G;
             unsigned n = 0;
-            while (ld_acquire(a.ctrl) < target && ++n < kFrPolls) {
+            while (ld_acquire(a.ctrl) < target && ++n < a.polls) {
             }
-            ok = n < kFrPolls;
+            ok = n < a.polls;
             if (!ok) atomicOr(a.err, 4);
         }
         return __syncthreads_and(ok ? 1 : 0) != 0;

@@ -299,6 +299,7 @@ struct ResidentFrame {
     ConvState *cstate;
     int *ctrl;              // the barrier counter
     int *err;               // bit 4: a barrier gave up
+    unsigned polls;         // its limit
     int W, H, C, S, ns_c, ns_r, K, iterations, perturb, connect, labels_vec, labels_vec2;
     float w, fix_scale, eps;
     int units, max_units, win, cw, uh, ncx, ncy, ppr, conn_rows;  // (from the plan)

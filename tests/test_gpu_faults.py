@@ -137,6 +137,78 @@ def test_fused_passes_timeout_is_reported(slic_gpu):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("noalloc", [False, True])
+@pytest.mark.parametrize("kw", [dict(iterations=0), dict(iterations=4), dict(iterations=2, enforce_connectivity=0),
+                                dict(iterations=3, convergence=0.1, enforce_connectivity=2)])
+def test_one_launch_barrier_timeout_is_reported(slic_gpu, kw, noalloc):
+    """The grid barrier of the one-launch segmentation gives up after one poll:
+    every CTA leaves (those that arrived last go on to a later barrier first),
+    SLIC_ERR_TIMEOUT is reported once, and the next call is exact."""
+    import torch
+    pkg = slic_gpu
+    W, H = 320, 240
+    img = _img(W, H, 70)
+    seg = pkg.Segmenter(W, H, S=16, **kw)
+    want = seg.segment(img)
+    seg.status()
+    labels, centres = torch.empty_like(want[0]), torch.empty_like(want[1])
+
+    def run():
+        if noalloc:
+            pkg.slic_segment_noalloc(seg.params, img.data_ptr(), labels.data_ptr(), centres.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+        else:
+            seg.segment(img, labels, centres)
+
+    check = pkg.slic_noalloc_status_check if noalloc else seg.status
+    check()
+    try:
+        pkg.slic_fault_inject(pkg.SLIC_FAULT_BARRIER_LIMIT, 1)
+        for _ in range(3):
+            run()
+        with pytest.raises(pkg.SlicError) as ei:
+            check()
+        assert ei.value.status == pkg.SLIC_ERR_TIMEOUT
+    finally:
+        pkg.slic_fault_inject(pkg.SLIC_FAULT_BARRIER_LIMIT, 0)
+    check()  # cleared by the failed check
+    run()
+    check()
+    assert torch.equal(labels, want[0]) and torch.equal(centres, want[1])
+    with pytest.raises(pkg.SlicError):
+        pkg.slic_fault_inject(pkg.SLIC_FAULT_BARRIER_LIMIT, (1 << 22) + 1)
+
+
+@pytest.mark.parametrize("S,shape", [(16, (0, 3, 1, 32)), (8, (0, 3, 1, 32)), (13, (0, 4, 1, 32)),
+                                     (24, (0, 3, 2, 32)), (40, (0, 3, 2, 64))])
+def test_copies_that_never_come_are_reported(slic_gpu, S, shape):
+    """The waits for copies that are never issued run out in every pass kernel:
+    blocks of one cell and of 2x2 cells, tiles of one and of two row groups and
+    32x64 tiles, in a middle pass and in the last one after it."""
+    import torch
+    pkg = slic_gpu
+    W, H = 200, 150
+    imgs = [_img(W, H, 60 + k) for k in range(2)]
+    bs = pkg.BatchSegmenter([dict(width=W, height=H, S=S)] * 2, iterations=1)
+    bs.bind(imgs)
+    bs.set_tuning(*shape)
+    assert bs.info[3] > 0, "the pipelined path is in use"
+    want = [l.clone() for l in bs.segment()[0]]
+    bs.status()
+    try:
+        pkg.slic_fault_inject(pkg.SLIC_FAULT_ABORT_COPIES, 1)
+        bs.segment()
+        with pytest.raises(pkg.SlicError) as ei:
+            bs.status()
+        assert ei.value.status == pkg.SLIC_ERR_TIMEOUT
+    finally:
+        pkg.slic_fault_inject(pkg.SLIC_FAULT_ABORT_COPIES, 0)
+    labels, _ = bs.segment()
+    bs.status()
+    for a, b in zip(labels, want):
+        assert torch.equal(a, b)
+
+
 def test_fault_inject_rejects_bad_arguments(slic_gpu):
     pkg = slic_gpu
     for kind, value in ((0, 1), (9, 1), (pkg.SLIC_FAULT_ALLOC, -1), (pkg.SLIC_FAULT_WALK_LIMIT, 1 << 40)):
