@@ -73,6 +73,76 @@ def test_blocks_of_many_frames_per_warp(slic_gpu):
             assert torch.equal(labels[f], want[k][0]) and torch.equal(centres[f], want[k][1]), f
 
 
+SHAPES = [(0, 3, 1, 32), (2, 4, 1, 32), (0, 3, 2, 32), (1, 4, 2, 32), (0, 3, 2, 64), (1, 3, 2, 64)]
+TILES = [  # (W, H, S, options): S = 24, 40 and 56 run over tiles, the others over blocks
+    [(333, 211, 24, {}), (200, 130, 40, dict(m=20.0))],
+    [(1, 1, 24, {}), (33, 65, 40, {}), (64, 32, 24, {}), (31, 100, 56, {})],
+    [(320, 240, 16, {}), (333, 257, 24, {}), (100, 90, 8, {}), (130, 211, 40, dict(in_channels=4)), (97, 64, 32, {})],
+    [(200, 150, 40, dict(convergence=0.5)), (96, 96, 16, {}), (210, 64, 24, dict(perturb_seeds=True)),
+     (70, 130, 24, dict(color_space=1)), (48, 48, 8, {})],
+]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("frames", TILES)
+def test_tiles_of_every_shape_equal_launch_per_stage(slic_gpu, frames, shape):
+    """One launch per pass over tiles, in every tile shape and group count,
+    alone and among frames that run over blocks: bit-identical to single frames
+    run stage by stage."""
+    import torch
+    bs = slic_gpu.BatchSegmenter([dict(width=W, height=H, S=S, **kw) for W, H, S, kw in frames], iterations=3)
+    imgs = [_img(W, H, 500 + k, kw.get("in_channels", 3)) for k, (W, H, S, kw) in enumerate(frames)]
+    bs.bind(imgs)
+    bs.set_tuning(*shape)
+    assert bs.info[3:6] == shape[1:]
+    want = []
+    for k, (W, H, S, kw) in enumerate(frames):
+        seg = slic_gpu.Segmenter(W, H, S=S, iterations=3, **kw)
+        slic_gpu.slic_profile_enable(seg.handle, True)
+        want.append(seg.segment(imgs[k]))
+    for groups in (1, 2, min(4, len(frames))):
+        bs.set_groups(groups)
+        labels, centres = bs.segment()
+        bs.status()
+        for k in range(len(frames)):
+            assert torch.equal(labels[k], want[k][0]) and torch.equal(centres[k], want[k][1]), (groups, k)
+
+
+@pytest.mark.parametrize("S", [24, 40])
+def test_large_clusters_over_tiles_sum_exactly(slic_gpu, S):
+    """One centre wins the 3x3 cells around it (a white square on black, the
+    other eight centres on black dots, m small): more pixels of a 32x32 and of a
+    32x64 tile than a 32-bit sum of their colours holds (1000 x 100 x 2^15 >
+    2^31), in every tile shape of the plain passes."""
+    import torch
+    W, H = 8 * S, 8 * S
+    ns_c = W // S
+    img = np.zeros((H, W, 3), np.uint8)
+    img[2 * S:5 * S, 3 * S:6 * S] = 255
+    white = 3 * ns_c + 4
+    cen = oracle.init_centres(oracle.convert(img), S)
+    for r in (2, 3, 4):
+        for c in (3, 4, 5):
+            if r * ns_c + c != white:
+                x, y = (int(np.floor(v)) for v in cen[r * ns_c + c, 3:5])
+                img[y - 1:y + 2, x - 1:x + 2] = 0
+    d_img = torch.from_numpy(img).cuda()
+    seg = slic_gpu.Segmenter(W, H, S=S, m=1.0, iterations=3, enforce_connectivity=0)
+    slic_gpu.slic_profile_enable(seg.handle, True)
+    l1, c1 = seg.segment(d_img)
+    lab = l1.cpu().numpy() == white
+    tiles = lab[:H // 32 * 32, :W // 32 * 32].reshape(H // 32, 32, W // 32, 32).sum((1, 3))
+    assert tiles.max() >= 990 and (tiles[::2][:len(tiles[1::2])] + tiles[1::2]).max() >= 1100
+    assert float(c1[white, 0]) > 99.0
+    bs = slic_gpu.BatchSegmenter([dict(width=W, height=H, S=S, m=1.0)], iterations=3, enforce_connectivity=0)
+    bs.bind([d_img])
+    for shape in SHAPES:
+        bs.set_tuning(*shape)
+        labels, centres = bs.segment()
+        bs.status()
+        assert torch.equal(labels[0], l1) and torch.equal(centres[0], c1), shape
+
+
 def _start_centres(seg, kind):
     """Initial centres that the grid's sentinel centres (1e18) can beat: all of
     them, or those around the first and the last cell."""
