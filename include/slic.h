@@ -261,10 +261,11 @@ slic_status slic_batch_segment_host(slic_batch b, const uint8_t *const *host_ima
 
 /* Launch shape of the persistent assignment kernels. Frames whose S is 8 or
    a multiple of 16 run over 16x16-pixel blocks, one warp each, unless fused
-   passes are set (slic_batch_set_fused); the shape below is that of all
-   other frames. ctas_per_sm holds for both, for blocks only while frame
-   groups (slic_batch_set_groups) run side by side (else as many as fit).
-   Resident CTAs per SM (0 = as many as fit, capped by each kernel's occupancy), the number of
+   passes are set (slic_batch_set_fused); the tile shape below is that of all
+   other frames. ctas_per_sm holds for both: resident CTAs per SM (0 = as many
+   as fit, capped by each kernel's occupancy) of each frame group
+   (slic_batch_set_groups; the block passes of groups that have to run as one
+   take the CTAs of all of them). Further, the number of
    TMA pipeline stages (3 or 4; 0 keeps the current value, default 4 where it
    fits), the row groups per warp (1: 256 threads, 4 pixels per thread;
    2: 128 threads per 32 tile rows, 8 pixels per thread, only when every

@@ -200,6 +200,17 @@ int grid_for(const slic_batch_ctx *b, int occ) {
     return std::max(1, per_sm) * b->sms;
 }
 
+// Resident CTAs per SM of the block passes. ctas_per_sm counts for each frame
+// group: groups that have to run as one span (component connectivity, the warm
+// start, the timers) take the CTAs of all of them. As many
+// as fit, 2 per SM, is the fastest for one span (32 x 1080p: 417 us a pass, 602
+// at 1 per SM), 1 per SM and group for four (10-iteration step 4.69 ms, 4.79 at
+// 2).
+int block_ctas(const slic_batch_ctx *b, bool whole) {
+    if (b->ctas_per_sm < 1) return b->block_occ;
+    return (int)std::min<long long>((long long)b->ctas_per_sm * (whole ? b->groups : 1), b->block_occ);
+}
+
 int pipe_occ(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
     return std::max(1, assign_pipe_occupancy(b->same, tile_h == 64 ? b->win_max64 : b->win_max, stages, rows, tile_h));
 }
@@ -701,13 +712,8 @@ cudaError_t enqueue_span(slic_batch_ctx *b, const Span &sp, cudaStream_t s, bool
                                            b->smem, grid, s);
             const int rest = b->tile_h == 64 ? sp.rest64 : sp.rest;
             n_launch += std::max(0, (sp.blocks > 0) + (sp.blocks8 > 0) + (rest > 0) - 1);  // (one launch each)
-            // Blocks: every CTA that fits (2 per SM, 417 us; 1 per SM, 602 us),
-            // but as many as asked for while frame groups share the GPU
-            // (10-iteration step with 4 groups: 4.69 ms at 1 per SM and group,
-            // 4.79 ms at 2)
-            const int grid_blocks = whole ? b->block_occ * b->sms : grid_for(b, b->block_occ);
-            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, sp.blocks8, last, grid_blocks, b->d_err,
-                                                 b->any_conv ? 1 : 0, s);
+            cudaError_t r = launch_assign_blocks(sp.frames, sp.n, sp.blocks, sp.blocks8, last,
+                                                 block_ctas(b, whole) * b->sms, b->d_err, b->any_conv ? 1 : 0, s);
             if (r == cudaSuccess)
                 r = launch_assign_pipe(sp.frames, sp.n, rest, win_th, b->same, last, b->stages, b->rows, b->tile_h,
                                        pipe_per_sm, grid_pipe, b->d_err, b->any_conv ? 1 : 0, s);

@@ -470,3 +470,52 @@ def test_frame_groups_are_bit_exact(slic_gpu):
     with pytest.raises(pkg.SlicError):
         bs.set_groups(5)
     bs.close()
+
+
+def _kernel_grids(call, stream):
+    """(grid x, block x) of every kernel of the graph that `call` is captured into on `stream`."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    class Params(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS (v2)
+        _fields_ = [("func", ctypes.c_void_p)] + [(n, ctypes.c_uint) for n in (
+            "gx", "gy", "gz", "bx", "by", "bz", "smem")] + [("args", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                                                            ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+    graph, n, kind = ctypes.c_void_p(), ctypes.c_size_t(), ctypes.c_int()
+    ok = lambda r: r == 0 or pytest.fail(f"driver call failed: {r}")  # noqa: E731
+    ok(cu.cuStreamBeginCapture_v2(ctypes.c_void_p(stream.cuda_stream), 1))  # (thread-local mode)
+    call()
+    ok(cu.cuStreamEndCapture(ctypes.c_void_p(stream.cuda_stream), ctypes.byref(graph)))
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    grids = []
+    for node in nodes:
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value == 0:
+            p = Params()
+            ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+            grids.append((p.gx, p.bx))
+    ok(cu.cuGraphDestroy(graph))
+    return grids
+
+
+@pytest.mark.parametrize("S", [16, 8])
+@pytest.mark.parametrize("connectivity,groups,ctas,per_sm,spans", [
+    (1, 1, 0, 2, 1), (1, 1, 1, 1, 1), (1, 1, 2, 2, 1), (1, 1, 9, 2, 1),   # as asked, at most what fits
+    (1, 2, 1, 1, 2), (1, 2, 0, 2, 2),                                     # of each group
+    (2, 1, 1, 1, 1), (2, 2, 1, 2, 1)])                                    # two groups that run as one
+def test_block_passes_take_the_ctas_asked_for(slic_gpu, S, connectivity, groups, ctas, per_sm, spans):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bs = slic_gpu.BatchSegmenter([dict(width=1280, height=720, S=S)] * 2, iterations=2,
+                                 enforce_connectivity=connectivity)
+    bs.bind([_cuda(synth.voronoi_frame(1280, 720, 30, 6.0, s)) for s in (1, 2)])
+    bs.set_tuning(ctas, groups=groups)
+    stream = torch.cuda.Stream()
+    bs.segment(stream=stream)
+    torch.cuda.synchronize()
+    grids = _kernel_grids(lambda: bs.segment(stream=stream), stream)
+    for c in (1, 2):  # (no other stage has such a grid)
+        assert grids.count((c * sms, 256)) == (3 * spans if c == per_sm else 0)
