@@ -309,12 +309,14 @@ slic_status slic_batch_set_groups(slic_batch b, int groups);
 /* Autotuner: time slic_batch_segment on the bound buffers for every launch
    shape that fits (3 timed runs each, CUDA events on `stream`; this waits
    for the device), keep the fastest, and append it to the JSON-lines file
-   cache_path (may be NULL) under a key of GPU name, frame count,
-   iterations and the distinct (width, height, S). When the key is already
-   in the file its entry is used without timing. The search covers tile
+   cache_path (may be NULL) under a key of GPU name, kernel set, frame count,
+   iterations, connectivity mode, warm start or not and the distinct (width,
+   height, S). When the key is already in the file its entry is used without
+   timing (entries of an older kernel set are not). The search covers tile
    shapes x row groups per warp x pipeline stages x CTAs per SM x fused
    passes or not (slic_batch_set_fused) x frame groups (1, 2 or 4;
-   slic_batch_set_groups); the choice is set on the batch and returned in
+   slic_batch_set_groups), as far as they change what runs: the tile shape
+   does not where every frame runs over blocks; the choice is set on the batch and returned in
    *ctas_per_sm, *stages, *rows, *tile_h, *fused and *groups (any may be
    NULL). */
 slic_status slic_batch_autotune(slic_batch b, const char *cache_path, void *stream, int *ctas_per_sm, int *stages,

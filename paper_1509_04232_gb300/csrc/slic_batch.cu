@@ -215,6 +215,12 @@ int pipe_occ(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
     return std::max(1, assign_pipe_occupancy(b->same, tile_h == 64 ? b->win_max64 : b->win_max, stages, rows, tile_h));
 }
 
+// The same for the fused passes.
+int multi_occ(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
+    return std::max(
+        1, assign_pipe_occupancy(b->same, tile_h == 64 ? b->win_max64 : b->win_max, stages, rows, tile_h, true));
+}
+
 // Whether a launch shape of the pipelined kernel fits (shared memory) and is
 // allowed for the batch.
 bool shape_fits(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
@@ -224,12 +230,17 @@ bool shape_fits(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
     return assign_pipe_occupancy(b->same, tile_h == 64 ? b->win_max64 : b->win_max, stages, rows, tile_h) > 0;
 }
 
+// What the best launch shape depends on: the GPU, the kernels that serve a
+// frame (kernels=2: blocks for S = 8 and multiples of 16; a line written for
+// other kernels is not served), whether frame groups can run side by side
+// (connectivity mode, warm start), and the frames.
 std::string tune_key(const slic_batch_ctx *b) {
     cudaDeviceProp prop;
     std::string gpu = cudaGetDeviceProperties(&prop, b->device) == cudaSuccess ? prop.name : "unknown";
     std::set<std::tuple<int, int, int>> shapes;
     for (const FrameArgs &f : b->frames) shapes.insert(std::make_tuple(f.W, f.H, f.S));
-    std::string key = gpu + "|frames=" + std::to_string(b->n) + "|it=" + std::to_string(b->iterations);
+    std::string key = gpu + "|kernels=2|frames=" + std::to_string(b->n) + "|it=" + std::to_string(b->iterations) +
+                      "|conn=" + std::to_string(b->connectivity) + "|net=" + (b->net ? "1" : "0");
     for (const auto &s : shapes)
         key += "|" + std::to_string(std::get<0>(s)) + "x" + std::to_string(std::get<1>(s)) + "s" +
                std::to_string(std::get<2>(s));
@@ -723,8 +734,7 @@ cudaError_t enqueue_span(slic_batch_ctx *b, const Span &sp, cudaStream_t s, bool
     if (e == cudaSuccess && b->pipe && b->fused && whole && b->iterations > 0) {
         // Passes 0 .. n-1 with updates 1 .. n in one cooperative launch
         // (per-frame phase counters order them), then the last pass.
-        const int occ = std::max(1, assign_pipe_occupancy(b->same, win_th, b->stages, b->rows, b->tile_h, true));
-        const int grid_multi = grid_for(b, occ);
+        const int grid_multi = grid_for(b, multi_occ(b, b->stages, b->rows, b->tile_h));
         e = timed([&]() {
             return launch_assign_multi(sp.frames, sp.n, tiles_th, sp.chunks, win_th, b->same, b->iterations,
                                        b->stages, b->rows, b->tile_h, grid_multi / std::max(1, b->sms), grid_multi,
@@ -989,20 +999,28 @@ slic_status slic_batch_autotune(slic_batch b, const char *cache_path, void *stre
     // pipelined path only) x tile shape (32x32, or 32x64 with two row
     // groups) x row groups per warp (pixels per thread and block size) x
     // pipeline stages x resident CTAs per SM (up to what fits) x fused passes
-    // or not (one group only).
+    // or not (one group only). Where every frame runs over blocks the tile
+    // shape, row groups and stages matter to the fused passes alone: one
+    // launch per pass is timed in the first shape only.
+    const bool tiles = !b->pipe || b->total_rest > 0;
     const bool can_split = b->pipe && !b->net && b->connectivity != 2;
     const int st_lo = b->pipe ? 3 : b->stages, st_hi = b->pipe ? 4 : b->stages;
     const int rw_hi = (b->pipe && b->same8) ? 2 : 1;
     for (int gr = 1; gr <= (can_split ? std::min(4, b->n) : 1) && st == SLIC_OK; gr *= 2) {
         if ((st = slic_batch_set_groups(b, gr)) != SLIC_OK) break;
         const int fu_hi = b->pipe && b->iterations > 0 && gr == 1 ? 1 : 0;
+        bool passes_timed = false;  // (one launch per pass, in some shape)
         for (int th = 32; th <= 64 && st == SLIC_OK; th += 32) {
             for (int rw = 1; rw <= rw_hi && st == SLIC_OK; ++rw) {
                 for (int nst = st_lo; nst <= st_hi && st == SLIC_OK; ++nst) {
                     if (b->pipe ? !shape_fits(b, nst, rw, th) : th != 32) continue;
-                    const int occ = std::max(b->occupancy, b->pipe ? pipe_occ(b, nst, rw, th) : 0);
-                    for (int k = 0; k < occ * (fu_hi + 1) && st == SLIC_OK; ++k) {
-                        const int c = 1 + k / (fu_hi + 1), fu = k % (fu_hi + 1);
+                    int occ[2] = {0, fu_hi ? multi_occ(b, nst, rw, th) : 0};  // plain, fused
+                    if (tiles || !passes_timed)
+                        occ[0] = std::max(b->total_blocks + b->total_blocks8 > 0 ? b->block_occ : 0,
+                                          !b->pipe ? b->occupancy : (tiles ? pipe_occ(b, nst, rw, th) : 0));
+                    passes_timed = true;
+                    for (int k = 0; k < occ[0] + occ[1] && st == SLIC_OK; ++k) {
+                        const int fu = k < occ[0] ? 0 : 1, c = 1 + k - (fu ? occ[0] : 0);
                         b->ctas_per_sm = c;
                         b->stages = nst;
                         b->rows = rw;

@@ -519,3 +519,41 @@ def test_block_passes_take_the_ctas_asked_for(slic_gpu, S, connectivity, groups,
     grids = _kernel_grids(lambda: bs.segment(stream=stream), stream)
     for c in (1, 2):  # (no other stage has such a grid)
         assert grids.count((c * sms, 256)) == (3 * spans if c == per_sm else 0)
+
+
+def test_autotune_times_what_changes_the_launches(slic_gpu):
+    """A batch whose frames all run over blocks: only the CTAs per SM are
+    searched (no fused passes without a middle pass, one frame: one group),
+    each with one warm-up and three timed calls of four launches. A frame over
+    tiles brings the tile shapes back."""
+    calls = []
+    for S in (16, 8, 24):
+        bs = slic_gpu.BatchSegmenter([dict(width=320, height=240, S=S)], iterations=0)
+        bs.bind([_cuda(synth.small_image(1))])
+        n0 = bs.info[1]
+        c, stages, rows, tile_h, fused, groups = bs.autotune()
+        calls.append((bs.info[1] - n0) // 4)
+        assert 1 <= c <= (2 if S != 24 else 8) and stages in (3, 4) and fused == 0 and groups == 1
+    assert calls[0] == calls[1] == 2 * 4 and calls[2] >= 6 * 4
+
+
+def test_autotune_cache_key(slic_gpu, tmp_path):
+    """Entries of an older kernel set, of another connectivity mode or of a
+    batch without the warm start are not served."""
+    import torch
+    from paper_1509_04232_gb300.warmstart import WarmStartNet
+    cache = str(tmp_path / "tune.jsonl")
+    gpu = torch.cuda.get_device_name(0)
+    with open(cache, "w") as f:
+        f.write(json.dumps({"key": f"{gpu}|frames=2|it=1|320x240s16", "ctas_per_sm": 1, "stages": 4, "rows": 2,
+                            "tile_h": 64, "fused": 1, "groups": 1, "ms": 0.01}) + "\n")
+    net = WarmStartNet(320, 240, 16, max_batch=2)
+    for conn, warm in ((1, False), (2, False), (1, True)):
+        bs = slic_gpu.BatchSegmenter([dict(width=320, height=240, S=16)] * 2, iterations=1, enforce_connectivity=conn)
+        bs.bind([_cuda(synth.small_image(k)) for k in (1, 2)])
+        if warm:
+            bs.set_warmstart(net)
+        first = bs.autotune(cache)
+        n = len(open(cache).read().splitlines())
+        assert bs.autotune(cache) == first and len(open(cache).read().splitlines()) == n
+    assert n == 4
