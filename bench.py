@@ -522,7 +522,7 @@ def run_ours(args):
                          "unit": "Tsqrt/s", "achieved": achieved_tops, "peak": xu_peak, "frac": achieved_tops / xu_peak,
                          "peak_source": f"16 MUFU lanes/clk/SM x {sms} SMs x max SM clock (recipe unit counts)",
                          "traffic": traffic, "avg_launch_us": mid_ms * 1e3, "launches_timed": len(mid),
-                         "measured_as": f"one frame group at full occupancy ({occ_alone if fused_dom else 2} CTAs/SM); the step runs "
+                         "measured_as": f"one frame group at full occupancy ({occ_alone} CTAs/SM); the step runs "
                                         f"{groups} group(s) concurrently at {ctas_per_sm} CTAs/SM each",
                          "in_step": {"achieved": in_step_tops,
                                      "frac": in_step_tops / xu_peak if in_step_tops else None,

@@ -323,7 +323,8 @@ slic_status slic_batch_autotune(slic_batch b, const char *cache_path, void *stre
                                int *rows, int *tile_h, int *fused, int *groups);
 
 /* Pixels of all frames, kernel launches enqueued so far, and the launch
-   shape of the assignment passes: CTAs per SM (as requested, capped by what
+   shape of the assignment passes: CTAs per SM of the kernel that most pixels
+   go through (blocks, tiles or the fused passes; as requested, capped by what
    fits), pipeline stages, row groups per warp, tile rows, fused passes and
    frame groups (stages and rows 0, tile rows 32, fused 0 when the
    pipelined kernel is not used); any pointer may be NULL. */

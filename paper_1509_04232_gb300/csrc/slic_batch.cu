@@ -221,6 +221,25 @@ int multi_occ(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
         1, assign_pipe_occupancy(b->same, tile_h == 64 ? b->win_max64 : b->win_max, stages, rows, tile_h, true));
 }
 
+// Groups run concurrently only on the plain pipelined path (the warm start,
+// component connectivity and the per-launch timers take the whole batch at
+// once).
+bool split_groups(const slic_batch_ctx *b) {
+    return b->groups > 1 && b->pipe && !b->net && b->connectivity != 2 && !b->profiling;
+}
+
+// Resident CTAs per SM of the assignment kernel that most pixels go through, as
+// the next call launches it.
+int dominant_ctas(const slic_batch_ctx *b) {
+    const bool whole = !split_groups(b);
+    if (!b->pipe) return grid_for(b, b->occupancy) / b->sms;
+    if (b->fused && whole && b->iterations > 0) return grid_for(b, multi_occ(b, b->stages, b->rows, b->tile_h)) / b->sms;
+    long long px = 0;
+    for (const FrameArgs &a : b->frames) px += a.blocks_x > 0 ? (long long)a.W * a.H : 0;
+    return 2 * px >= b->total_pixels ? block_ctas(b, whole)
+                                     : grid_for(b, pipe_occ(b, b->stages, b->rows, b->tile_h)) / b->sms;
+}
+
 // Whether a launch shape of the pipelined kernel fits (shared memory) and is
 // allowed for the batch.
 bool shape_fits(const slic_batch_ctx *b, int stages, int rows, int tile_h) {
@@ -773,13 +792,6 @@ cudaError_t enqueue_span(slic_batch_ctx *b, const Span &sp, cudaStream_t s, bool
 
 extern "C" {
 
-// Groups run concurrently only on the plain pipelined path (the warm start,
-// component connectivity and the per-launch timers take the whole batch at
-// once).
-static bool split_groups(const slic_batch_ctx *b) {
-    return b->groups > 1 && b->pipe && !b->net && b->connectivity != 2 && !b->profiling;
-}
-
 slic_status slic_batch_segment(slic_batch b, void *stream) {
     if (!b) return bfail(nullptr, SLIC_ERR_INVALID, "NULL batch");
     if (!b->buffers_set) return bfail(b, SLIC_ERR_STATE, "slic_batch_set_buffers has not been called");
@@ -1065,8 +1077,7 @@ slic_status slic_batch_info(slic_batch b, long long *total_pixels, long long *la
     if (!b) return bfail(nullptr, SLIC_ERR_INVALID, "NULL batch");
     if (total_pixels) *total_pixels = b->total_pixels;
     if (launches) *launches = b->launches;
-    if (ctas_per_sm)  // resident CTAs per SM of the dominant assignment kernel
-        *ctas_per_sm = grid_for(b, b->pipe ? pipe_occ(b, b->stages, b->rows, b->tile_h) : b->occupancy) / b->sms;
+    if (ctas_per_sm) *ctas_per_sm = dominant_ctas(b);
     if (stages) *stages = b->pipe ? b->stages : 0;
     if (rows) *rows = b->pipe ? b->rows : 0;
     if (tile_h) *tile_h = b->pipe ? b->tile_h : 32;

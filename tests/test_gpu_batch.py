@@ -557,3 +557,34 @@ def test_autotune_cache_key(slic_gpu, tmp_path):
         n = len(open(cache).read().splitlines())
         assert bs.autotune(cache) == first and len(open(cache).read().splitlines()) == n
     assert n == 4
+
+
+def test_info_reports_the_ctas_that_run(slic_gpu):
+    """CTAs per SM of the kernel that most pixels go through: the blocks' two at
+    most, the tiles' and the fused passes' own limits."""
+    def batch(sizes, **kw):
+        frames = [dict(width=W, height=H, S=S) for W, H, S in sizes]
+        bs = slic_gpu.BatchSegmenter(frames, iterations=1, **kw)
+        bs.bind([_cuda(synth.voronoi_frame(W, H, 20, 6.0, 1)) for W, H, _ in sizes])
+        return bs
+
+    bs = batch([(320, 240, 16), (100, 100, 24)])      # most pixels over blocks
+    for asked, got in ((0, 2), (1, 1), (2, 2), (7, 2)):
+        bs.set_tuning(asked)
+        assert bs.info[2] == got
+    bs.set_tuning(0, 3, 2, 64)
+    assert bs.info[2] == 2
+    tiles = batch([(320, 240, 24), (100, 100, 16)])   # most over tiles
+    tiles.set_tuning(0, 3, 1, 32)
+    most = tiles.info[2]
+    assert most >= 3
+    tiles.set_tuning(most + 1)
+    assert tiles.info[2] == most
+    tiles.set_tuning(1)
+    assert tiles.info[2] == 1
+    both = batch([(320, 240, 16)] * 2, enforce_connectivity=2)  # two groups that run as one
+    both.set_tuning(1, groups=2)
+    assert both.info[2] == 2
+    fused = batch([(320, 240, 16)] * 2)
+    fused.set_tuning(0, 3, 1, 32, fused=True)
+    assert fused.info[2] >= 2 and fused.info[6] == 1
