@@ -193,10 +193,10 @@ class BatchSegmenter:
             init = [t.data_ptr() if t is not None else None for t in init_centres]
         args = ([t.data_ptr() for t in self.images], [t.data_ptr() for t in self.labels],
                 [t.data_ptr() for t in self.centres], init)
+        self._init_refs = init_centres  # (kept alive until the next binding)
         if first:
             slic_batch_set_buffers(self.handle, *args)
         else:
-            self._init_refs = init_centres  # (kept alive until the next binding)
             slic_batch_rebind(self.handle, *args, _stream_handle(stream))
 
     def segment(self, stream=None):

@@ -588,3 +588,26 @@ def test_info_reports_the_ctas_that_run(slic_gpu):
     fused = batch([(320, 240, 16)] * 2)
     fused.set_tuning(0, 3, 1, 32, fused=True)
     assert fused.info[2] >= 2 and fused.info[6] == 1
+
+
+def test_bound_initial_centres_stay_alive(slic_gpu):
+    """Every segmentation reads the initial centres of the binding, the first
+    binding's as well: the batch keeps their tensors."""
+    import gc
+    import weakref
+    import torch
+    bs = slic_gpu.BatchSegmenter([dict(width=64, height=48, S=16)], iterations=1)
+    img = _cuda(synth.voronoi_frame(64, 48, 8, 6.0, 1))
+    start = torch.rand(bs.K_eff[0], 6, device="cuda") * 40
+    want = [t.clone() for t in (lambda s: s.segment(img, init_centres=start))(
+        slic_gpu.Segmenter(64, 48, S=16, iterations=1))]
+    for _ in range(2):  # the first binding, then a later one
+        given = start.clone()
+        alive = weakref.ref(given)
+        bs.bind([img], init_centres=[given])
+        del given
+        gc.collect()
+        torch.full((bs.K_eff[0], 6), 7.0, device="cuda")  # (would take a freed tensor's memory)
+        labels, centres = bs.segment()
+        assert alive() is not None
+        assert torch.equal(labels[0], want[0]) and torch.equal(centres[0], want[1])
