@@ -178,9 +178,9 @@ slic_status slic_update(slic_handle h, const float *d_features, const int32_t *d
    writes d_out; they must not overlap. */
 slic_status slic_connectivity_pass(slic_handle h, const int32_t *d_in, int32_t *d_out, void *stream);
 
-/* Kernel launches enqueued by this handle since creation (all calls). A
-   launch that runs several stages counts once per stage, as if each had a
-   launch of its own: slic_segment runs a frame whose features fit in the
+/* Stages enqueued by this handle since creation (all calls): a kernel launch
+   counts once for each stage it runs, as if each had a launch of its own.
+   slic_segment runs a frame whose features fit in the
    GPU's shared memory (up to about 2.5 Mpx, S >= 7) as one cooperative
    launch, unless the learned warm start is armed or profiling is enabled. */
 slic_status slic_launch_count(slic_handle h, long long *count);
@@ -301,8 +301,10 @@ slic_status slic_batch_set_fused(slic_batch b, int enable);
    boundaries (the last tiles of a pass, the update) overlap another group's
    passes. Results are bit-identical for any grouping. The learned warm
    start, component connectivity (mode 2), the non-pipelined kernels and
-   profiling (slic_batch_profile_enable) run the batch as one group, as do
-   fused passes. A change after the buffers are bound waits for the device.
+   profiling (slic_batch_profile_enable) run the batch as one group. Groups
+   run one launch per pass: fused passes (slic_batch_set_fused) take effect
+   where the batch runs as one group. A change after the buffers are bound
+   waits for the device.
    SLIC_ERR_INVALID outside the range. */
 slic_status slic_batch_set_groups(slic_batch b, int groups);
 

@@ -134,6 +134,7 @@ class Segmenter:
 
     @property
     def launches(self) -> int:
+        """Stages enqueued since creation; one launch may run several (slic_launch_count)."""
         return slic_launch_count(self.handle)
 
     @property

@@ -558,10 +558,11 @@ slic_status slic_batch_create(const slic_params *params, int n_frames, slic_batc
     }
     {
         // Blocks or tiles, per frame: at other S a 16x16 block is neither part
-        // of a cell nor made of whole ones. 32 x 1080p, S = 16, middle pass:
-        // 417 us over blocks, 432 over 32x64 tiles, 549 over 32x32 tiles with
-        // one row group. S = 8, 14.8 Mpx of a mixed batch, middle / last pass:
-        // 114 / 85 us over blocks, 134 / 99 over 32x32 tiles.
+        // of a cell nor made of whole ones. 32 x 1080p, middle / last pass, us:
+        //   S           8        16       32       48       64
+        //   blocks   471/346  417/350  407/350  402/351  400/351
+        //   32x64    616/463  432/365  436/365  430/365  463/365
+        //   32x32    547/403  512/402  604/387  598/388  596/387 (one row group)
         b->block_occ = b->pipe ? assign_blocks_occupancy() : 0;
         for (FrameArgs &a : b->frames) {
             a.block_base = b->total_blocks;

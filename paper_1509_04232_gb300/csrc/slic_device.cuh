@@ -161,7 +161,8 @@ __device__ __forceinline__ float fmin3_nan(float a, float b, float c) {
 // at scale 1), and equal to __float2int_rn(x * fs) + kFixBias there since fs
 // is a power of two. Sums of such words taken mod 2^32, minus count *
 // kFixBias, are the sums of the rounded values, exactly, whenever those fit
-// in 31 bits (at most 2^22 per value, 128 values per private copy).
+// in 31 bits: at most 2^22 per value, and at most 256 values (a 16x16 block or
+// unit, a pair of a tile's private copies) go into one word, 2^30 in all.
 constexpr unsigned kFixBias = 0x4B400000u;
 __device__ __forceinline__ void fix_round2_biased(float x0, float x1, float fs, unsigned &r0, unsigned &r1) {
     const unsigned long long m = fma2(pack2(x0, x1), pack2(fs, fs), pack2(12582912.0f, 12582912.0f));

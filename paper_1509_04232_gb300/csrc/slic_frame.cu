@@ -12,10 +12,12 @@
 // local connectivity rule one more barrier separates them from its two
 // passes. The launch replaces 2 * iterations + 4 launches whose gaps, feature
 // traffic and partly filled last waves took most of a single frame's time:
-// 320x240, 10 iterations, 119 -> 46 us; 1920x1080, 5 iterations, 193 -> 105 us.
-// A small frame is bound by the latency of a pass (centres 1.3, evaluation 1.1,
-// barrier 1.5 us), a large one by instruction issue (46 % of the cycles, 9.6 of
-// 14.8 us per pass) and the drain of its sums before the barrier.
+// 320x240, 10 iterations, 119 -> 48 us; 1920x1080, 5 iterations, 193 -> 107 us.
+// A small frame is bound by the latency of a pass, 3.5 us at 320x240: centres
+// 1.2, evaluation 0.9, barrier 1.4 (clock stamps). A large one is bound by
+// instruction issue (46 % of the cycles) and by the drain of its sums before the
+// barrier: 13.8 us per pass at 1920x1080, S = 16, of which centres 1.3,
+// evaluation 9.4, barrier 3.1.
 //
 // Results are those of the launch-per-stage path, bit for bit: the same
 // operations on the same values, and exact integer sums.

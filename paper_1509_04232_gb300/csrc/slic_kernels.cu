@@ -1661,10 +1661,10 @@ cudaError_t launch_assign_pipe(const FrameArgs *d_frames, int n, int total_tiles
 // l holds the pixel pairs at columns 2 * (l % 8) of rows l / 8 + 4 i: its loads
 // are 256 contiguous bytes per warp. Pixels that stay with their own cell, the
 // most frequent winner, add up in registers and across the warp; the others go
-// to the warp's bins in shared memory (see FrameBins). Running 64-bit totals
-// of the nine cells stay in the lanes' registers while the run moves along a
-// row, shifted by one cell at a time: only the three cells left behind go to
-// global memory, so a block costs 18 atomic lanes, not 54.
+// to the warp's bins in shared memory (laid out as BlkGeo says). Running 64-bit
+// totals of the nine cells stay in shared memory (BlockState) while the run
+// moves along a row, shifted by one cell at a time: only the three cells left
+// behind go to global memory, so a block costs 18 atomic lanes, not 54.
 //
 // CS = 2: frames with S = 8, a block of 2x2 cells. Eight lanes take a cell
 // (columns 2 * (l % 4), rows l / 4 % 2 + 2 i of it): a lane's pixels share one
