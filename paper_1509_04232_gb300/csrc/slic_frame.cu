@@ -12,7 +12,7 @@
 // local connectivity rule one more barrier separates them from its two
 // passes. The launch replaces 2 * iterations + 4 launches whose gaps, feature
 // traffic and partly filled last waves took most of a single frame's time:
-// 320x240, 10 iterations, 119 -> 48 us; 1920x1080, 5 iterations, 193 -> 107 us.
+// 320x240, 10 iterations, 119 -> 47 us; 1920x1080, 5 iterations, 193 -> 107 us.
 // A small frame is bound by the latency of a pass, 3.5 us at 320x240: centres
 // 1.2, evaluation 0.9, barrier 1.4 (clock stamps). A large one is bound by
 // instruction issue (46 % of the cycles) and by the drain of its sums before the
